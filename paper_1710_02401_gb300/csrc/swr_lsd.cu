@@ -34,6 +34,7 @@
 // and the index tables.
 #include <math.h>
 #include <stdio.h>
+#include <string.h>
 
 #include <algorithm>
 #include <string>
@@ -75,7 +76,7 @@ __device__ inline double lsd_ven(const LsdDev& d, double x) {
 __global__ void k_lsd_gl(int q, double* t, double* w) {
     const int k = threadIdx.x;
     if (k >= q) return;
-    double x = cos(3.14159265358979323846 * (k + 0.75) / (q + 0.5)), dp = 1.0;
+    double x = cos(3.14159265358979323846 * (k + 0.75) / (q + 0.5)), dp = 1.0, last = 1.0;
     for (int it = 0; it < 100; ++it) {
         double p0 = 1.0, p1 = x;
         for (int j = 2; j <= q; ++j) {
@@ -86,7 +87,8 @@ __global__ void k_lsd_gl(int q, double* t, double* w) {
         dp = q * (x * p1 - p0) / (x * x - 1.0);
         const double dx = p1 / dp;
         x -= dx;
-        if (fabs(dx) < 1e-16) break;
+        if (last < 1e-8) break;  // quadratic convergence: this step was the last that changes x
+        last = fabs(dx);
     }
     t[q - 1 - k] = x;  // ascending
     w[q - 1 - k] = 2.0 / ((1.0 - x * x) * dp * dp);
@@ -106,67 +108,152 @@ __global__ void k_lsd_nodes(const double* edges, const int* ebase, int n_panels,
 
 // ------------------------------------------------------ 1. local orbitals
 //
-// One CTA per subdomain.  Shared memory: A (overlap, then its Cholesky factor
-// in the lower triangle) | B (Hamiltonian, then L^-1 H L^-T, then its
-// eigenvalues on the diagonal) | V (eigenvectors) | scratch, each n x n with
-// n = kd rounded up to even (a padded row is decoupled with a large diagonal).
-__device__ void lsd_jacobi(double* B, double* V, int n, double* red) {
-    const int tid = threadIdx.x, nt = blockDim.x, half = n / 2;
-    __shared__ int s_pair[LSD_KD_MAX][2];
+// Three kernels: Gaussians and weights at the local nodes (one thread per
+// value: every exponential, square root and barrier switch evaluated once),
+// the overlap and Hamiltonian entries (one warp per entry of the upper
+// triangle, lanes over the nodes), and the dense eigenproblem (one CTA per
+// subdomain).  FP64 runs at 1.6 multiply-adds per clock on an SM of this
+// part, so what one CTA does alone is kept to the O(kd^3) of the
+// eigenproblem: with the quadrature inside that CTA (potential and switch per
+// entry and node) the L = 5, M = 10, kd = 40 build took 25.5 ms in this
+// stage, now 1.07 ms (1.03 of it the eigenproblem: ~350 Jacobi rounds bound by
+// the FP64 pipe of one SM and two barriers each); whole call 27.3 -> 2.0 ms.
+
+// Table rows of subdomain i, each nn nodes long: kd rows of g_k, kd rows of
+// g_k', then w, 1/2 w a, w (V_en + V_b) and w exp(0.37 (x - x_ci)).
+#define LSD_WROWS 4
+__host__ __device__ inline size_t lsd_tab0(int n0, int kd) { return (size_t)n0 * (2 * kd + LSD_WROWS); }
+
+__global__ void k_lsd_local_tab(LsdDev d, const double* xl, const double* wl, const int* nbase, double* gtab) {
+    const int i = blockIdx.y, kd = d.kd, n0 = nbase[i], nn = nbase[i + 1] - n0;
+    const double xc = lsd_centre(d, i), h = 2.0 * d.xb / (kd - 1);
+    double* g = gtab + lsd_tab0(n0, kd);
+    double* dg = g + (size_t)kd * nn;
+    double* wr = dg + (size_t)kd * nn;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < nn * kd) {
+        const int k = e / nn, m = e - k * nn;
+        const double al = (k == kd - 1) ? xc + d.xb : (double)k * h + (xc - d.xb);
+        const double u = xl[n0 + m] - al, gv = exp(-d.delta * u * u);
+        g[e] = gv;
+        dg[e] = -2.0 * d.delta * u * gv;
+    } else if (e < nn * (kd + 1)) {
+        const int m = e - nn * kd;
+        const double x = xl[n0 + m], w = wl[n0 + m], sw = lsd_switch(d, x, xc);
+        wr[m] = w;
+        wr[nn + m] = 0.5 * w * (1.0 - sw);
+        wr[2 * nn + m] = w * (lsd_ven(d, x) + d.v_inf * sw);
+        wr[3 * nn + m] = w * exp(0.37 * (x - xc));
+    }
+}
+
+// Entry (r, c), c >= r, of the overlap and the Hamiltonian of subdomain i (one
+// warp), then the kd sign weights int g_k exp(0.37 (x - x_ci)): mat[i] = overlap
+// [kd][kd] | Hamiltonian [kd][kd] | sign weights [kd].
+__global__ void k_lsd_local_mat(LsdDev d, const int* nbase, const double* gtab, double* mat) {
+    const int i = blockIdx.y, kd = d.kd, n0 = nbase[i], nn = nbase[i + 1] - n0;
+    const int it = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const double* g = gtab + lsd_tab0(n0, kd);
+    const double* dg = g + (size_t)kd * nn;
+    const double* wr = dg + (size_t)kd * nn;
+    double* Mi = mat + (size_t)i * kd * (2 * kd + 1);
+    if (it < kd * kd) {
+        const int r = it / kd, c = it - r * kd;
+        if (c < r) return;
+        const double *gr = g + (size_t)r * nn, *gc = g + (size_t)c * nn, *dr = dg + (size_t)r * nn, *dc = dg + (size_t)c * nn;
+        double s = 0.0, hh = 0.0;
+        for (int m = lane; m < nn; m += 32) {
+            const double gg = gr[m] * gc[m];
+            s += wr[m] * gg;
+            hh += wr[nn + m] * (dr[m] * dc[m]) + wr[2 * nn + m] * gg;
+        }
+        s = warp_sum(s);
+        hh = warp_sum(hh);
+        if (lane == 0) {
+            Mi[r * kd + c] = Mi[c * kd + r] = s;
+            Mi[kd * kd + r * kd + c] = Mi[kd * kd + c * kd + r] = hh;
+        }
+    } else if (it < kd * kd + kd) {
+        const int k = it - kd * kd;
+        double s = 0.0;
+        for (int m = lane; m < nn; m += 32) s += wr[3 * nn + m] * g[(size_t)k * nn + m];
+        s = warp_sum(s);
+        if (lane == 0) Mi[2 * kd * kd + k] = s;
+    }
+}
+
+// Cyclic Jacobi of the symmetric n x n matrix B (n even, round-robin pairs):
+// a round rotates n/2 disjoint index pairs.  The 2 x 2 block of two pairs is
+// transformed from both sides by one thread (and mirrored), so a round is one
+// pass over the upper triangle.  The rotations themselves go to `rot`
+// ([round][pair] as (c, s), at most LSD_SWEEPS sweeps); the eigenvectors are
+// formed from them afterwards for the wanted columns only, a quarter of the
+// FP64 work of updating all of V in every round at M = 10 of 40.  The tangent
+// of the angle is an FP32 estimate (the FP64 divisions and roots would be a
+// serial chain of several hundred clocks in every round): the rotation stays
+// orthogonal to rounding because c = 1 / sqrt(1 + t^2) is FP64, and a rotated
+// entry is left at 1e-7 of what it was, which the next sweep removes.  Sweeps
+// run until the off-diagonal mass is below 1e-32 of the diagonal one.
+// Returns the number of rounds.
+#define LSD_SWEEPS 60
+__device__ inline void lsd_round_pair(int r, int k, int n, int& p, int& q) {
+    // circle method: player 0 against 1 + r mod (n-1), then symmetric pairs
+    if (k == 0) {
+        p = 0;
+        q = 1 + (r % (n - 1));
+    } else {
+        p = 1 + ((r + k) % (n - 1));
+        q = 1 + ((r + n - 1 - k) % (n - 1));
+    }
+    if (p > q) {
+        const int t = p;
+        p = q;
+        q = t;
+    }
+}
+
+__device__ int lsd_jacobi(double* B, int n, double2* rot, double* red) {
+    const int tid = threadIdx.x, nt = blockDim.x, half = n / 2, nblk = half * (half + 1) / 2;
+    __shared__ int s_pair[LSD_KD_MAX / 2][2];
     __shared__ double s_cs[LSD_KD_MAX / 2][2];
     __shared__ int s_go;
-    for (int sweep = 0; sweep < 60; ++sweep) {
-        for (int r = 0; r < n - 1; ++r) {
+    int rounds = 0;
+    for (int sweep = 0; sweep < LSD_SWEEPS; ++sweep) {
+        for (int r = 0; r < n - 1; ++r, ++rounds) {
             if (tid < half) {
-                // circle method: player 0 against 1 + r mod (n-1), then symmetric pairs
-                int p, qq;
-                if (tid == 0) {
-                    p = 0;
-                    qq = 1 + (r % (n - 1));
-                } else {
-                    p = 1 + ((r + tid) % (n - 1));
-                    qq = 1 + ((r + n - 1 - tid) % (n - 1));
-                }
-                if (p > qq) {
-                    const int tmp = p;
-                    p = qq;
-                    qq = tmp;
-                }
+                int p, q;
+                lsd_round_pair(r, tid, n, p, q);
+                const double apq = B[p * n + q];
+                const float th = (float)(B[q * n + q] - B[p * n + p]) / (float)(2.0 * apq);
+                // no rotation where the entry is zero (in FP32: negligible) or the angle is
+                const float t = fabsf(th) < 1e18f ? copysignf(1.0f, th) / (fabsf(th) + sqrtf(th * th + 1.0f)) : 0.0f;
+                const double td = (double)t, c = rsqrt(1.0 + td * td);
                 s_pair[tid][0] = p;
-                s_pair[tid][1] = qq;
-                const double app = B[p * n + p], aqq = B[qq * n + qq], apq = B[p * n + qq];
-                double c = 1.0, s = 0.0;
-                if (fabs(apq) > 1e-300) {
-                    const double th = (aqq - app) / (2.0 * apq);
-                    const double tt = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-                    c = 1.0 / sqrt(tt * tt + 1.0);
-                    s = tt * c;
-                }
+                s_pair[tid][1] = q;
                 s_cs[tid][0] = c;
-                s_cs[tid][1] = s;
+                s_cs[tid][1] = td * c;
+                rot[(size_t)rounds * half + tid] = make_double2(c, td * c);
             }
             __syncthreads();
-            // rows p, q of B <- J^T B
-            for (int e = tid; e < half * n; e += nt) {
-                const int k = e / n, col = e - k * n;
-                const int p = s_pair[k][0], qq = s_pair[k][1];
-                const double c = s_cs[k][0], s = s_cs[k][1];
-                const double bp = B[p * n + col], bq = B[qq * n + col];
-                B[p * n + col] = c * bp - s * bq;
-                B[qq * n + col] = s * bp + c * bq;
-            }
-            __syncthreads();
-            // columns p, q of B <- B J, and of V
-            for (int e = tid; e < half * n; e += nt) {
-                const int k = e / n, row = e - k * n;
-                const int p = s_pair[k][0], qq = s_pair[k][1];
-                const double c = s_cs[k][0], s = s_cs[k][1];
-                const double bp = B[row * n + p], bq = B[row * n + qq];
-                B[row * n + p] = c * bp - s * bq;
-                B[row * n + qq] = s * bp + c * bq;
-                const double vp = V[row * n + p], vq = V[row * n + qq];
-                V[row * n + p] = c * vp - s * vq;
-                V[row * n + qq] = s * vp + c * vq;
+            for (int e = tid; e < nblk; e += nt) {
+                // block (k1, k2), k1 <= k2, of the triangle in row order
+                int k2 = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+                while (k2 * (k2 + 1) / 2 > e) --k2;
+                while ((k2 + 1) * (k2 + 2) / 2 <= e) ++k2;
+                const int k1 = e - k2 * (k2 + 1) / 2;
+                const int p1 = s_pair[k1][0], q1 = s_pair[k1][1], p2 = s_pair[k2][0], q2 = s_pair[k2][1];
+                const double c1 = s_cs[k1][0], s1 = s_cs[k1][1], c2 = s_cs[k2][0], s2 = s_cs[k2][1];
+                const double a = B[p1 * n + p2], b = B[p1 * n + q2], c = B[q1 * n + p2], dd = B[q1 * n + q2];
+                const double ra = c1 * a - s1 * c, rb = c1 * b - s1 * dd, rc = s1 * a + c1 * c, rd = s1 * b + c1 * dd;
+                const double oa = c2 * ra - s2 * rb, ob = s2 * ra + c2 * rb, oc = c2 * rc - s2 * rd, od = s2 * rc + c2 * rd;
+                B[p1 * n + p2] = B[p2 * n + p1] = oa;
+                B[q1 * n + q2] = B[q2 * n + q1] = od;
+                if (k1 == k2) {
+                    B[p1 * n + q1] = B[q1 * n + p1] = 0.5 * (ob + oc);
+                } else {
+                    B[p1 * n + q2] = B[q2 * n + p1] = ob;
+                    B[q1 * n + p2] = B[p2 * n + q1] = oc;
+                }
             }
             __syncthreads();
         }
@@ -177,190 +264,212 @@ __device__ void lsd_jacobi(double* B, double* V, int n, double* red) {
             if (rr == cc) dia += B[e] * B[e];
             else off += B[e] * B[e];
         }
-        red[tid] = off;
-        red[nt + tid] = dia;
+        off = warp_sum(off);
+        dia = warp_sum(dia);
+        if ((tid & 31) == 0) {
+            red[tid >> 5] = off;
+            red[32 + (tid >> 5)] = dia;
+        }
         __syncthreads();
         if (tid == 0) {
-            double o = 0.0, d = 0.0;
-            for (int k = 0; k < nt; ++k) {
+            double o = 0.0, dsum = 0.0;
+            for (int k = 0; k < nt / 32; ++k) {
                 o += red[k];
-                d += red[nt + k];
+                dsum += red[32 + k];
             }
-            s_go = o > 1e-32 * d;
+            s_go = o > 1e-32 * dsum;
         }
         __syncthreads();
         if (!s_go) break;
     }
+    return rounds;
 }
 
-__global__ void k_lsd_local(LsdDev d, const double* xl, const double* wl, const int* nbase, double* gtab, double* lam_out,
-                            double* coef_out, int* err) {
+// Eigenproblem of one subdomain: Cholesky of the overlap, L^-1 H L^-T, Jacobi,
+// the M lowest eigenvectors, back substitution and the sign.  Shared memory:
+// A (overlap, then its factor in the lower triangle) | B (Hamiltonian, then
+// L^-1 H L^-T) | V (scratch, then the wanted eigenvectors) | W (scratch), each
+// n x n with n = kd rounded up to even; the padded index is decoupled (zero
+// off-diagonal entries, so no rotation touches it) and not ranked.
+__global__ void __launch_bounds__(256) k_lsd_local(LsdDev d, const double* mat, double2* rot_all, double* lam_out,
+                                                   double* coef_out, int* err) {
     extern __shared__ double lsm[];
-    const int i = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-    const int kd = d.kd, n = (kd + 1) & ~1;
+    const int i = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int kd = d.kd, n = (kd + 1) & ~1, half = n / 2;
     double* A = lsm;
     double* B = A + n * n;
     double* V = B + n * n;
-    double* W = V + n * n;  // scratch n x n
-    double* red = W + n * n;  // 2 nt
+    double* W = V + n * n;
+    double* red = W + n * n;  // 64
     __shared__ int s_ord[LSD_KD_MAX];
-    __shared__ double s_sign[LSD_KD_MAX];
-    const int n0 = nbase[i], nn = nbase[i + 1] - n0;
-    const double* x = xl + n0;
-    const double* w = wl + n0;
-    const double xc = lsd_centre(d, i);
-    const double h = 2.0 * d.xb / (kd - 1);
-    double* g = gtab + (size_t)n0 * 2 * LSD_KD_MAX;  // [nn][kd] values then [nn][kd] derivatives
-    double* dg = g + (size_t)nn * LSD_KD_MAX;
-    for (int e = tid; e < nn * kd; e += nt) {
-        const int m = e / kd, k = e - m * kd;
-        const double al = (k == kd - 1) ? xc + d.xb : (double)k * h + (xc - d.xb);
-        const double u = x[m] - al, gv = exp(-d.delta * u * u);
-        g[(size_t)m * LSD_KD_MAX + k] = gv;
-        dg[(size_t)m * LSD_KD_MAX + k] = -2.0 * d.delta * u * gv;
-    }
-    __syncthreads();
-    // overlap and Hamiltonian (upper triangle computed, both filled)
+    __shared__ double s_inv[LSD_KD_MAX];  // 1 / L_jj
+    const double* Mi = mat + (size_t)i * kd * (2 * kd + 1);
+    double2* rot = rot_all + (size_t)i * LSD_SWEEPS * (n - 1) * half;
     for (int e = tid; e < n * n; e += nt) {
         const int r = e / n, c = e - r * n;
-        if (r >= kd || c >= kd) {
-            A[e] = (r == c) ? 1.0 : 0.0;
-            B[e] = (r == c) ? 1e30 : 0.0;
-            continue;
-        }
-        if (c < r) continue;
-        double s = 0.0, hh = 0.0;
-        for (int m = 0; m < nn; ++m) {
-            const double sw = lsd_switch(d, x[m], xc);
-            const double gr = g[(size_t)m * LSD_KD_MAX + r], gc = g[(size_t)m * LSD_KD_MAX + c];
-            const double dr = dg[(size_t)m * LSD_KD_MAX + r], dc = dg[(size_t)m * LSD_KD_MAX + c];
-            s += w[m] * gr * gc;
-            hh += w[m] * (0.5 * (1.0 - sw) * dr * dc + (lsd_ven(d, x[m]) + d.v_inf * sw) * gr * gc);
-        }
-        A[r * n + c] = A[c * n + r] = s;
-        B[r * n + c] = B[c * n + r] = hh;
+        const bool in = r < kd && c < kd;
+        A[e] = in ? Mi[r * kd + c] : (r == c ? 1.0 : 0.0);
+        B[e] = in ? Mi[kd * kd + r * kd + c] : 0.0;
     }
     __syncthreads();
-    // Cholesky A = L L^T (lower triangle of A)
+    // Cholesky A = L L^T (right-looking, lower triangle of A)
     for (int j = 0; j < n; ++j) {
-        if (tid == 0) {
+        double ljj = 1.0;
+        if (j + tid < n) {  // only the warps that hold rows take the FP64 root and division
             double s = A[j * n + j];
-            for (int k = 0; k < j; ++k) s -= A[j * n + k] * A[j * n + k];
             if (!(s > 0.0)) {
-                atomicOr(err, 1);
+                if (tid == 0) atomicOr(err, 1);
                 s = 1e-300;
             }
-            A[j * n + j] = sqrt(s);
+            ljj = sqrt(s);
+        }
+        __syncthreads();  // the pivot has been read
+        if (j + tid < n) {
+            const int r = j + tid;
+            A[r * n + j] = r == j ? ljj : A[r * n + j] / ljj;
+            if (r == j) s_inv[j] = 1.0 / ljj;
         }
         __syncthreads();
-        for (int r = j + 1 + tid; r < n; r += nt) {
-            double s = A[r * n + j];
-            for (int k = 0; k < j; ++k) s -= A[r * n + k] * A[j * n + k];
-            A[r * n + j] = s / A[j * n + j];
+        const int m = n - j - 1;
+        for (int e = tid; e < m * m; e += nt) {
+            const int r = j + 1 + e / m, c = j + 1 + e % m;
+            if (c <= r) A[r * n + c] -= A[r * n + j] * A[c * n + j];
         }
         __syncthreads();
     }
-    // W = L^-1 B (forward substitution per column), then B = L^-1 W^T
+    // W = L^-1 B, then V = L^-1 W^T, right-looking row by row
     for (int pass = 0; pass < 2; ++pass) {
-        for (int c = tid; c < n; c += nt) {
-            for (int r = 0; r < n; ++r) {
-                double s = pass == 0 ? B[r * n + c] : W[c * n + r];
-                for (int k = 0; k < r; ++k) s -= A[r * n + k] * (pass == 0 ? W[k * n + c] : V[k * n + c]);
-                if (pass == 0) W[r * n + c] = s / A[r * n + r];
-                else V[r * n + c] = s / A[r * n + r];
-            }
-        }
+        double* X = pass == 0 ? W : V;
+        for (int e = tid; e < n * n; e += nt) X[e] = pass == 0 ? B[e] : W[(e % n) * n + e / n];
         __syncthreads();
+        for (int r = 0; r < n; ++r) {
+            if (tid < n) X[r * n + tid] *= s_inv[r];
+            __syncthreads();
+            for (int e = tid; e < (n - r - 1) * n; e += nt) {
+                const int k = r + 1 + e / n, c = e % n;
+                X[k * n + c] -= A[k * n + r] * X[r * n + c];
+            }
+            __syncthreads();
+        }
     }
     for (int e = tid; e < n * n; e += nt) {
         const int r = e / n, c = e - r * n;
         B[e] = 0.5 * (V[r * n + c] + V[c * n + r]);
     }
     __syncthreads();
-    for (int e = tid; e < n * n; e += nt) V[e] = (e / n == e % n) ? 1.0 : 0.0;
-    __syncthreads();
-    lsd_jacobi(B, V, n, red);
+    const int rounds = lsd_jacobi(B, n, rot, red);
     // ascending order of the eigenvalues (ties by index)
-    if (tid < n) {
+    if (tid < kd) {
         const double lv = B[tid * n + tid];
         int rank = 0;
-        for (int k = 0; k < n; ++k) {
+        for (int k = 0; k < kd; ++k) {
             const double lk = B[k * n + k];
             rank += (lk < lv || (lk == lv && k < tid)) ? 1 : 0;
         }
         s_ord[rank] = tid;
     }
     __syncthreads();
-    // X = L^-T V[:, ord] for the M lowest (back substitution), into W's columns
-    for (int l = tid; l < d.M; l += nt) {
-        const int col = s_ord[l];
+    // the wanted columns of V = J_1 J_2 ... J_R: the rotations applied in reverse
+    // to the unit vectors, one warp per column (lanes over the pairs of a round)
+    for (int l = warp; l < d.M; l += nw) {
+        double* v = V + l * n;
+        for (int k = lane; k < n; k += 32) v[k] = k == s_ord[l] ? 1.0 : 0.0;
+        __syncwarp();
+        for (int t0 = rounds; t0 > 0; t0 -= 4) {
+            double2 cs[4];  // the next four rounds' rotations in flight together
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                cs[u] = t0 - 1 - u >= 0 && lane < half ? rot[(size_t)(t0 - 1 - u) * half + lane] : make_double2(1.0, 0.0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int t = t0 - 1 - u;
+                if (t < 0) break;
+                if (lane < half) {
+                    int p, q;
+                    lsd_round_pair(t % (n - 1), lane, n, p, q);
+                    const double vp = v[p], vq = v[q];
+                    v[p] = cs[u].x * vp + cs[u].y * vq;
+                    v[q] = cs[u].x * vq - cs[u].y * vp;
+                }
+                __syncwarp();
+            }
+        }
+        // X = L^-T v (back substitution, right-looking), then the sign
         for (int r = n - 1; r >= 0; --r) {
-            double s = V[r * n + col];
-            for (int k = r + 1; k < n; ++k) s -= A[k * n + r] * W[k * n + l];
-            W[r * n + l] = s / A[r * n + r];
+            const double x = v[r] * s_inv[r];
+            __syncwarp();
+            for (int k = lane; k <= r; k += 32) v[k] = k == r ? x : v[k] - A[r * n + k] * x;
+            __syncwarp();
         }
-    }
-    __syncthreads();
-    // sign: int phi exp(0.37 (x - xc)) dx > 0
-    for (int l = tid; l < d.M; l += nt) {
         double pr = 0.0;
-        for (int m = 0; m < nn; ++m) {
-            double v = 0.0;
-            for (int k = 0; k < kd; ++k) v += W[k * n + l] * g[(size_t)m * LSD_KD_MAX + k];
-            pr += w[m] * exp(0.37 * (x[m] - xc)) * v;
-        }
-        s_sign[l] = pr < 0.0 ? -1.0 : 1.0;
+        for (int k = lane; k < kd; k += 32) pr += v[k] * Mi[2 * kd * kd + k];
+        pr = warp_sum(pr);
+        const double sg = pr < 0.0 ? -1.0 : 1.0;  // int phi exp(0.37 (x - xc)) dx > 0
+        for (int k = lane; k < kd; k += 32) coef_out[((size_t)i * kd + k) * d.M + l] = sg * v[k];
+        if (lane == 0) lam_out[i * d.M + l] = B[s_ord[l] * n + s_ord[l]];
     }
-    __syncthreads();
-    for (int e = tid; e < kd * d.M; e += nt) {
-        const int k = e / d.M, l = e - k * d.M;
-        coef_out[((size_t)i * kd + k) * d.M + l] = s_sign[l] * W[k * n + l];
-    }
-    for (int l = tid; l < d.M; l += nt) lam_out[i * d.M + l] = B[s_ord[l] * n + s_ord[l]];
 }
 
 // ------------------------------------------- 2. orbitals on the global rule
-__global__ void k_lsd_table(LsdDev d, const double* xg, const double* coef, double* F, double* dF) {
+// Gaussians of subdomain i at global node m (row k: [i][k][ng], values then
+// derivatives) and, in row L kd, w V_en: shared by the M orbitals of i.
+__global__ void k_lsd_gauss(LsdDev d, const double* xg, const double* wg, double* G, double* dG, double* wv) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x, row = blockIdx.y, kd = d.kd;
+    if (m >= d.ng) return;
+    const double x = xg[m];
+    if (row == d.L * kd) {
+        wv[m] = wg[m] * lsd_ven(d, x);
+        return;
+    }
+    const int i = row / kd, k = row - i * kd;
+    const double xc = lsd_centre(d, i), h = 2.0 * d.xb / (kd - 1);
+    const double al = (k == kd - 1) ? xc + d.xb : (double)k * h + (xc - d.xb);
+    const double u = x - al, gv = exp(-d.delta * u * u);
+    G[(size_t)row * d.ng + m] = gv;
+    dG[(size_t)row * d.ng + m] = -2.0 * d.delta * u * gv;
+}
+
+__global__ void k_lsd_table(LsdDev d, const double* G, const double* dG, const double* coef, double* F, double* dF) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.y;
     if (m >= d.ng) return;
     const int i = o / d.M, l = o - i * d.M, kd = d.kd;
-    const double xc = lsd_centre(d, i), h = 2.0 * d.xb / (kd - 1), x = xg[m];
     double v = 0.0, dv = 0.0;
+#pragma unroll 4
     for (int k = 0; k < kd; ++k) {
-        const double al = (k == kd - 1) ? xc + d.xb : (double)k * h + (xc - d.xb);
-        const double u = x - al, gv = exp(-d.delta * u * u), c = coef[((size_t)i * kd + k) * d.M + l];
-        v += c * gv;
-        dv += c * (-2.0 * d.delta * u * gv);
+        const double c = coef[((size_t)i * kd + k) * d.M + l];
+        v += c * G[((size_t)i * kd + k) * d.ng + m];
+        dv += c * dG[((size_t)i * kd + k) * d.ng + m];
     }
     F[(size_t)o * d.ng + m] = v;
     dF[(size_t)o * d.ng + m] = dv;
 }
 
-// One warp per orbital pair (a, b): overlap, one-electron Hamiltonian, position.
-__global__ void k_lsd_one(LsdDev d, const double* xg, const double* wg, const double* F, const double* dF, double* S1,
-                          double* h1, double* J1) {
+// One warp per orbital pair (a, b), b >= a: overlap, one-electron Hamiltonian, position.
+__global__ void k_lsd_one(LsdDev d, const double* xg, const double* wg, const double* wv, const double* F,
+                          const double* dF, double* S1, double* h1, double* J1) {
     const int LM = d.L * d.M;
     const int pr = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (pr >= LM * LM) return;
     const int a = pr / LM, b = pr - a * LM;
+    if (b < a) return;
     const double* fa = F + (size_t)a * d.ng;
     const double* fb = F + (size_t)b * d.ng;
     const double* da = dF + (size_t)a * d.ng;
     const double* db = dF + (size_t)b * d.ng;
     double s = 0.0, hh = 0.0, jj = 0.0;
     for (int m = lane; m < d.ng; m += 32) {
-        const double ff = wg[m] * fa[m] * fb[m];
+        const double pf = fa[m] * fb[m], ff = wg[m] * pf;
         s += ff;
-        hh += 0.5 * wg[m] * da[m] * db[m] + lsd_ven(d, xg[m]) * ff;
+        hh += 0.5 * wg[m] * (da[m] * db[m]) + wv[m] * pf;
         jj += xg[m] * ff;
     }
     s = warp_sum(s);
     hh = warp_sum(hh);
     jj = warp_sum(jj);
     if (lane == 0) {
-        S1[pr] = s;
-        h1[pr] = hh;
-        J1[pr] = jj;
+        S1[pr] = S1[b * LM + a] = s;
+        h1[pr] = h1[b * LM + a] = hh;
+        J1[pr] = J1[b * LM + a] = jj;
     }
 }
 
@@ -523,18 +632,19 @@ void lsd_panels(double lo, double hi, double panel, const std::vector<double>& b
     }
 }
 
+// Device memory of one call: pieces of one allocation, 256-byte aligned.
 struct DevBuf {
-    std::vector<void*> ptrs;
-    ~DevBuf() {
-        for (void* p : ptrs) cudaFree(p);
+    char* base = nullptr;
+    size_t used = 0;
+    ~DevBuf() { cudaFree(base); }
+    template <class T>
+    size_t add(size_t n) {
+        const size_t o = used;
+        used += ((n ? n : 1) * sizeof(T) + 255) & ~(size_t)255;
+        return o;
     }
     template <class T>
-    T* get(size_t n) {
-        void* p = nullptr;
-        if (cudaMalloc(&p, (n ? n : 1) * sizeof(T)) != cudaSuccess) return nullptr;
-        ptrs.push_back(p);
-        return (T*)p;
-    }
+    T* at(size_t o) const { return reinterpret_cast<T*>(base + o); }
 };
 }  // namespace
 
@@ -621,91 +731,101 @@ extern "C" swr_status swr_lsd_build(const swr_lsd_problem* p, swr_lsd_result* ou
         }
     d.n_pairs = (int)pa.size();
     if (d.n_pairs > 65535) return lsd_fail(SWR_EINVAL, "swr_lsd_build: more than 65535 orbital pairs (L M too large)");
-    // device work
+    // device work: the host tables packed into one upload, the results into one
+    // read-back (an allocation and a copy for each array cost a millisecond)
     DevBuf db;
-    double* dt = db.get<double>(LSD_Q_MAX);
-    double* dw = db.get<double>(LSD_Q_MAX);
-    double* dedges = db.get<double>(edges.size());
-    int* debase = db.get<int>(ebase.size());
-    double* dx = db.get<double>((size_t)(nloc + d.ng));
-    double* dwx = db.get<double>((size_t)(nloc + d.ng));
-    int* dnbase = db.get<int>(nbase.size());
-    double* dgtab = db.get<double>((size_t)nloc * 2 * LSD_KD_MAX);
-    double* dlam = db.get<double>((size_t)LM);
-    double* dcoef = db.get<double>((size_t)p->L * p->kd * p->M);
-    double* dF = db.get<double>((size_t)LM * d.ng);
-    double* ddF = db.get<double>((size_t)LM * d.ng);
-    double* dS1 = db.get<double>((size_t)LM * LM);
-    double* dh1 = db.get<double>((size_t)LM * LM);
-    double* dJ1 = db.get<double>((size_t)LM * LM);
-    int* dpa = db.get<int>(pa.size());
-    int* dpc = db.get<int>(pc.size());
-    int* dplo = db.get<int>(plo.size());
-    int* dphi = db.get<int>(phi.size());
-    int* dpid = db.get<int>(pid.size());
-    double* dP = db.get<double>((size_t)d.n_pairs * d.ng);
-    double* dT = db.get<double>((size_t)d.n_pairs * d.ng);
-    double* dWm = db.get<double>((size_t)d.ng * d.ng);
+    const int n = (p->kd + 1) & ~1, np = n_local_panels + n_global_panels;
     const size_t nblk = (size_t)p->L * p->L * p->K * p->K;
-    int* dpairs = db.get<int>((size_t)p->L * p->L * p->K * 2);
-    double* dSl = db.get<double>(nblk);
-    double* dHl = db.get<double>(nblk);
-    double* dGn = db.get<double>(nblk);
-    int* derr = db.get<int>(1);
-    if (!dt || !dw || !dedges || !debase || !dx || !dwx || !dnbase || !dgtab || !dlam || !dcoef || !dF || !ddF ||
-        !dS1 || !dh1 || !dJ1 || !dpa || !dpc || !dplo || !dphi || !dpid || !dP || !dT || !dpairs || !dSl || !dHl ||
-        !dGn || !derr || !dWm) {
+    const size_t o_edges = db.add<double>(edges.size()), o_ebase = db.add<int>(ebase.size()),
+                 o_nbase = db.add<int>(nbase.size()), o_pa = db.add<int>(pa.size()), o_pc = db.add<int>(pc.size()),
+                 o_lo = db.add<int>(plo.size()), o_hi = db.add<int>(phi.size()), o_pid = db.add<int>(pid.size()),
+                 up_bytes = db.used;
+    const size_t o_lam = db.add<double>(LM), o_coef = db.add<double>((size_t)p->L * p->kd * p->M),
+                 o_S1 = db.add<double>((size_t)LM * LM), o_h1 = db.add<double>((size_t)LM * LM),
+                 o_J1 = db.add<double>((size_t)LM * LM), o_pairs = db.add<int>((size_t)p->L * p->L * p->K * 2),
+                 o_Sl = db.add<double>(nblk), o_Hl = db.add<double>(nblk), o_Gn = db.add<double>(nblk),
+                 o_err = db.add<int>(1), down_end = db.used;
+    const size_t o_t = db.add<double>(LSD_Q_MAX), o_w = db.add<double>(LSD_Q_MAX),
+                 o_x = db.add<double>((size_t)(nloc + d.ng)), o_wx = db.add<double>((size_t)(nloc + d.ng)),
+                 o_gtab = db.add<double>(lsd_tab0(nloc, p->kd)),
+                 o_mat = db.add<double>((size_t)p->L * p->kd * (2 * p->kd + 1)),
+                 o_rot = db.add<double2>((size_t)p->L * LSD_SWEEPS * (n - 1) * (n / 2)),
+                 o_G = db.add<double>((size_t)p->L * p->kd * d.ng), o_dG = db.add<double>((size_t)p->L * p->kd * d.ng),
+                 o_wv = db.add<double>(d.ng), o_F = db.add<double>((size_t)LM * d.ng),
+                 o_dF = db.add<double>((size_t)LM * d.ng), o_P = db.add<double>((size_t)d.n_pairs * d.ng),
+                 o_T = db.add<double>((size_t)d.n_pairs * d.ng), o_W = db.add<double>((size_t)d.ng * d.ng);
+    if (cudaMalloc((void**)&db.base, db.used) != cudaSuccess) {
+        db.base = nullptr;
         cudaGetLastError();
         return lsd_fail(SWR_ENOMEM, "swr_lsd_build: device allocation failed");
     }
+    std::vector<char> hbuf(std::max(up_bytes, down_end - up_bytes));
+    auto pack = [&](size_t o, const void* src, size_t bytes) { memcpy(hbuf.data() + o, src, bytes); };
+    pack(o_edges, edges.data(), edges.size() * sizeof(double));
+    pack(o_ebase, ebase.data(), ebase.size() * sizeof(int));
+    pack(o_nbase, nbase.data(), nbase.size() * sizeof(int));
+    pack(o_pa, pa.data(), pa.size() * sizeof(int));
+    pack(o_pc, pc.data(), pc.size() * sizeof(int));
+    pack(o_lo, plo.data(), plo.size() * sizeof(int));
+    pack(o_hi, phi.data(), phi.size() * sizeof(int));
+    pack(o_pid, pid.data(), pid.size() * sizeof(int));
+    double *dt = db.at<double>(o_t), *dw = db.at<double>(o_w), *dx = db.at<double>(o_x), *dwx = db.at<double>(o_wx);
+    double *dlam = db.at<double>(o_lam), *dcoef = db.at<double>(o_coef), *dF = db.at<double>(o_F), *ddF = db.at<double>(o_dF);
+    double *dS1 = db.at<double>(o_S1), *dh1 = db.at<double>(o_h1), *dJ1 = db.at<double>(o_J1);
+    double *dP = db.at<double>(o_P), *dT = db.at<double>(o_T), *dWm = db.at<double>(o_W);
+    const int *dnbase = db.at<int>(o_nbase), *dplo = db.at<int>(o_lo), *dphi = db.at<int>(o_hi), *dpid = db.at<int>(o_pid);
+    int *dpairs = db.at<int>(o_pairs), *derr = db.at<int>(o_err);
     cudaError_t e = cudaSuccess;
 #define LSD_CU(call)                                                               \
     do {                                                                           \
         if (e == cudaSuccess) e = (call);                                          \
     } while (0)
-    LSD_CU(cudaMemcpy(dedges, edges.data(), edges.size() * sizeof(double), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemcpy(debase, ebase.data(), ebase.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemcpy(dnbase, nbase.data(), nbase.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemcpy(dpa, pa.data(), pa.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemcpy(dpc, pc.data(), pc.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemcpy(dplo, plo.data(), plo.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemcpy(dphi, phi.data(), phi.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemcpy(dpid, pid.data(), pid.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LSD_CU(cudaMemset(dpairs, 0xff, (size_t)p->L * p->L * p->K * 2 * sizeof(int)));
-    LSD_CU(cudaMemset(derr, 0, sizeof(int)));
+    LSD_CU(cudaMemcpy(db.base, hbuf.data(), up_bytes, cudaMemcpyHostToDevice));
+    LSD_CU(cudaMemsetAsync(dpairs, 0xff, (size_t)p->L * p->L * p->K * 2 * sizeof(int)));
+    LSD_CU(cudaMemsetAsync(derr, 0, sizeof(int)));
     if (e == cudaSuccess) {
+        int nn_max = 0;
+        for (int i = 0; i < p->L; ++i) nn_max = std::max(nn_max, nbase[i + 1] - nbase[i]);
         k_lsd_gl<<<1, LSD_Q_MAX>>>(p->q_p, dt, dw);
-        const int nn = (n_local_panels + n_global_panels) * p->q_p;
-        k_lsd_nodes<<<(nn + 255) / 256, 256>>>(dedges, debase, n_local_panels + n_global_panels, dt, dw, p->q_p, dx,
-                                                dwx);
-        const int n = (p->kd + 1) & ~1, nt = 256;
-        const size_t smem = (4 * (size_t)n * n + 2 * nt) * sizeof(double);
+        const int nn = np * p->q_p;
+        k_lsd_nodes<<<(nn + 255) / 256, 256>>>(db.at<double>(o_edges), db.at<int>(o_ebase), np, dt, dw, p->q_p, dx, dwx);
+        const int nt = 256;
+        const size_t smem = (4 * (size_t)n * n + 64) * sizeof(double);
         LSD_CU(cudaFuncSetAttribute(k_lsd_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_lsd_local<<<p->L, nt, smem>>>(d, dx, dwx, dnbase, dgtab, dlam, dcoef, derr);
+        k_lsd_local_tab<<<dim3((nn_max * (p->kd + 1) + 255) / 256, p->L), 256>>>(d, dx, dwx, dnbase, db.at<double>(o_gtab));
+        k_lsd_local_mat<<<dim3((p->kd * (p->kd + 1) + 7) / 8, p->L), 256>>>(d, dnbase, db.at<double>(o_gtab),
+                                                                           db.at<double>(o_mat));
+        k_lsd_local<<<p->L, nt, smem>>>(d, db.at<double>(o_mat), db.at<double2>(o_rot), dlam, dcoef, derr);
         const double* xg = dx + nloc;
         const double* wg = dwx + nloc;
-        k_lsd_table<<<dim3((d.ng + 127) / 128, LM), 128>>>(d, xg, dcoef, dF, ddF);
-        k_lsd_one<<<(LM * LM + 7) / 8, 256>>>(d, xg, wg, dF, ddF, dS1, dh1, dJ1);
-        k_lsd_pairs<<<dim3((d.ng + 255) / 256, d.n_pairs), 256>>>(d, wg, dF, dpa, dpc, dP);
+        k_lsd_gauss<<<dim3((d.ng + 127) / 128, p->L * p->kd + 1), 128>>>(d, xg, wg, db.at<double>(o_G), db.at<double>(o_dG),
+                                                                       db.at<double>(o_wv));
+        k_lsd_table<<<dim3((d.ng + 127) / 128, LM), 128>>>(d, db.at<double>(o_G), db.at<double>(o_dG), dcoef, dF, ddF);
+        k_lsd_one<<<(LM * LM + 7) / 8, 256>>>(d, xg, wg, db.at<double>(o_wv), dF, ddF, dS1, dh1, dJ1);
+        k_lsd_pairs<<<dim3((d.ng + 255) / 256, d.n_pairs), 256>>>(d, wg, dF, db.at<int>(o_pa), db.at<int>(o_pc), dP);
         k_lsd_w<<<dim3((d.ng + 255) / 256, d.ng), 256>>>(d, xg, dWm);
         k_lsd_pw<<<dim3((d.ng + 255) / 256, d.n_pairs), 256>>>(d, dWm, dP, dplo, dphi, dT);
         k_lsd_select<<<p->L * p->L, 256>>>(d, dlam, dpairs, derr);
         k_lsd_blocks<<<dim3((p->K * p->K + 7) / 8, p->L * p->L), 256>>>(d, dpairs, dS1, dh1, dT, dP, dpid, dplo, dphi,
-                                                                       dSl, dHl, dGn);
+                                                                       db.at<double>(o_Sl), db.at<double>(o_Hl),
+                                                                       db.at<double>(o_Gn));
         LSD_CU(cudaGetLastError());
-        LSD_CU(cudaDeviceSynchronize());
     }
     int herr = 0;
-    LSD_CU(cudaMemcpy(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->lam, dlam, (size_t)LM * sizeof(double), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->coef, dcoef, (size_t)p->L * p->kd * p->M * sizeof(double), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->S1, dS1, (size_t)LM * LM * sizeof(double), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->h1, dh1, (size_t)LM * LM * sizeof(double), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->J1, dJ1, (size_t)LM * LM * sizeof(double), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->pairs, dpairs, (size_t)p->L * p->L * p->K * 2 * sizeof(int), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->S_lsd, dSl, nblk * sizeof(double), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->H_lsd, dHl, nblk * sizeof(double), cudaMemcpyDeviceToHost));
-    LSD_CU(cudaMemcpy(out->G_next, dGn, nblk * sizeof(double), cudaMemcpyDeviceToHost));
+    LSD_CU(cudaMemcpy(hbuf.data(), db.base + up_bytes, down_end - up_bytes, cudaMemcpyDeviceToHost));
+    if (e == cudaSuccess) {
+        auto take = [&](void* dst, size_t o, size_t bytes) { memcpy(dst, hbuf.data() + (o - up_bytes), bytes); };
+        take(&herr, o_err, sizeof(int));
+        take(out->lam, o_lam, (size_t)LM * sizeof(double));
+        take(out->coef, o_coef, (size_t)p->L * p->kd * p->M * sizeof(double));
+        take(out->S1, o_S1, (size_t)LM * LM * sizeof(double));
+        take(out->h1, o_h1, (size_t)LM * LM * sizeof(double));
+        take(out->J1, o_J1, (size_t)LM * LM * sizeof(double));
+        take(out->pairs, o_pairs, (size_t)p->L * p->L * p->K * 2 * sizeof(int));
+        take(out->S_lsd, o_Sl, nblk * sizeof(double));
+        take(out->H_lsd, o_Hl, nblk * sizeof(double));
+        take(out->G_next, o_Gn, nblk * sizeof(double));
+    }
 #undef LSD_CU
     if (e != cudaSuccess) {
         char msg[256];

@@ -96,3 +96,20 @@ def test_lsd_build_rejects_invalid_problems(S):
     with pytest.raises(S.SWRError) as e:
         S.lsd_build(kd=65)
     assert e.value.status == S.SWR_EINVAL
+
+
+@pytest.mark.parametrize("kd", [2, 3, 25, 33, 64])
+def test_lsd_orbitals_across_basis_sizes(S, kd):
+    """The eigenproblem kernel at its edges: the smallest basis, odd bases (a
+    padded index that must not be ranked), more than one warp of rows, the
+    largest.  Orbital energies of a well-conditioned basis agree to 1e-10 of
+    the largest one, S1 of a subdomain's own orbitals is the identity."""
+    kw = dict(box=(-4.0, 4.0), L=2, overlap=0.3, M=min(kd, 6), K=1, kd=kd, q_p=10, panel=0.25)
+    p = Lo.LsdProblem(**kw)
+    ref = np.array([o.lam for o in Lo.all_orbitals(p)])
+    got = S.lsd_build(**kw)
+    assert np.abs(got["lam"] - ref).max() <= 1e-10 * max(1.0, np.abs(ref).max())
+    M = kw["M"]
+    for i in range(2):
+        blk = got["S1"][i * M:(i + 1) * M, i * M:(i + 1) * M]
+        assert np.abs(blk - np.eye(M)).max() <= 1e-10
