@@ -65,6 +65,30 @@ def test_mlp_full_width_products_match_oracle(mods):
     assert np.abs(y - yr).max() <= 1e-2 * np.abs(yr).max()
 
 
+@pytest.mark.parametrize("batch", [1, 127, 128, 129, 700])
+@pytest.mark.parametrize("dims", [[1, 3, 2], [17, 65, 65, 100], [130, 192, 64]])
+def test_mlp_products_at_tile_edges(mods, batch, dims):
+    # rows and columns one short of, at and past the 128-row and 64-column
+    # tiles, a contraction padded to 64, one to several row blocks in the
+    # gradients' sums; BF16 operand rounding (2^-9) and its flips bound the
+    # gradient at 1e-2 of its norm, the output at 1e-2 of its largest value
+    torch, S, Lrn = mods
+    rng = np.random.default_rng(batch)
+    x = rng.normal(size=(batch, dims[0])).astype(np.float32)
+    t = rng.normal(size=(batch, dims[-1])).astype(np.float32)
+    p = Lrn.init_params(dims, 11)
+    mlp = S.MLP(dims[0], dims[1], len(dims) - 2, dims[-1])
+    mlp.set_params(p)
+    xd, td = torch.as_tensor(x, device="cuda"), torch.as_tensor(t, device="cuda")
+    loss, g = mlp.train_step(xd, td, 0.0, want_grad=True)
+    ref_loss, ref_g = M.loss_and_grad(p.astype(np.float64), dims, x, t, bf16=True)
+    assert abs(loss - ref_loss) <= 2e-3 * ref_loss
+    assert np.linalg.norm(g - ref_g) <= 1e-2 * np.linalg.norm(ref_g)
+    y = mlp.forward(xd).cpu().numpy()
+    yr = M.forward(p.astype(np.float64), dims, x, bf16=True)[-1]
+    assert np.abs(y - yr).max() <= 1e-2 * np.abs(yr).max()
+
+
 def test_mlp_training_reduces_loss(mods):
     torch, S, Lrn = mods
     rng = np.random.default_rng(2)
