@@ -59,7 +59,9 @@ typedef enum swr_precision {
     SWR_PREC_MIXED = 1,  /* step matrices stored as FP32 hi/lo pairs (four planes for
                             the complex real-time G0) with error-free FP32
                             accumulation: FP64-level accuracy on the FP32 pipes;
-                            FP64 reductions, norms, orthogonalisation, inversion  */
+                            FP64 reductions, norms, orthogonalisation, inversion.
+                            Real time runs the same fixed-point window as
+                            SWR_PREC_FP64 (56-bit matrices and vectors)          */
     SWR_PREC_FP32_REFINED = 2 /* the Schwarz iterations first run with the step
                             matrices rounded to FP32 (only the hi plane of
                             SWR_PREC_MIXED is read: 4 bytes per real element, 8
@@ -351,7 +353,9 @@ typedef enum swr_field {
                                    [10] algorithmic step-matrix bytes of the window
                                        kernels: per real matrix element 8 (the FP64
                                        value or its FP32 hi/lo pair) or 4 (FP32-rounded
-                                       matrix), per complex one 16 or 8; K^2 elements
+                                       matrix), per complex one 8 (half of a symmetric
+                                       matrix at 16; SWR_PREC_FP32_REFINED: 8 or 16 of
+                                       all of it); K^2 elements
                                        per local step solve (imaginary time) or per
                                        matrix sweep (real time)                     */
     SWR_FIELD_CVTOT = 12        /* double[n_instances]: interface mismatch of the last

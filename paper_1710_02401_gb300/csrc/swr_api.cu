@@ -50,7 +50,7 @@ cudaError_t launch_energy(const SwrDeviceView& v, cudaStream_t st, const int* d_
 size_t energy_smem(const SubDev& s);
 cudaError_t launch_tdse_window(const SwrDeviceView& v, cudaStream_t st, const long long* d_boff, const int* d_win_prev,
                                int n_steps, const unsigned char* h_need, const unsigned char* d_need, int max_K,
-                               int max_kd, bool df32, bool onep, long long* launches);
+                               int max_kd, bool onep, long long* launches);
 cudaError_t launch_split_c_df32(const SwrDeviceView& v, cudaStream_t st, int max_K);
 }  // namespace swr
 
@@ -89,6 +89,11 @@ struct swr_ctx {
     std::vector<unsigned char> cn_need;  // real time: fixed-point iterations [step][subdomain]
     std::vector<double> cn_sweeps;       // real time: matvecs with G0 per subdomain over the whole window
     unsigned char* d_cn_need = nullptr;
+    bool rt = false;                     // real time in fixed point (every precision but SWR_PREC_FP32_REFINED)
+    RtPlan rt_shape = {1, 1, 0};
+    int qel = 0;                         // real time: elements of the largest subdomain's Q' factors
+    unsigned* d_sweeps = nullptr;
+    std::vector<unsigned> sweeps_h;
     int* d_rtiles = nullptr;        // Robin response: first product tile of every subdomain
     double* d_dipole = nullptr;
     std::vector<double> dipole_h;
@@ -596,6 +601,8 @@ static void plan(swr_ctx* c) {
     long long off = 0, po = 0;
     c->cap = 0;
     c->tdse = p.instances[0].mode == SWR_MODE_TDSE;
+    c->rt = c->tdse && p.precision != SWR_PREC_FP32_REFINED;
+    c->qel = 0;
     const int cx = c->tdse ? 2 : 1;
     for (int i = 0; i < p.n_instances; ++i) {
         const swr_instance& in = c->inst_h[i];
@@ -709,6 +716,10 @@ static void plan(swr_ctx* c) {
                     off = align32(off + 2LL * K);
                 }
             }
+            if (c->tdse) {
+                const int qe = (d.N == 2 ? 2 : 1) * kd * kd;
+                if (qe > c->qel) c->qel = qe;
+            }
             s.Gf = 0;
             s.Wf = 0;
             s.GE = s.Hr = s.Wr = 0;
@@ -752,9 +763,9 @@ static void plan(swr_ctx* c) {
             s.Wr = off; off = align32(off + (long long)(c->cap + 1) * df32_ld((int)K));
             if (J > c->max_J) c->max_J = (int)J;
         }
-        if (c->df32 && c->tdse) {
+        if (c->df32 && c->tdse && !c->rt) {
             s.Gf = off; off = align32(off + 2LL * K * df32_ld((int)K));  // four FP32 planes of the complex G0 [K][ld]
-        } else if (c->df32) {
+        } else if (c->df32 && !c->tdse) {
             s.Gf = off; off = align32(off + K * df32_ld((int)K));  // G_hi, G_lo planes [K][ldg]
             if (c->has_w) {
                 s.Wf = off; off = align32(off + K * df32_ld((int)K));  // W_hi, W_lo planes [K][ld]
@@ -765,7 +776,9 @@ static void plan(swr_ctx* c) {
     c->psi_total = po;
     int nmax = 0;
     for (const InstDev& d : c->inst) nmax = (d.mode == SWR_MODE_TDSE && d.window_cap > nmax) ? d.window_cap : nmax;
-    plan_cn_iterations(c, nmax);
+    c->cn_need.clear();
+    c->cn_sweeps.assign(c->sub.size(), 0.0);
+    if (!c->rt) plan_cn_iterations(c, nmax);
     c->energy_smem = 0;
     for (const SubDev& s : c->sub) c->energy_smem = energy_smem(s) > c->energy_smem ? energy_smem(s) : c->energy_smem;
 }
@@ -774,7 +787,7 @@ static void plan(swr_ctx* c) {
 struct AuxPlan {
     size_t inst, sub, err, jobs1, jobs2, norm_part, tasks, task0, part_s, part_d, cta0, tc, scal, alive, own,
         ctal, wfix, snorm, sums_s, sums_d,
-        n_active, win, win_prev, bar, queue, qlist, clslots, cnneed, rtiles, res_part, res, cv_part, cvtot, epart, energy, norm2, dipole, boff,
+        n_active, win, win_prev, bar, queue, qlist, clslots, cnneed, sweeps, rtiles, res_part, res, cv_part, cvtot, epart, energy, norm2, dipole, boff,
         psi, psi_off, tg, total;
 };
 static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -819,6 +832,7 @@ static AuxPlan aux_plan(const swr_ctx* c) {
     a.dipole = o; o = al256(o + ni * sizeof(double));
     a.boff = o; o = al256(o + (c->boff.size() + 1) * sizeof(long long));
     a.cnneed = o; o = al256(o + c->cn_need.size() + 1);
+    a.sweeps = o; o = al256(o + ns * sizeof(unsigned));
     a.rtiles = o; o = al256(o + (ns + 1) * sizeof(int));
     a.psi = o; o = al256(o + (size_t)c->psi_total * sizeof(double) * (c->tdse ? 2 : 1));
     a.psi_off = o; o = al256(o + ns * sizeof(long long));
@@ -994,6 +1008,7 @@ extern "C" swr_status swr_setup(const swr_problem* p, swr_ctx** out) {
     c->d_dipole = (double*)(b + a.dipole);
     c->d_boff = (long long*)(b + a.boff);
     c->d_cn_need = (unsigned char*)(b + a.cnneed);
+    c->d_sweeps = (unsigned*)(b + a.sweeps);
     c->d_rtiles = (int*)(b + a.rtiles);
     c->d_psi = (double*)(b + a.psi);
     c->d_psi_off = (long long*)(b + a.psi_off);
@@ -1044,6 +1059,9 @@ extern "C" swr_status swr_setup(const swr_problem* p, swr_ctx** out) {
         if (!c->cn_need.empty())
             CU(cudaMemcpyAsync(c->d_cn_need, c->cn_need.data(), c->cn_need.size(), cudaMemcpyHostToDevice, c->stream));
     c->counters[8] += (double)(c->inst.size() * sizeof(InstDev) + c->sub.size() * (sizeof(SubDev) + 2 * sizeof(GemmJob) + sizeof(long long)));
+    c->sweeps_h.assign(c->sub.size(), 0);
+    if (c->rt && !rt_plan((int)c->sub.size(), c->max_K, c->qel, &c->rt_shape))
+        return fail(c, SWR_EINVAL, "the real-time window does not fit on an SM");
     CU(cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream));
     CU(cudaMemsetAsync(c->d_win_prev, 0, c->inst.size() * sizeof(int), c->stream));
     CU(cudaMemsetAsync(c->d_win, 0, c->inst.size() * sizeof(int), c->stream));
@@ -1100,7 +1118,8 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     CU(launch_assemble(view(c), c->stream, c->max_q, c->max_kd, c->max_K, c->any_ee, c->tdse, !c->tdse,
                        c->d_jobs1, c->d_jobs2, c->d_norm_part, c->tg));
     if (c->df32 && !c->tdse) CU(launch_split_df32(view(c), c->stream, c->max_K, c->has_w));
-    if (c->df32 && c->tdse) CU(launch_split_c_df32(view(c), c->stream, c->max_K));
+    if (c->rt) CU(launch_rt_pack(view(c), c->stream, c->max_K));
+    else if (c->tdse) CU(launch_split_c_df32(view(c), c->stream, c->max_K));
     if (c->robin_w) CU(launch_robin_ge(view(c), c->stream, c->max_K, c->max_J));
     CU(cudaEventRecord(c->ev1, c->stream));
     swr_status st = check_err(c);
@@ -1110,7 +1129,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     c->counters[6] += ams;
     c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 3) : 0) +
                       (c->tg ? 4 : 2) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
-                      (c->df32 ? (c->tdse || !c->has_w ? 1 : 2) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0);
+                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0);
     c->assembled = true;
     c->k = 0;
     c->parity = 0;
@@ -1176,10 +1195,15 @@ static cudaError_t record_iteration(swr_ctx* c, cudaStream_t st, long long* win_
         int nmax = 0;
         for (size_t i = 0; i < c->inst.size(); ++i) nmax = c->inst[i].window_cap > nmax ? c->inst[i].window_cap : nmax;
         e = record_event(c->evw0, st);
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && c->rt) {
+            *win_launches = 2;
+            // (the normalisation factors' array holds the field: real time has none)
+            e = launch_rt_window(view(c), st, c->rt_shape, c->d_boff, c->d_win_prev, c->d_snorm, c->cap, c->d_sweeps,
+                                 c->max_K, c->qel, c->spin_limit);
+        } else if (e == cudaSuccess) {
             e = launch_tdse_window(view(c), st, c->d_boff, c->d_win_prev, nmax, c->cn_need.data(), c->d_cn_need,
-                                   c->max_K, c->max_kd,
-                                   c->df32, fp32_phase(c), win_launches);
+                                   c->max_K, c->max_kd, fp32_phase(c), win_launches);
+        }
         if (e == cudaSuccess) e = record_event(c->evw1, st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(c->d_win, c->d_wfix, c->inst.size() * sizeof(int), cudaMemcpyDeviceToDevice, st);
@@ -1268,6 +1292,11 @@ extern "C" swr_status swr_step(swr_ctx* c, swr_iter_report* rep) {
     CU(cudaMemcpyAsync(c->dipole_h.data(), c->d_dipole, ni * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     if (c->prob.cvtot_each_iteration)
         CU(cudaMemcpyAsync(c->cvtot_h.data(), c->d_cvtot, ni * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    if (c->rt) {
+        const size_t nb = c->sub.size() * sizeof(unsigned);
+        CU(cudaMemcpyAsync(c->sweeps_h.data(), c->d_sweeps, nb, cudaMemcpyDeviceToHost, c->stream));
+        c->counters[9] += (double)nb;
+    }
     c->counters[9] += (double)(ni * ((c->prob.cvtot_each_iteration ? 5 : 4) * sizeof(double) + sizeof(int)));
     swr_status st = check_err(c);
     if (st != SWR_OK) return st;
@@ -1297,19 +1326,20 @@ extern "C" swr_status swr_step(swr_ctx* c, swr_iter_report* rep) {
     {
         std::vector<int> nsolve(c->inst.size());
         for (size_t i = 0; i < ni; ++i) nsolve[i] = c->win_h[i];
-        // bytes per matrix element: complex G0 16 (FP64 pair or four FP32 planes);
+        // bytes per matrix element: complex G0 16 (four FP32 planes), 8 in fixed
+        // point (only the lower triangle is read);
         // real G 8 (FP64 or FP32 hi/lo); the fused variant also streams W (16);
         // half of each with the FP32-rounded matrices (hi planes only)
-        const double bel = (c->tdse ? 16.0 : (c->variant == WIN_FUSED ? 16.0 : 8.0)) * (go ? 0.5 : 1.0);
+        const double bel = (c->rt ? 8.0 : c->tdse ? 16.0 : (c->variant == WIN_FUSED ? 16.0 : 8.0)) * (go ? 0.5 : 1.0);
         for (size_t sid = 0; sid < c->sub.size(); ++sid) {
             const SubDev& sd = c->sub[sid];
             if (c->inst[sd.inst].anti && sd.N == 2 && sd.idx[0] > sd.idx[1]) continue;  // mirror image, not solved
             const double K2 = (double)sd.K * sd.K;
             // real time: (1 + fixed-point iterations) complex matvecs with G0 per step
-            const double mv = c->tdse ? c->cn_sweeps[sid] : (double)nsolve[sd.inst];
+            const double mv = c->rt ? (double)c->sweeps_h[sid] : c->tdse ? c->cn_sweeps[sid] : (double)nsolve[sd.inst];
             flops += (c->tdse ? 8.0 : 2.0) * K2 * mv;
             bytes += bel * K2 * mv;
-            bytes_alg += (c->tdse ? 16.0 : 8.0) * (go ? 0.5 : 1.0) * K2 * mv;
+            bytes_alg += (c->tdse && !c->rt ? 16.0 : 8.0) * (go ? 0.5 : 1.0) * K2 * mv;
         }
     }
     c->counters[0] += wms;

@@ -367,6 +367,16 @@ int robin_columns(const SubDev& s);
 cudaError_t launch_robin_ge(const SwrDeviceView& v, cudaStream_t st, int max_K, int max_J);
 cudaError_t launch_robin_w(const SwrDeviceView& v, cudaStream_t st, const int* d_win_prev, int kd2, int nsm,
                            int* d_tiles);
+// Real-time window (swr_realtime.cu): launch shape, G0 to fixed point at
+// assembly, the window.
+struct RtPlan {
+    int cs, nst, own;
+};
+bool rt_plan(int n_sub, int kmax, int qel, RtPlan* out);
+cudaError_t launch_rt_pack(const SwrDeviceView& v, cudaStream_t st, int max_K);
+cudaError_t launch_rt_window(const SwrDeviceView& v, cudaStream_t st, const RtPlan& plan, const long long* d_boff,
+                             const int* d_win_prev, double* d_theta, int cap, unsigned* d_sweeps, int max_K, int qel,
+                             long long spin_limit);
 void set_error(swr_ctx* c, const char* msg);
 void set_setup_error(const char* msg);
 // Blocks per subdomain of the energy kernel (partials [n_sub][ENERGY_BLOCKS][3]).

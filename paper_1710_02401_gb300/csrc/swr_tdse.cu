@@ -36,23 +36,8 @@ __device__ inline double field_e(const InstDev& in, double t) {
 
 // (Q' x)[r] for rows r of one subdomain, x planar channel in shared memory,
 // the first coordinate's factor transposed (X1t[c kd + a] = Xp1[a][c]: the
-// lanes of a warp, consecutive rows, read consecutive words): FP64 for the
-// plain FP64 path; for the mixed path factors and x as double-single pairs
-// (the products on the FP32 pipes: this part's FP64 unit spends tens of
-// microseconds per launch on them).
-__device__ inline double qx_row(const SubDev& s, const double* X1t, const double* Xp2, const double* x, int r) {
-    const int kd = s.kd;
-    if (s.N == 1) {
-        double acc = 0;
-        for (int c = 0; c < kd; ++c) acc += X1t[c * kd + r] * x[c];
-        return acc;
-    }
-    const int a = r % kd, b = r / kd;
-    double acc = 0;
-    for (int c = 0; c < kd; ++c) acc += X1t[c * kd + a] * x[c + kd * b];
-    for (int e = 0; e < kd; ++e) acc += Xp2[b * kd + e] * x[a + kd * e];
-    return acc;
-}
+// lanes of a warp, consecutive rows, read consecutive words); factors and x as
+// double-single pairs (products on the FP32 pipes).
 __device__ inline double qx_row(const SubDev& s, const float2* X1t, const float2* Xp2, const float2* x, int r) {
     const int kd = s.kd;
     float h = 0.f, l = 0.f;
@@ -74,22 +59,10 @@ __device__ inline bool cn_mirror_skip(const SwrDeviceView& v, const SubDev& s) {
     return in.anti && s.N == 2 && s.idx[0] > s.idx[1];
 }
 
-struct CnBufs {
-    long long r, u, x;   // per-subdomain planar vectors (offsets in doubles, 2K each)
-};
-
-// Shared-memory element of the element-wise kernels: FP64, or a double-single
-// pair on the mixed path.
-template <bool DS> struct CnElem { typedef double T; };
-template <> struct CnElem<true> { typedef float2 T; };
-template <bool DS> __device__ inline typename CnElem<DS>::T cn_elem(double x);
-template <> __device__ inline double cn_elem<false>(double x) { return x; }
-template <> __device__ inline float2 cn_elem<true>(double x) { return dsp_split_int(x); }
-
-// dst[e] (TR: dst[(e % kd) kd + e / kd]) = src[e] for e < n, by the whole
-// CTA: eight loads per thread in flight before the first store.
-template <bool DS, bool TR>
-__device__ inline void cn_stage(typename CnElem<DS>::T* dst, const double* src, int n, int kd) {
+// dst[e] (TR: dst[(e % kd) kd + e / kd]) = src[e] for e < n as double-single
+// pairs, by the whole CTA: eight loads per thread in flight before the first store.
+template <bool TR>
+__device__ inline void cn_stage(float2* dst, const double* src, int n, int kd) {
     for (int base = threadIdx.x; base < n; base += 8 * CN_THREADS) {
         double t[8];
 #pragma unroll
@@ -100,13 +73,12 @@ __device__ inline void cn_stage(typename CnElem<DS>::T* dst, const double* src, 
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int e = base + u * CN_THREADS;
-            if (e < n) dst[TR ? (e % kd) * kd + e / kd : e] = cn_elem<DS>(t[u]);
+            if (e < n) dst[TR ? (e % kd) * kd + e / kd : e] = dsp_split_int(t[u]);
         }
     }
 }
 
 // r = 2c^n + i dth Q' c^n + i hk (b^{n+1} + b^n);  u = r
-template <bool DS>
 __global__ void k_cn_rhs(SwrDeviceView v, const long long* boff, const int* win_prev, int n) {
     const int sid = blockIdx.y;
     const SubDev& s = v.sub[sid];
@@ -114,16 +86,15 @@ __global__ void k_cn_rhs(SwrDeviceView v, const long long* boff, const int* win_
     const int K = s.K, kd = s.kd;
     const int r0 = blockIdx.x * CN_ROWS;
     if (r0 >= K || cn_mirror_skip(v, s)) return;
-    typedef typename CnElem<DS>::T E;
     extern __shared__ double sm_raw[];
-    E* c = reinterpret_cast<E*>(sm_raw);  // 2K
-    E* X1 = c + 2 * K;                     // kd^2, transposed
-    E* X2 = X1 + kd * kd;                  // kd^2
+    float2* c = reinterpret_cast<float2*>(sm_raw);  // 2K
+    float2* X1 = c + 2 * K;                     // kd^2, transposed
+    float2* X2 = X1 + kd * kd;                  // kd^2
     T1Layout lay(s.q, kd);
     const double* cn = v.arena + s.hist + (long long)n * 2 * K;
-    cn_stage<DS, false>(c, cn, 2 * K, kd);
-    cn_stage<DS, true>(X1, v.arena + s.t1[0] + lay.mat(M_XP), kd * kd, kd);
-    cn_stage<DS, false>(X2, v.arena + s.t1[s.N == 2 ? 1 : 0] + lay.mat(M_XP), kd * kd, kd);
+    cn_stage<false>(c, cn, 2 * K, kd);
+    cn_stage<true>(X1, v.arena + s.t1[0] + lay.mat(M_XP), kd * kd, kd);
+    cn_stage<false>(X2, v.arena + s.t1[s.N == 2 ? 1 : 0] + lay.mat(M_XP), kd * kd, kd);
     // the field at t_n and t_{n+1}: once per CTA (the FP64 sines of every
     // thread would take most of the launch on this part's FP64 unit)
     __shared__ double s_th[2];
@@ -155,44 +126,8 @@ __global__ void k_cn_rhs(SwrDeviceView v, const long long* boff, const int* win_
     }
 }
 
-// x = G0 u  (complex, FP64); one warp per row, lanes over the columns.
-// need (nullable): fixed-point iterations of this step per subdomain; the
-// launch of iteration m skips the subdomains that need no more than m.
-__global__ void __launch_bounds__(256) k_cmv(SwrDeviceView v, const long long* boff, const unsigned char* need,
-                                             int m) {
-    const int sid = blockIdx.y;
-    const SubDev& s = v.sub[sid];
-    const int K = s.K;
-    const int r0 = blockIdx.x * MV_ROWS;
-    if (r0 >= K || (need && m >= need[sid]) || cn_mirror_skip(v, s)) return;
-    extern __shared__ double sm[];
-    const double* U = v.arena + boff[3 * sid + 1];
-    for (int e = threadIdx.x; e < 2 * K; e += blockDim.x) sm[e] = U[e];
-    __syncthreads();
-    const double2* G = (const double2*)(v.arena + s.Gm);
-    double* X = v.arena + boff[3 * sid + 2];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int r = r0 + warp; r < min(K, r0 + MV_ROWS); r += nw) {
-        const double2* g = G + (long long)r * K;
-        double are = 0, aim = 0;
-        for (int c = lane; c < K; c += 32) {
-            const double2 gg = g[c];
-            const double ur = sm[c], ui = sm[K + c];
-            are = fma(gg.x, ur, fma(-gg.y, ui, are));
-            aim = fma(gg.x, ui, fma(gg.y, ur, aim));
-        }
-        are = warp_sum(are);
-        aim = warp_sum(aim);
-        if (lane == 0) {
-            X[r] = are;
-            X[K + r] = aim;
-        }
-    }
-}
-
 // u = r - i theta_{n+1} Q' x  (fixed-point iteration m; the subdomains that
 // need no more than m iterations at this step are skipped)
-template <bool DS>
 __global__ void k_cn_update(SwrDeviceView v, const long long* boff, int n, const unsigned char* need, int m) {
     const int sid = blockIdx.y;
     const SubDev& s = v.sub[sid];
@@ -200,16 +135,15 @@ __global__ void k_cn_update(SwrDeviceView v, const long long* boff, int n, const
     const int K = s.K, kd = s.kd;
     const int r0 = blockIdx.x * CN_ROWS;
     if (r0 >= K || m >= need[sid] || cn_mirror_skip(v, s)) return;
-    typedef typename CnElem<DS>::T E;
     extern __shared__ double sm_raw[];
-    E* x = reinterpret_cast<E*>(sm_raw);
-    E* X1 = x + 2 * K;
-    E* X2 = X1 + kd * kd;
+    float2* x = reinterpret_cast<float2*>(sm_raw);
+    float2* X1 = x + 2 * K;
+    float2* X2 = X1 + kd * kd;
     T1Layout lay(s.q, kd);
     const double* Xg = v.arena + boff[3 * sid + 2];
-    cn_stage<DS, false>(x, Xg, 2 * K, kd);
-    cn_stage<DS, true>(X1, v.arena + s.t1[0] + lay.mat(M_XP), kd * kd, kd);
-    cn_stage<DS, false>(X2, v.arena + s.t1[s.N == 2 ? 1 : 0] + lay.mat(M_XP), kd * kd, kd);
+    cn_stage<false>(x, Xg, 2 * K, kd);
+    cn_stage<true>(X1, v.arena + s.t1[0] + lay.mat(M_XP), kd * kd, kd);
+    cn_stage<false>(X2, v.arena + s.t1[s.N == 2 ? 1 : 0] + lay.mat(M_XP), kd * kd, kd);
     __shared__ double s_th1;
     if (threadIdx.x == 0) s_th1 = 0.5 * in.dt * field_e(in, (n + 1) * in.dt);  // once per CTA
     __syncthreads();
@@ -245,6 +179,8 @@ __device__ inline void ds_mac(float& ah, float& al, float gh, float gl, float xh
 // independent 512-byte requests per warp are in flight.  ONEP: only the hi
 // planes are read (the FP32-rounded G0 of SWR_PREC_FP32_REFINED before its
 // switch, 8 bytes per complex element), their lo terms taken as 0.
+// need (nullable): fixed-point iterations of this step per subdomain; the
+// launch of iteration m skips the subdomains that need no more than m.
 template <bool ONEP>
 __global__ void __launch_bounds__(256) k_cmv_df32(SwrDeviceView v, const long long* boff, const unsigned char* need,
                                                   int m) {
@@ -384,20 +320,13 @@ cudaError_t launch_split_c_df32(const SwrDeviceView& v, cudaStream_t st, int max
 
 cudaError_t launch_tdse_window(const SwrDeviceView& v, cudaStream_t st, const long long* d_boff, const int* d_win_prev,
                                int n_steps, const unsigned char* h_need, const unsigned char* d_need, int max_K,
-                               int max_kd, bool df32, bool onep, long long* launches) {
+                               int max_kd, bool onep, long long* launches) {
     const size_t sm_el = (2 * (size_t)max_K + 2 * (size_t)max_kd * max_kd) * sizeof(double);
     const size_t sm_mv = 2 * (size_t)df32_ld(max_K) * sizeof(double);
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaFuncSetAttribute(k_cn_rhs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        cudaFuncSetAttribute(k_cn_rhs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        cudaFuncSetAttribute(k_cn_update<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        cudaFuncSetAttribute(k_cn_update<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        cudaFuncSetAttribute(k_cmv, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        cudaFuncSetAttribute(k_cmv_df32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        cudaFuncSetAttribute(k_cmv_df32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        attr_done = true;
-    }
+    cudaFuncSetAttribute(k_cn_rhs, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    cudaFuncSetAttribute(k_cn_update, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    cudaFuncSetAttribute(k_cmv_df32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    cudaFuncSetAttribute(k_cmv_df32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
     const dim3 ge(div_up(max_K, CN_ROWS), v.n_sub), gm(div_up(max_K, MV_ROWS), v.n_sub), gf(div_up(2 * max_K, 256), v.n_sub);
     long long nl = 0;
     k_cn_init<<<gf, 256, 0, st>>>(v);
@@ -406,17 +335,13 @@ cudaError_t launch_tdse_window(const SwrDeviceView& v, cudaStream_t st, const lo
         const unsigned char* nd = d_need + (size_t)n * v.n_sub;
         int iters = 0;
         for (int s = 0; s < v.n_sub; ++s) iters = h_need[(size_t)n * v.n_sub + s] > iters ? h_need[(size_t)n * v.n_sub + s] : iters;
-        if (df32) k_cn_rhs<true><<<ge, CN_THREADS, sm_el, st>>>(v, d_boff, d_win_prev, n);
-        else k_cn_rhs<false><<<ge, CN_THREADS, sm_el, st>>>(v, d_boff, d_win_prev, n);
-        if (df32 && onep) k_cmv_df32<true><<<gm, 256, sm_mv, st>>>(v, d_boff, nullptr, 0);
-        else if (df32) k_cmv_df32<false><<<gm, 256, sm_mv, st>>>(v, d_boff, nullptr, 0);
-        else k_cmv<<<gm, 256, sm_mv, st>>>(v, d_boff, nullptr, 0);
+        k_cn_rhs<<<ge, CN_THREADS, sm_el, st>>>(v, d_boff, d_win_prev, n);
+        if (onep) k_cmv_df32<true><<<gm, 256, sm_mv, st>>>(v, d_boff, nullptr, 0);
+        else k_cmv_df32<false><<<gm, 256, sm_mv, st>>>(v, d_boff, nullptr, 0);
         for (int m = 0; m < iters; ++m) {
-            if (df32) k_cn_update<true><<<ge, CN_THREADS, sm_el, st>>>(v, d_boff, n, nd, m);
-            else k_cn_update<false><<<ge, CN_THREADS, sm_el, st>>>(v, d_boff, n, nd, m);
-            if (df32 && onep) k_cmv_df32<true><<<gm, 256, sm_mv, st>>>(v, d_boff, nd, m);
-            else if (df32) k_cmv_df32<false><<<gm, 256, sm_mv, st>>>(v, d_boff, nd, m);
-            else k_cmv<<<gm, 256, sm_mv, st>>>(v, d_boff, nd, m);
+            k_cn_update<<<ge, CN_THREADS, sm_el, st>>>(v, d_boff, n, nd, m);
+            if (onep) k_cmv_df32<true><<<gm, 256, sm_mv, st>>>(v, d_boff, nd, m);
+            else k_cmv_df32<false><<<gm, 256, sm_mv, st>>>(v, d_boff, nd, m);
         }
         k_cn_finish<<<gf, 256, 0, st>>>(v, d_boff, n);
         nl += 3 + 2 * iters;

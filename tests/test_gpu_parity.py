@@ -280,6 +280,22 @@ def test_parity_real_time_mixed_precision(swr_mod):
     _compare(swr_mod, P.small_tdse_2d(), kmax=3, precision=swr_mod.PREC_MIXED)
 
 
+@pytest.mark.parametrize("n_elec,L,K_d", [(1, 3, 2), (1, 2, 64), (1, 2, 65), (1, 2, 96), (2, 2, 3), (2, 2, 8), (2, 3, 9),
+                                          (2, 2, 12), (2, 2, 16)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_parity_real_time_tile_edges(swr_mod, n_elec, L, K_d, precision):
+    # the smallest bases, K one tile exactly and one past it, the largest
+    # one-electron basis, several block columns held on chip, clusters of more
+    # than one CTA per subdomain
+    if n_elec == 1:
+        inst = P.tise_1d_two_subdomains().replace(mode=P.TDSE, mu=-10j, dt=0.01, n_steps=9, L=L, K_d=K_d,
+                                                  delta=max(0.05, P.spacing_rule_delta((-10.0, 10.0), L, 1.0, K_d)),
+                                                  q_p=24, field=(0.5, 0.09, 8.0, 0.3))
+    else:
+        inst = P.small_tdse_2d(L=L, K_d=K_d, q_p=max(6, K_d), n_mid=2, n_steps=9).replace(field=(0.5, 0.09, 8.0, 0.3))
+    _compare(swr_mod, inst, kmax=2, precision=precision)
+
+
 def test_parity_classical_swr_imaginary_time(swr_mod):
     # classical SWR (Dirichlet data mu psi_j, imposed by penalty): FP64 and mixed
     inst = P.small_tise_2d().replace(tc="dirichlet", mu=50.0)
