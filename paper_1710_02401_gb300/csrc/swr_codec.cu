@@ -36,79 +36,72 @@ void codec_release(const swr_ctx* c);
 #define CODEC_SMAX 16
 #define CODEC_TMAX 32
 
-// Gram-Schmidt of the monomials/Chebyshev polynomials on the node set.
-// Phi: [sid][4][q][S] (spatial, per slot), Psi: [window+1][Tm] (shared by all).
-__global__ void k_codec_basis(SwrDeviceView v, double* Phi, double* Psi, int S, int Tm, int W, int qmax) {
-    const int sid = blockIdx.x;
-    const SubDev& s = v.sub[sid];
-    T1Layout lay(s.q, s.kd);
-    if (threadIdx.x == 0) {
-        for (int slot = 0; slot < 4; ++slot) {
-            double* P = Phi + ((long long)sid * 4 + slot) * qmax * S;
-            for (int e = 0; e < qmax * S; ++e) P[e] = 0.0;
-            if (s.gam_off[slot] < 0) continue;
-            const int d = slot / 2;
-            if (s.N == 1) {  // a point: one basis function equal to 1
-                P[0] = 1.0;
-                continue;
+// Orthonormal polynomials of degree < S on m nodes x (given by pos(t) in
+// [-1, 1]) with weights w(t), by one warp: Chebyshev starting vectors, two
+// passes of Gram-Schmidt, lanes over the nodes.  P[t][k], row length ld.
+template <class Pos, class Wt>
+__device__ inline void codec_ortho(double* P, int ld, int m, int S, int lane, Pos pos, Wt wt) {
+    for (int k = 0; k < S; ++k) {
+        for (int t = lane; t < m; t += 32) {
+            const double x = pos(t);
+            double t0 = 1.0, t1 = x, tk = (k == 0) ? 1.0 : x;
+            for (int q = 2; q <= k; ++q) {
+                tk = 2.0 * x * t1 - t0;
+                t0 = t1;
+                t1 = tk;
             }
-            const double* To = v.arena + s.t1[1 - d];
-            const int q = s.q;
-            const double lo = s.lo[1 - d], hi = s.hi[1 - d];
-            for (int k = 0; k < S; ++k) {
-                for (int t = 0; t < q; ++t) {
-                    double x = 2.0 * (To[lay.x() + t] - lo) / (hi - lo) - 1.0;
-                    // Chebyshev T_k(x) as the starting vector
-                    double t0 = 1.0, t1 = x, tk = (k == 0) ? 1.0 : x;
-                    for (int m = 2; m <= k; ++m) {
-                        tk = 2.0 * x * t1 - t0;
-                        t0 = t1;
-                        t1 = tk;
-                    }
-                    P[t * S + k] = tk;
-                }
-                for (int pass = 0; pass < 2; ++pass)
-                    for (int j = 0; j < k; ++j) {
-                        double dot = 0;
-                        for (int t = 0; t < q; ++t) dot += To[lay.w() + t] * P[t * S + k] * P[t * S + j];
-                        for (int t = 0; t < q; ++t) P[t * S + k] -= dot * P[t * S + j];
-                    }
-                double nrm = 0;
-                for (int t = 0; t < q; ++t) nrm += To[lay.w() + t] * P[t * S + k] * P[t * S + k];
-                nrm = sqrt(nrm);
-                for (int t = 0; t < q; ++t) P[t * S + k] /= nrm;
-            }
+            P[(long long)t * ld + k] = tk;
         }
-        if (sid == 0) {
-            for (int k = 0; k < Tm; ++k) {
-                for (int n = 0; n <= W; ++n) {
-                    double x = (W > 0) ? 2.0 * n / W - 1.0 : 0.0;
-                    double t0 = 1.0, t1 = x, tk = (k == 0) ? 1.0 : x;
-                    for (int m = 2; m <= k; ++m) {
-                        tk = 2.0 * x * t1 - t0;
-                        t0 = t1;
-                        t1 = tk;
-                    }
-                    Psi[n * Tm + k] = tk;
-                }
-                for (int pass = 0; pass < 2; ++pass)
-                    for (int j = 0; j < k; ++j) {
-                        double dot = 0;
-                        for (int n = 0; n <= W; ++n) dot += Psi[n * Tm + k] * Psi[n * Tm + j];
-                        for (int n = 0; n <= W; ++n) Psi[n * Tm + k] -= dot * Psi[n * Tm + j];
-                    }
-                double nrm = 0;
-                for (int n = 0; n <= W; ++n) nrm += Psi[n * Tm + k] * Psi[n * Tm + k];
-                nrm = sqrt(nrm);
-                for (int n = 0; n <= W; ++n) Psi[n * Tm + k] /= nrm;
+        for (int pass = 0; pass < 2; ++pass)
+            for (int j = 0; j < k; ++j) {
+                double dot = 0;
+                for (int t = lane; t < m; t += 32) dot += wt(t) * P[(long long)t * ld + k] * P[(long long)t * ld + j];
+                dot = warp_sum(dot);
+                for (int t = lane; t < m; t += 32) P[(long long)t * ld + k] -= dot * P[(long long)t * ld + j];
             }
-        }
+        double nrm = 0;
+        for (int t = lane; t < m; t += 32) nrm += wt(t) * P[(long long)t * ld + k] * P[(long long)t * ld + k];
+        nrm = sqrt(warp_sum(nrm));
+        for (int t = lane; t < m; t += 32) P[(long long)t * ld + k] /= nrm;
     }
 }
 
-// code[sid][slot][ch][s][t] = sum_{node, n} w Phi[node][s] Psi[n][t] g[n][ch][node]
+// Phi: [sid][4][q][S] (spatial, per slot), Psi: [window+1][Tm] (shared by all).
+// One warp per slot of a subdomain, and one for Psi (of block 0): one thread
+// doing all of them took 6.7 ms on 192 subdomains.
+__global__ void k_codec_basis(SwrDeviceView v, double* Phi, double* Psi, int S, int Tm, int W, int qmax) {
+    const int sid = blockIdx.x, slot = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (slot == 4) {
+        if (sid == 0)
+            codec_ortho(Psi, Tm, W + 1, Tm, lane, [&](int n) { return W > 0 ? 2.0 * n / W - 1.0 : 0.0; },
+                        [](int) { return 1.0; });
+        return;
+    }
+    const SubDev& s = v.sub[sid];
+    T1Layout lay(s.q, s.kd);
+    double* P = Phi + ((long long)sid * 4 + slot) * qmax * S;
+    for (int e = lane; e < qmax * S; e += 32) P[e] = 0.0;
+    __syncwarp();
+    if (s.gam_off[slot] < 0) return;
+    if (s.N == 1) {  // a point: one basis function equal to 1
+        if (lane == 0) P[0] = 1.0;
+        return;
+    }
+    const int o = 1 - slot / 2;
+    const double* To = v.arena + s.t1[o];
+    const double lo = s.lo[o], hi = s.hi[o];
+    codec_ortho(P, S, s.q, S, lane, [&](int t) { return 2.0 * (To[lay.x() + t] - lo) / (hi - lo) - 1.0; },
+                [&](int t) { return To[lay.w() + t]; });
+}
+
+// code[sid][slot][ch][s][t] = sum_n Psi[n][t] (sum_node w Phi[node][s] g[n][ch][node]):
+// the inner sums of CODEC_CHUNK steps once into shared memory, then the outer
+// ones (summing over the nodes again for every t did Tm times the work on the
+// FP64 pipe).  Both sums run in the same order as the nested one.
+#define CODEC_CHUNK 32
 __global__ void k_codec_encode(SwrDeviceView v, const double* Phi, const double* Psi, int S, int Tm, int W, int qmax,
                                float* code) {
+    __shared__ double sp[2][CODEC_CHUNK][CODEC_SMAX];
     const int sid = blockIdx.x, slot = blockIdx.y;
     const SubDev& s = v.sub[sid];
     const InstDev& in = v.inst[s.inst];
@@ -119,21 +112,36 @@ __global__ void k_codec_encode(SwrDeviceView v, const double* Phi, const double*
     T1Layout lay(s.q, s.kd);
     const double* P = Phi + ((long long)sid * 4 + slot) * qmax * S;
     const double* To = v.arena + s.t1[s.N == 2 ? 1 - slot / 2 : 0];
-    for (int e = threadIdx.x; e < 2 * S * Tm; e += blockDim.x) {
-        const int ch = e / (S * Tm), k = (e / Tm) % S, t = e % Tm;
-        double acc = 0;
-        if (s.gam_off[slot] >= 0 && ch < nch) {
-            for (int n = 0; n <= W; ++n) {
-                const double* g = v.arena + s.g + ((long long)n * nch + ch) * s.ngam + s.gam_off[slot];
-                double sp = 0;
+    const bool have = s.gam_off[slot] >= 0;
+    double acc[4] = {0, 0, 0, 0};  // entries threadIdx.x + u blockDim.x (at most 2 x 16 x 32 of them)
+    if (have)
+        for (int n0 = 0; n0 <= W; n0 += CODEC_CHUNK) {
+            const int cnt = min(CODEC_CHUNK, W + 1 - n0);
+            for (int e = threadIdx.x; e < nch * cnt * S; e += blockDim.x) {
+                const int k = e % S, r = e / S, ch = r % nch, i = r / nch;
+                const double* g = v.arena + s.g + ((long long)(n0 + i) * nch + ch) * s.ngam + s.gam_off[slot];
+                double a = 0;
                 for (int p = 0; p < npts; ++p) {
                     const double w = (s.N == 1) ? 1.0 : To[lay.w() + p];
-                    sp += w * P[p * S + k] * g[p];
+                    a += w * P[p * S + k] * g[p];
                 }
-                acc += Psi[n * Tm + t] * sp;
+                sp[ch][i][k] = a;
             }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e = threadIdx.x + u * blockDim.x;
+                if (e < nch * S * Tm) {
+                    const int ch = e / (S * Tm), k = (e / Tm) % S, t = e % Tm;
+                    for (int i = 0; i < cnt; ++i) acc[u] += Psi[(n0 + i) * Tm + t] * sp[ch][i][k];
+                }
+            }
+            __syncthreads();
         }
-        out[e] = (float)acc;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int e = threadIdx.x + u * blockDim.x;
+        if (e < 2 * S * Tm) out[e] = (float)acc[u];
     }
 }
 
@@ -257,7 +265,7 @@ extern "C" swr_status swr_trace_codec(swr_ctx* ctx, int S, int Tm, size_t* float
         set_error(ctx, cudaGetErrorString(e));
         return SWR_ENOMEM;
     }
-    k_codec_basis<<<r.n_sub, 32, 0, r.stream>>>(r.v, cs.Phi, cs.Psi, S, Tm, cs.W, cs.qmax);
+    k_codec_basis<<<r.n_sub, 160, 0, r.stream>>>(r.v, cs.Phi, cs.Psi, S, Tm, cs.W, cs.qmax);
     e = cudaStreamSynchronize(r.stream);
     if (e != cudaSuccess) {
         set_error(ctx, cudaGetErrorString(e));
