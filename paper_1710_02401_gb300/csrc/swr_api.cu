@@ -89,6 +89,9 @@ struct swr_ctx {
     std::vector<unsigned char> cn_need;  // real time: fixed-point iterations [step][subdomain]
     std::vector<double> cn_sweeps;       // real time: matvecs with G0 per subdomain over the whole window
     unsigned char* d_cn_need = nullptr;
+    bool oc = false;                     // FP64, automatic plan: on-chip window, one cluster per instance
+    OcPlan oc_shape;
+    int *d_oc_bounds = nullptr, *d_oc_row0 = nullptr;
     bool rt = false;                     // real time in fixed point (every precision but SWR_PREC_FP32_REFINED)
     RtPlan rt_shape = {1, 1, 0};
     int qel = 0;                         // real time: elements of the largest subdomain's Q' factors
@@ -531,6 +534,11 @@ static bool plan_cluster(swr_ctx* c, int rows_req, bool have_dev) {
 
 static bool plan_window(swr_ctx* c, int variant_req, int rows_req, bool have_dev) {
     const int nsm = c->nsm > 0 ? c->nsm : 152;
+    // FP64, nothing asked for: the two-phase recursion on chip where every
+    // instance fits one cluster (2 subdomains of 40 Gaussians: 15.6 -> 2.9 us per
+    // step, 9 of K = 121: 16.0 -> 6.0); the plan below is kept for its tasks
+    c->oc = variant_req == 0 && rows_req == 0 && !c->df32 && !c->tdse && !c->any_anti && have_dev &&
+            oc_plan(c->inst, c->sub, nsm, &c->oc_shape);
     if (variant_req == WIN_CLUSTER) return plan_cluster(c, rows_req, have_dev);
     // automatic plan: the cluster window wherever it fits (mixed precision,
     // imaginary time, every subdomain's rows on chip, one resident cluster per
@@ -787,7 +795,7 @@ static void plan(swr_ctx* c) {
 struct AuxPlan {
     size_t inst, sub, err, jobs1, jobs2, norm_part, tasks, task0, part_s, part_d, cta0, tc, scal, alive, own,
         ctal, wfix, snorm, sums_s, sums_d,
-        n_active, win, win_prev, bar, queue, qlist, clslots, cnneed, sweeps, rtiles, res_part, res, cv_part, cvtot, epart, energy, norm2, dipole, boff,
+        n_active, win, win_prev, bar, queue, qlist, clslots, cnneed, sweeps, ocb, ocr, rtiles, res_part, res, cv_part, cvtot, epart, energy, norm2, dipole, boff,
         psi, psi_off, tg, total;
 };
 static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -833,6 +841,8 @@ static AuxPlan aux_plan(const swr_ctx* c) {
     a.boff = o; o = al256(o + (c->boff.size() + 1) * sizeof(long long));
     a.cnneed = o; o = al256(o + c->cn_need.size() + 1);
     a.sweeps = o; o = al256(o + ns * sizeof(unsigned));
+    a.ocb = o; o = al256(o + ni * 17 * sizeof(int));
+    a.ocr = o; o = al256(o + ns * sizeof(int));
     a.rtiles = o; o = al256(o + (ns + 1) * sizeof(int));
     a.psi = o; o = al256(o + (size_t)c->psi_total * sizeof(double) * (c->tdse ? 2 : 1));
     a.psi_off = o; o = al256(o + ns * sizeof(long long));
@@ -920,6 +930,14 @@ static cudaError_t upload_tasks(swr_ctx* c) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->d_cta_list, c->cta_list.data(), c->cta_list.size() * sizeof(int),
                             cudaMemcpyHostToDevice, c->stream);
+    if (c->oc) {
+        const std::vector<int>&bd = c->oc_shape.bounds, &r0 = c->oc_shape.row0;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(c->d_oc_bounds, bd.data(), bd.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(c->d_oc_row0, r0.data(), r0.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream);
+        c->counters[8] += (double)((bd.size() + r0.size()) * sizeof(int));
+    }
     c->counters[8] += (double)(c->tasks.size() * sizeof(Task) +
                                (c->inst_task0.size() + c->cta_task0.size() + c->cta_list.size()) * sizeof(int));
     return e;
@@ -1009,6 +1027,8 @@ extern "C" swr_status swr_setup(const swr_problem* p, swr_ctx** out) {
     c->d_boff = (long long*)(b + a.boff);
     c->d_cn_need = (unsigned char*)(b + a.cnneed);
     c->d_sweeps = (unsigned*)(b + a.sweeps);
+    c->d_oc_bounds = (int*)(b + a.ocb);
+    c->d_oc_row0 = (int*)(b + a.ocr);
     c->d_rtiles = (int*)(b + a.rtiles);
     c->d_psi = (double*)(b + a.psi);
     c->d_psi_off = (long long*)(b + a.psi_off);
@@ -1121,6 +1141,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     if (c->rt) CU(launch_rt_pack(view(c), c->stream, c->max_K));
     else if (c->tdse) CU(launch_split_c_df32(view(c), c->stream, c->max_K));
     if (c->robin_w) CU(launch_robin_ge(view(c), c->stream, c->max_K, c->max_J));
+    if (c->oc) CU(launch_oc_make_w(view(c), c->stream, c->max_K));
     CU(cudaEventRecord(c->ev1, c->stream));
     swr_status st = check_err(c);
     if (st != SWR_OK) return st;
@@ -1129,7 +1150,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     c->counters[6] += ams;
     c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 3) : 0) +
                       (c->tg ? 4 : 2) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
-                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0);
+                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (c->oc ? 1 : 0);
     c->assembled = true;
     c->k = 0;
     c->parity = 0;
@@ -1185,6 +1206,16 @@ static SweepArgs sweep_args(swr_ctx* c) {
     return a;
 }
 
+// The imaginary-time window between its two events.
+static cudaError_t run_window(swr_ctx* c, SweepArgs& a, cudaStream_t st) {
+    if (!c->oc)
+        return launch_window(a, c->grid, c->win_smem, st, (int)c->inst.size(), c->variant, c->df32, fp32_phase(c), c->evw0,
+                             c->evw1);
+    cudaError_t e = record_event(c->evw0, st);
+    if (e == cudaSuccess) e = launch_oc_window(a, c->oc_shape, c->d_oc_bounds, c->d_oc_row0, st);
+    return e == cudaSuccess ? record_event(c->evw1, st) : e;
+}
+
 // Every launch of one Schwarz iteration (Sec. 5.4 steps 1-5) on stream st:
 // the time window, line traces, averaged Robin data, residual, energy.
 static cudaError_t record_iteration(swr_ctx* c, cudaStream_t st, long long* win_launches) {
@@ -1215,9 +1246,7 @@ static cudaError_t record_iteration(swr_ctx* c, cudaStream_t st, long long* win_
             for (const SubDev& sd : c->sub) kd2 = (sd.N == 2 && sd.kd > kd2) ? sd.kd : kd2;
             e = launch_robin_w(view(c), st, c->d_win_prev, kd2, c->nsm > 0 ? c->nsm : 152, c->d_rtiles);
         }
-        if (e == cudaSuccess)
-            e = launch_window(a, c->grid, c->win_smem, st, (int)c->inst.size(), c->variant, c->df32, fp32_phase(c),
-                              c->evw0, c->evw1);
+        if (e == cudaSuccess) e = run_window(c, a, st);
     }
     if (e == cudaSuccess)
         e = launch_post(view(c), st, c->d_win, c->d_win_prev, c->d_snorm, c->cap, c->parity, c->k == 0 ? 1 : 0,
@@ -1344,7 +1373,7 @@ extern "C" swr_status swr_step(swr_ctx* c, swr_iter_report* rep) {
     }
     c->counters[0] += wms;
     c->counters[1] += 1;
-    c->counters[2] += kStepLaunches - 1 + win_launches + (c->any_anti ? 1 : 0) + (c->prob.cvtot_each_iteration ? 2 : 0) +
+    c->counters[2] += kStepLaunches - 1 + win_launches - (c->oc ? 1 : 0) + (c->any_anti ? 1 : 0) + (c->prob.cvtot_each_iteration ? 2 : 0) +
                       (!c->tdse && c->robin_w && (c->variant == WIN_CLUSTER || c->variant == WIN_SPLIT) ? 3 : 0);
     c->counters[3] += flops;
     c->counters[4] += bytes;
@@ -1386,10 +1415,8 @@ static swr_status time_window_plan(swr_ctx* c, int steps, double* sec_per_step) 
     float best = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
         CU(cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream));
-        CU(launch_window(a, c->grid, c->win_smem, c->stream, (int)c->inst.size(), c->variant, c->df32, fp32_phase(c),
-                         c->evw0,
-                         c->evw1));
-        c->counters[2] += 2;
+        CU(run_window(c, a, c->stream));
+        c->counters[2] += c->oc ? 1 : 2;
         swr_status st = check_err(c);
         if (st != SWR_OK) return st;
         float ms = 0;
@@ -1406,8 +1433,8 @@ extern "C" swr_status swr_window_plan(const swr_ctx* c, swr_tune_report* out) {
     out->variant = c->tdse ? 0 : c->variant;
     out->rows_per_task = c->rows_target;
     out->tasks = (int)c->tasks.size();
-    out->ctas = c->grid;
-    out->task_state_global = c->many;
+    out->ctas = c->oc ? (int)c->inst.size() * c->oc_shape.cs : c->grid;
+    out->task_state_global = c->oc ? 0 : c->many;
     out->graph = (c->prob.launch_mode == SWR_LAUNCH_GRAPH && !c->graph_failed) ? 1 : 0;
     out->tensor_contractions = c->use_tg ? 1 : 0;
     return SWR_OK;
@@ -1439,7 +1466,7 @@ extern "C" swr_status swr_autotune(swr_ctx* c, int steps, swr_tune_report* out) 
     for (size_t i = 0; i < cands.size(); ++i) {
         if (!plan_window(c, cands[i].variant, cands[i].rows, true)) continue;
         if (c->bps < 1 || c->grid > c->bps * c->nsm) continue;
-        std::vector<int> sig = {c->variant, (int)c->tasks.size(), c->grid, c->rows_target};
+        std::vector<int> sig = {c->variant, (int)c->tasks.size(), c->grid, c->rows_target, c->oc ? 1 : 0};
         bool dup = false;
         for (const auto& x : seen) dup = dup || x == sig;
         if (dup) continue;
@@ -1451,7 +1478,7 @@ extern "C" swr_status swr_autotune(swr_ctx* c, int steps, swr_tune_report* out) 
         if (i == 0) t_default = t;
         if (t < best_t) {
             best_t = t;
-            best = {c->variant, c->rows_target};
+            best = c->oc ? cands[i] : Cand{c->variant, c->rows_target};  // (on chip: the automatic plan as it is)
         }
     }
     drop_graphs(c);  // captured with the old plan's launch configuration
@@ -1464,8 +1491,8 @@ extern "C" swr_status swr_autotune(swr_ctx* c, int steps, swr_tune_report* out) 
         out->variant = c->variant;
         out->rows_per_task = c->rows_target;
         out->tasks = (int)c->tasks.size();
-        out->ctas = c->grid;
-        out->task_state_global = c->many;
+        out->ctas = c->oc ? (int)c->inst.size() * c->oc_shape.cs : c->grid;
+        out->task_state_global = c->oc ? 0 : c->many;
         out->candidates = timed;
         out->graph = (c->prob.launch_mode == SWR_LAUNCH_GRAPH && !c->graph_failed) ? 1 : 0;
         out->seconds_per_step = best_t;

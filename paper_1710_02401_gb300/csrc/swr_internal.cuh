@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/swr.h"
 
 #define SWR_MAX_NUC 3
@@ -367,6 +369,15 @@ int robin_columns(const SubDev& s);
 cudaError_t launch_robin_ge(const SwrDeviceView& v, cudaStream_t st, int max_K, int max_J);
 cudaError_t launch_robin_w(const SwrDeviceView& v, cudaStream_t st, const int* d_win_prev, int kd2, int nsm,
                            int* d_tiles);
+// On-chip FP64 window of small instances (swr_onchip.cu): CTAs per instance and
+// the rows of each, W at assembly, the window.
+struct OcPlan {
+    int cs, rows_max, nv_max, lim_max;
+    std::vector<int> bounds, row0;
+};
+bool oc_plan(const std::vector<InstDev>& inst, const std::vector<SubDev>& sub, int nsm, OcPlan* p);
+cudaError_t launch_oc_make_w(const SwrDeviceView& v, cudaStream_t st, int max_K);
+cudaError_t launch_oc_window(const SweepArgs& s, const OcPlan& p, const int* d_bounds, const int* d_row0, cudaStream_t st);
 // Real-time window (swr_realtime.cu): launch shape, G0 to fixed point at
 // assembly, the window.
 struct RtPlan {

@@ -296,6 +296,20 @@ def test_parity_real_time_tile_edges(swr_mod, n_elec, L, K_d, precision):
     _compare(swr_mod, inst, kmax=2, precision=precision)
 
 
+@pytest.mark.parametrize("inst", [
+    P.tise_1d_two_subdomains().replace(K_d=3, delta=0.05, max_steps=60),    # 6 rows in all, one CTA
+    P.small_tise_2d(L=2, K_d=16, q_p=16, n_mid=2, max_steps=60),            # K = 256, the largest
+    P.small_tise_2d(L=2, K_d=17, q_p=17, n_mid=2, max_steps=40),            # K = 289: the two-phase grid
+    P.small_tise_2d(L=2, K_d=7, q_p=6, n_mid=2, max_steps=60).replace(
+        K_d=[7, 3, 9, 6], delta=[1.3, 0.4, 1.7, 1.1]),                      # uneven rows per subdomain
+    P.tise_1d_two_subdomains().replace(L=12, K_d=33, delta=P.spacing_rule_delta((-10.0, 10.0), 12, 1.0, 33), q_p=24,
+                                       n_mid=1, max_steps=60),              # several subdomains in one CTA
+    P.tise_1d_two_subdomains().replace(normalize=False, kinetic=1.0, mu=1.0, n_steps=20, ngf_tol=0.0)],
+    ids=["tiny", "k256", "k289", "uneven", "12-subdomains", "no-normalisation"])
+def test_parity_fp64_window_on_chip_edges(swr_mod, inst):
+    _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE)
+
+
 def test_parity_classical_swr_imaginary_time(swr_mod):
     # classical SWR (Dirichlet data mu psi_j, imposed by penalty): FP64 and mixed
     inst = P.small_tise_2d().replace(tc="dirichlet", mu=50.0)
