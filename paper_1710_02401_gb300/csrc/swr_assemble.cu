@@ -14,7 +14,7 @@
 #include <math.h>
 #include <stdio.h>
 
-#include "swr_internal.cuh"
+#include "swr_fixed.cuh"
 
 namespace swr {
 
@@ -26,7 +26,7 @@ __device__ void gauss_legendre(int n, double* t, double* wt) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         // i-th root in decreasing order, initial guess of Tricomi type
         double x = cos(M_PI * (i + 0.75) / (n + 0.5));
-        double dp = 1.0;
+        double dp = 1.0, last = 1.0;
         for (int it = 0; it < 100; ++it) {
             double p0 = 1.0, p1 = x;
             for (int k = 2; k <= n; ++k) {
@@ -39,7 +39,8 @@ __device__ void gauss_legendre(int n, double* t, double* wt) {
             dp = n * (x * pn - pm) / (x * x - 1.0);
             double dx = pn / dp;
             x -= dx;
-            if (fabs(dx) < 1e-16) break;
+            if (last < 1e-8) break;  // quadratic convergence: this step was the last that changes x
+            last = fabs(dx);
         }
         // recompute derivative at the converged root
         double p0 = 1.0, p1 = x;
@@ -466,8 +467,15 @@ __global__ void k_ee_operands(SwrDeviceView v) {
     }
 }
 
-// Batched FP64 GEMM  C = op(A) * B  with 64x64 tiles.  One batch entry per
-// subdomain (blockIdx.z); its sizes and offsets come from a GemmJob.
+// Batched GEMM  C = op(A) * B  of FP64 matrices with 64x64 tiles, in 56-bit fixed
+// point on the integer pipes (swr_fixed.cuh: 4.5 multiply-adds per clock and SM
+// against 1.6 on the FP64 pipe).  Rows of op(A) are scaled by their largest
+// entry over the whole inner dimension with two bits kept free (sums of up to
+// 384 terms stay below 2^63), columns of B by theirs; the cross products are
+// folded every 64 terms.  One batch entry per subdomain (blockIdx.z); its sizes
+// and offsets come from a GemmJob.  2-electron workload (16 subdomains, q =
+// 132, kd = 24): 0.88 ms per product on the FP64 pipe, 0.35 here (integer
+// products and the conversion of every tile's operands bound it).
 
 #define GT 64
 #define GK 16
@@ -475,27 +483,55 @@ __global__ void __launch_bounds__(256) k_dgemm(SwrDeviceView v, const GemmJob* j
     const GemmJob jb = jobs[blockIdx.z];
     const int tm = blockIdx.y * GT, tn = blockIdx.x * GT;
     if (jb.M <= 0 || tm >= jb.M || tn >= jb.N) return;
-    __shared__ double As[GK][GT + 1];
-    __shared__ double Bs[GK][GT + 1];
+    __shared__ int2 As[GK][GT + 1];
+    __shared__ int2 Bs[GK][GT + 1];
+    __shared__ int ea[GT], eb[GT];
     const double* A = v.arena + jb.a;
     const double* B = v.arena + jb.b;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4] = {};
+    const int tid = threadIdx.x;
+    if (tid < GT) ea[tid] = eb[tid] = 0;
+    __syncthreads();
+    // exponents of the tile's rows and columns
+    if (jb.transA) {
+        const int mm = tid % GT;
+        int e = 0;
+        if (tm + mm < jb.M)
+            for (int k = tid / GT; k < jb.K; k += 256 / GT) e = max(e, fx_exp(A[(long long)k * jb.lda + tm + mm]));
+        atomicMax(&ea[mm], e + 2);
+    } else {
+        for (int mm = tid >> 5; mm < GT; mm += 8) {
+            int e = 0;
+            if (tm + mm < jb.M)
+                for (int k = tid & 31; k < jb.K; k += 32) e = max(e, fx_exp(A[(long long)(tm + mm) * jb.lda + k]));
+            e = __reduce_max_sync(0xffffffffu, e);
+            if ((tid & 31) == 0) ea[mm] = e + 2;
+        }
+    }
+    {
+        const int nn = tid % GT;
+        int e = 0;
+        if (tn + nn < jb.N)
+            for (int k = tid / GT; k < jb.K; k += 256 / GT) e = max(e, fx_exp(B[(long long)k * jb.ldb + tn + nn]));
+        atomicMax(&eb[nn], e);
+    }
+    __syncthreads();
+    const int tx = tid % 16, ty = tid / 16;
+    long long s1[4][4] = {}, s2[4][4] = {};
     for (int k0 = 0; k0 < jb.K; k0 += GK) {
-        for (int e = threadIdx.x; e < GK * GT; e += 256) {
-            int kk = e / GT, mm = e % GT;
-            int gk = k0 + kk, gm = tm + mm;
+        for (int e = tid; e < GK * GT; e += 256) {
+            const int kk = jb.transA ? e / GT : e % GK, mm = jb.transA ? e % GT : e / GK;
+            const int gk = k0 + kk, gm = tm + mm;
             double val = 0.0;
             if (gk < jb.K && gm < jb.M)
                 val = jb.transA ? A[(long long)gk * jb.lda + gm] : A[(long long)gm * jb.lda + gk];
-            As[kk][mm] = val;
-            int gn = tn + mm;
-            Bs[kk][mm] = (gk < jb.K && gn < jb.N) ? B[(long long)gk * jb.ldb + gn] : 0.0;
+            As[kk][mm] = fx_limbs(val, ea[mm]);
+            const int kb = e / GT, nn = e % GT, gn = tn + nn;
+            Bs[kb][nn] = fx_limbs((k0 + kb < jb.K && gn < jb.N) ? B[(long long)(k0 + kb) * jb.ldb + gn] : 0.0, eb[nn]);
         }
         __syncthreads();
-#pragma unroll
+#pragma unroll 4
         for (int kk = 0; kk < GK; ++kk) {
-            double ar[4], br[4];
+            int2 ar[4], br[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) ar[i] = As[kk][ty + 16 * i];
 #pragma unroll
@@ -503,8 +539,16 @@ __global__ void __launch_bounds__(256) k_dgemm(SwrDeviceView v, const GemmJob* j
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(ar[i], br[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) fx_mac2(s1[i][j], s2[i][j], ar[i].x, ar[i].y, br[j].x, br[j].y);
         }
+        if ((k0 / GK & 3) == 3)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    s1[i][j] = fx_fold(s1[i][j], s2[i][j]);
+                    s2[i][j] = 0;
+                }
         __syncthreads();
     }
     double* C = v.arena + jb.c;
@@ -514,14 +558,17 @@ __global__ void __launch_bounds__(256) k_dgemm(SwrDeviceView v, const GemmJob* j
         for (int j = 0; j < 4; ++j) {
             int gm = tm + ty + 16 * i, gn = tn + tx + 16 * j;
             if (gm >= jb.M || gn >= jb.N) continue;
+            const int xa = ea[ty + 16 * i], xb = eb[tx + 16 * j];
+            const double c = (xa >= FX_BAD || xb >= FX_BAD) ? nan("")
+                                                            : fx_double(fx_fold(s1[i][j], s2[i][j]), xa + xb - 2044 - 56);
             if (jb.mode == 0) {
-                C[(long long)gm * jb.ldc + gn] = acc[i][j];
+                C[(long long)gm * jb.ldc + gn] = c;
             } else {
                 // gm = (a,c) = a*kd + c, gn = (b,d) = b*kd + e; H'[(a + kd b), (c + kd e)]
                 int kd = jb.kd;
-                int a = gm / kd, c = gm % kd, b = gn / kd, e = gn % kd;
+                int a = gm / kd, cc = gm % kd, b = gn / kd, e = gn % kd;
                 long long K = (long long)kd * kd;
-                C[(long long)(a + kd * b) * K + (c + kd * e)] = acc[i][j];
+                C[(long long)(a + kd * b) * K + (cc + kd * e)] = c;
             }
         }
 }
@@ -620,11 +667,6 @@ template <> __device__ inline cplx ld_el<cplx>(const double* p, long long i) { r
 template <typename T> __device__ inline void st_el(double* p, long long i, T x);
 template <> __device__ inline void st_el<double>(double* p, long long i, double x) { p[i] = x; }
 template <> __device__ inline void st_el<cplx>(double* p, long long i, cplx x) { p[2 * i] = x.re; p[2 * i + 1] = x.im; }
-__device__ inline double inv_el(double x) { return 1.0 / x; }
-__device__ inline cplx inv_el(cplx x) {
-    double d = x.re * x.re + x.im * x.im;
-    return mkc(x.re / d, -x.im / d);
-}
 __device__ inline double mag2(double x) { return x * x; }
 __device__ inline double mag2(cplx x) { return x.re * x.re + x.im * x.im; }
 __device__ inline double neg(double x) { return -x; }
@@ -635,133 +677,295 @@ __device__ inline double one_el(double) { return 1.0; }
 __device__ inline cplx one_el(cplx) { return mkc(1.0, 0.0); }
 
 #define GJ_NB 32
+#define GJ_T 64   // columns of the row-block kernel, tile edge of the real update
+// 1/x by two Newton steps from the FP32 reciprocal (264 clocks on the FP64 pipe
+// instead of 550 for the division); the division where FP32 does not reach.
+__device__ inline double gj_rcp(double x) {
+    const double ax = fabs(x);
+    if (!(ax > 1e-30 && ax < 1e30)) return 1.0 / x;
+    double r = (double)(1.0f / (float)x);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+__device__ inline double gj_inv(double x) { return gj_rcp(x); }
+__device__ inline cplx gj_inv(cplx x) {
+    const double d = gj_rcp(x.re * x.re + x.im * x.im);
+    return mkc(x.re * d, -x.im * d);
+}
+__device__ inline double gj_fnma(double a, double b, double c) { return fma(-a, b, c); }
+__device__ inline cplx gj_fnma(cplx a, cplx b, cplx c) { return c - a * b; }
+
 // Scratch per subdomain (elements of T): Pinv [NB][NB], Rp [NB][K], Cp [K][NB].
+// Inverse of the diagonal block kb of every subdomain (one CTA each; no
+// pivoting: the step matrices have a positive definite Hermitian part).  A
+// serial chain of nb pivots: each thread keeps one column of four rows, three
+// barriers and one reciprocal per pivot.  K = 576, 16 subdomains: 37 us per
+// block column (276 us when one CTA also formed Pinv M[kb, :] in FP64); complex
+// with several hundred subdomains it is the FP64 pipe (184 us).
 template <typename T>
-__global__ void k_gj_panel(SwrDeviceView v, int kb) {
-    const int sid = blockIdx.x;
-    const SubDev& s = v.sub[sid];
+__global__ void __launch_bounds__(256) k_gj_panel(SwrDeviceView v, int kb) {
+    const SubDev& s = v.sub[blockIdx.x];
     const int K = s.K, k0 = kb * GJ_NB;
     if (k0 >= K) return;
-    const int nb = min(GJ_NB, K - k0);
+    const int nb = min(GJ_NB, K - k0), j = threadIdx.x & 31, w = threadIdx.x >> 5;
     double* M = v.arena + s.Gm;
-    double* W = v.arena + s.work;
-    __shared__ T P[GJ_NB][GJ_NB + 1];
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int i = e / nb, j = e % nb;
-        P[i][j] = ld_el<T>(M, (long long)(k0 + i) * K + k0 + j);
+    double* Pinv = v.arena + s.work;
+    __shared__ T rowp[GJ_NB], colp[GJ_NB], s_pinv;
+    T a[4];  // rows w, w + 8, w + 16, w + 24 of column j
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = w + 8 * u;
+        a[u] = i < nb && j < nb ? ld_el<T>(M, (long long)(k0 + i) * K + k0 + j) : (i == j ? one_el(T()) : zero_el(T()));
     }
-    __syncthreads();
-    // unblocked in-place Gauss-Jordan inversion of the nb x nb block (no pivoting:
-    // the step matrices have a positive definite Hermitian part)
-    __shared__ int s_bad;
-    if (threadIdx.x == 0) s_bad = 0;
-    __syncthreads();
+    bool bad = false;
     for (int p = 0; p < nb; ++p) {
-        __shared__ T piv_inv;
-        if (threadIdx.x == 0) {
-            T pv = P[p][p];
-            double m = mag2(pv);
-            if (!(m > 1e-280) || !isfinite(m)) { s_bad = 1; pv = one_el(T()); }
-            piv_inv = inv_el(pv);
+        if (j == p)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) colp[w + 8 * u] = a[u];
+        __syncthreads();
+        if (w == (p & 7)) {  // the pivot row's warp
+            T pv = colp[p];
+            const double m = mag2(pv);
+            if (!(m > 1e-280) || !isfinite(m)) {
+                bad = true;
+                pv = one_el(T());
+            }
+            const T pi = gj_inv(pv);
+            const int up = p >> 3;
+            const T old = up == 0 ? a[0] : up == 1 ? a[1] : up == 2 ? a[2] : a[3];
+            const T scaled = j == p ? pi : pi * old;
+            if (up == 0) a[0] = scaled;
+            if (up == 1) a[1] = scaled;
+            if (up == 2) a[2] = scaled;
+            if (up == 3) a[3] = scaled;
+            rowp[j] = scaled;
+            if (j == 0) s_pinv = pi;
         }
         __syncthreads();
-        T pinv = piv_inv;
-        // column p of the other rows, saved before the update
-        __shared__ T colp[GJ_NB];
-        for (int i = threadIdx.x; i < nb; i += blockDim.x) colp[i] = P[i][p];
-        __syncthreads();
-        // row p scaled
-        for (int j = threadIdx.x; j < nb; j += blockDim.x) P[p][j] = (j == p) ? pinv : pinv * P[p][j];
-        __syncthreads();
-        for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-            int i = e / nb, j = e % nb;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = w + 8 * u;
             if (i == p) continue;
-            if (j == p) P[i][j] = neg(colp[i] * pinv);
-            else P[i][j] = P[i][j] - colp[i] * P[p][j];
+            a[u] = j == p ? neg(colp[i] * s_pinv) : gj_fnma(colp[i], rowp[j], a[u]);
         }
         __syncthreads();
     }
-    if (s_bad && threadIdx.x == 0) atomicOr(v.err, SWR_ERR_SINGULAR);
-    // scratch
-    double* Pinv = W;
-    double* Rp = W + (sizeof(T) / 8) * GJ_NB * GJ_NB;
-    double* Cp = Rp + (sizeof(T) / 8) * (long long)GJ_NB * K;
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) st_el<T>(Pinv, e / nb * GJ_NB + e % nb, P[e / nb][e % nb]);
-    // Rp = Pinv * M[kb, :]   (nb x K)
-    for (long long e = threadIdx.x; e < (long long)nb * K; e += blockDim.x) {
-        int i = (int)(e / K), j = (int)(e % K);
-        T acc = zero_el(T());
-        for (int t = 0; t < nb; ++t) acc = acc + P[i][t] * ld_el<T>(M, (long long)(k0 + t) * K + j);
-        st_el<T>(Rp, (long long)i * K + j, acc);
-    }
-    // Cp = M[:, kb]   (K x nb)
-    for (long long e = threadIdx.x; e < (long long)K * nb; e += blockDim.x) {
-        int i = (int)(e / nb), j = (int)(e % nb);
-        st_el<T>(Cp, (long long)i * GJ_NB + j, ld_el<T>(M, (long long)i * K + k0 + j));
+    if (bad) atomicOr(v.err, SWR_ERR_SINGULAR);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = w + 8 * u;
+        if (i < nb && j < nb) st_el<T>(Pinv, i * GJ_NB + j, a[u]);
     }
 }
 
-// Rank-nb update of the whole matrix for block column kb (TILE x TILE tiles:
-// 64 for real, 32 for complex so that the staged panels stay under 48 KB).
+// Components of an element as reals.
+template <typename T> struct GjParts { static const int v = 1; };
+template <> struct GjParts<cplx> { static const int v = 2; };
+__device__ inline double gj_part(double x, int) { return x; }
+__device__ inline double gj_part(cplx x, int p) { return p ? x.im : x.re; }
+__device__ inline int gj_exp(double x) { return fx_exp(x); }
+__device__ inline int gj_exp(cplx x) { return max(fx_exp(x.re), fx_exp(x.im)); }
+__device__ inline double gj_make(const double* x, double) { return x[0]; }
+__device__ inline cplx gj_make(const double* x, cplx) { return mkc(x[0], x[1]); }
+
+// Product of a GA x 32 block (rows scaled by ea) and a 32 x GB one (columns by
+// eb), limbs in shared memory, in fixed point (swr_fixed.cuh): thread (ty, tx)
+// of 16 x 16 gets rows ty + 16 i, columns tx + 16 j.  Both the row block Pinv M[kb, :]
+// and the rank-32 update are this product; in FP64 they filled the FP64 pipe
+// (1.6 multiply-adds per clock and SM, 4.5 here).
+template <typename T, int GA, int GB>
+__device__ inline void gj_product(const int2 (*A)[GA][GJ_NB + 1], const int2 (*B)[GJ_NB][GB + 1], const int* ea, const int* eb,
+                                  int tx, int ty, T (&out)[GA / 16][GB / 16]) {
+    constexpr int P = GjParts<T>::v;
+    long long s1[P][GA / 16][GB / 16] = {}, s2[P][GA / 16][GB / 16] = {};
+#pragma unroll 2
+    for (int t = 0; t < GJ_NB; ++t) {
+        int2 ar[P][GA / 16], br[P][GB / 16];
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+#pragma unroll
+            for (int i = 0; i < GA / 16; ++i) ar[p][i] = A[p][ty + 16 * i][t];
+#pragma unroll
+            for (int j = 0; j < GB / 16; ++j) br[p][j] = B[p][t][tx + 16 * j];
+        }
+#pragma unroll
+        for (int i = 0; i < GA / 16; ++i)
+#pragma unroll
+            for (int j = 0; j < GB / 16; ++j) {
+                fx_mac2(s1[0][i][j], s2[0][i][j], ar[0][i].x, ar[0][i].y, br[0][j].x, br[0][j].y);
+                if (P == 2) {
+                    fx_mac2(s1[0][i][j], s2[0][i][j], -ar[P - 1][i].x, -ar[P - 1][i].y, br[P - 1][j].x, br[P - 1][j].y);
+                    fx_mac2(s1[P - 1][i][j], s2[P - 1][i][j], ar[0][i].x, ar[0][i].y, br[P - 1][j].x, br[P - 1][j].y);
+                    fx_mac2(s1[P - 1][i][j], s2[P - 1][i][j], ar[P - 1][i].x, ar[P - 1][i].y, br[0][j].x, br[0][j].y);
+                }
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < GA / 16; ++i)
+#pragma unroll
+        for (int j = 0; j < GB / 16; ++j) {
+            const int xa = ea[ty + 16 * i], xb = eb[tx + 16 * j];
+            double x[2] = {0.0, 0.0};
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                x[p] = (xa == FX_BAD || xb == FX_BAD) ? nan("") : fx_double(fx_fold(s1[p][i][j], s2[p][i][j]), xa + xb - 2044 - 56);
+            out[i][j] = gj_make(x, T());
+        }
+}
+
+// Columns [tn, tn + GJ_T) of the pivot row block: Rp = Pinv M[kb, :], and the pivot
+// column block Cp = M[:, kb] of the same index range, by GJ_T columns per CTA
+// (one CTA doing all of it took 180 us of a 276 us panel at K = 576, 16 us here).
+template <typename T>
+__global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
+    constexpr int P = GjParts<T>::v;
+    const SubDev& s = v.sub[blockIdx.y];
+    const int K = s.K, k0 = kb * GJ_NB, tn = blockIdx.x * GJ_T;
+    if (k0 >= K || tn >= K) return;
+    const int nb = min(GJ_NB, K - k0), tid = threadIdx.x;
+    const double* M = v.arena + s.Gm;
+    double* Pinv = v.arena + s.work;
+    double* Rp = Pinv + P * GJ_NB * GJ_NB;
+    double* Cp = Rp + P * (long long)GJ_NB * K;
+    extern __shared__ int2 gj_sm[];
+    int2(*A)[GJ_NB][GJ_NB + 1] = reinterpret_cast<int2(*)[GJ_NB][GJ_NB + 1]>(gj_sm);
+    int2(*B)[GJ_NB][GJ_T + 1] = reinterpret_cast<int2(*)[GJ_NB][GJ_T + 1]>(gj_sm + P * GJ_NB * (GJ_NB + 1));
+    __shared__ int ea[GJ_NB], eb[GJ_T];
+    if (tid < GJ_T) eb[tid] = 0;
+    __syncthreads();
+    T pa[4], mb[8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int e = tid + 256 * u, i = e / GJ_NB, t = e % GJ_NB;
+        pa[u] = i < nb && t < nb ? ld_el<T>(Pinv, i * GJ_NB + t) : zero_el(T());
+        const int x = __reduce_max_sync(0xffffffffu, gj_exp(pa[u]));  // a warp holds one row
+        if (t == 0) ea[i] = x;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int e = tid + 256 * u, t = e / GJ_T, j = e % GJ_T;
+        mb[u] = t < nb && tn + j < K ? ld_el<T>(M, (long long)(k0 + t) * K + tn + j) : zero_el(T());
+        atomicMax(&eb[j], gj_exp(mb[u]));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = tid + 256 * u, i = e / GJ_NB, t = e % GJ_NB;
+            A[p][i][t] = fx_limbs(gj_part(pa[u], p), ea[i]);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int e = tid + 256 * u, t = e / GJ_T, j = e % GJ_T;
+            B[p][t][j] = fx_limbs(gj_part(mb[u], p), eb[j]);
+        }
+    }
+    __syncthreads();
+    const int tx = tid % 16, ty = tid / 16;
+    T out[2][4];
+    gj_product<T, GJ_NB, GJ_T>(A, B, ea, eb, tx, ty, out);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = ty + 16 * i, c = tn + tx + 16 * j;
+            if (r < nb && c < K) st_el<T>(Rp, (long long)r * K + c, out[i][j]);
+        }
+    for (int e = tid; e < GJ_T * nb; e += 256) {
+        const int i = tn + e / nb, t = e % nb;
+        if (i < K) st_el<T>(Cp, (long long)i * GJ_NB + t, ld_el<T>(M, (long long)i * K + k0 + t));
+    }
+}
+
+// Rank-nb update of the whole matrix for block column kb (TILE x TILE tiles: 64 for
+// real, 32 for complex data: larger ones spill).  K = 576, 16 subdomains: 321 us
+// per block column in FP64, 131 here, bound by the integer products (4.5
+// multiply-adds per clock and SM).
 template <typename T> struct GjTile { static const int v = 64; };
 template <> struct GjTile<cplx> { static const int v = 32; };
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb) {
-    constexpr int TL = GjTile<T>::v;
-    const int sid = blockIdx.z;
-    const SubDev& s = v.sub[sid];
+    constexpr int TL = GjTile<T>::v, P = GjParts<T>::v, N = TL * GJ_NB / 256, Q = TL / 16;
+    const SubDev& s = v.sub[blockIdx.z];
     const int K = s.K, k0 = kb * GJ_NB;
     if (k0 >= K) return;
     const int tm = blockIdx.y * TL, tn = blockIdx.x * TL;
     if (tm >= K || tn >= K) return;
-    const int nb = min(GJ_NB, K - k0);
+    const int nb = min(GJ_NB, K - k0), tid = threadIdx.x;
     double* M = v.arena + s.Gm;
-    const double* W = v.arena + s.work;
-    const double* Pinv = W;
-    const double* Rp = W + (sizeof(T) / 8) * GJ_NB * GJ_NB;
-    const double* Cp = Rp + (sizeof(T) / 8) * (long long)GJ_NB * K;
-    __shared__ T Cs[TL][GJ_NB + 1];
-    __shared__ T Rs[GJ_NB][TL + 1];
-    for (int e = threadIdx.x; e < TL * GJ_NB; e += 256) {
-        int i = e / GJ_NB, t = e % GJ_NB;
-        int gi = tm + i;
-        Cs[i][t] = (gi < K && t < nb) ? ld_el<T>(Cp, (long long)gi * GJ_NB + t) : zero_el(T());
-    }
-    for (int e = threadIdx.x; e < GJ_NB * TL; e += 256) {
-        int t = e / TL, j = e % TL;
-        int gj = tn + j;
-        T r = zero_el(T());
-        if (gj < K && t < nb) {
-            if (gj >= k0 && gj < k0 + nb) r = ld_el<T>(Pinv, (long long)t * GJ_NB + (gj - k0));
-            else r = ld_el<T>(Rp, (long long)t * K + gj);
-        }
-        Rs[t][j] = r;
+    const double* Pinv = v.arena + s.work;
+    const double* Rp = Pinv + P * GJ_NB * GJ_NB;
+    const double* Cp = Rp + P * (long long)GJ_NB * K;
+    extern __shared__ int2 gj_sm[];
+    int2(*A)[TL][GJ_NB + 1] = reinterpret_cast<int2(*)[TL][GJ_NB + 1]>(gj_sm);
+    int2(*B)[GJ_NB][TL + 1] = reinterpret_cast<int2(*)[GJ_NB][TL + 1]>(gj_sm + P * TL * (GJ_NB + 1));
+    __shared__ int ea[TL], eb[TL];
+    if (tid < TL) eb[tid] = 0;
+    __syncthreads();
+    T ca[N], rb[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const int e = tid + 256 * u, i = e / GJ_NB, t = e % GJ_NB;
+        ca[u] = tm + i < K && t < nb ? ld_el<T>(Cp, (long long)(tm + i) * GJ_NB + t) : zero_el(T());
+        const int x = __reduce_max_sync(0xffffffffu, gj_exp(ca[u]));  // a warp holds one row
+        if (t == 0) ea[i] = x;
+        const int t2 = e / TL, j = e % TL, gj = tn + j;
+        rb[u] = zero_el(T());
+        if (gj < K && t2 < nb)
+            rb[u] = gj >= k0 && gj < k0 + nb ? ld_el<T>(Pinv, t2 * GJ_NB + (gj - k0)) : ld_el<T>(Rp, (long long)t2 * K + gj);
+        atomicMax(&eb[j], gj_exp(rb[u]));
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < TL * TL; e += 256) {
-        int i = e / TL, j = e % TL;
-        int gi = tm + i, gj = tn + j;
-        if (gi >= K || gj >= K) continue;
-        bool ri = gi >= k0 && gi < k0 + nb, cj = gj >= k0 && gj < k0 + nb;
-        long long idx = (long long)gi * K + gj;
-        if (ri) {
-            st_el<T>(M, idx, Rs[gi - k0][j]);     // row block: Pinv * M[kb,:] (Pinv on the diagonal block)
-        } else {
-            T acc = zero_el(T());
-#pragma unroll 8
-            for (int t = 0; t < GJ_NB; ++t) acc = acc + Cs[i][t] * Rs[t][j];
-            if (cj) st_el<T>(M, idx, neg(acc));            // -C * Pinv
-            else st_el<T>(M, idx, ld_el<T>(M, idx) - acc); // M - C * R
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            const int e = tid + 256 * u;
+            A[p][e / GJ_NB][e % GJ_NB] = fx_limbs(gj_part(ca[u], p), ea[e / GJ_NB]);
+            B[p][e / TL][e % TL] = fx_limbs(gj_part(rb[u], p), eb[e % TL]);
         }
-    }
+    __syncthreads();
+    const int tx = tid % 16, ty = tid / 16;
+    T out[Q][Q];
+    gj_product<T, TL, TL>(A, B, ea, eb, tx, ty, out);
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            const int gi = tm + ty + 16 * i, gj = tn + tx + 16 * j;
+            if (gi >= K || gj >= K) continue;
+            const bool ri = gi >= k0 && gi < k0 + nb, cj = gj >= k0 && gj < k0 + nb;
+            const long long idx = (long long)gi * K + gj;
+            if (ri)  // row block: Pinv M[kb, :] (Pinv on the diagonal block)
+                st_el<T>(M, idx, cj ? ld_el<T>(Pinv, (gi - k0) * GJ_NB + (gj - k0)) : ld_el<T>(Rp, (long long)(gi - k0) * K + gj));
+            else if (cj) st_el<T>(M, idx, neg(out[i][j]));                   // -C Pinv
+            else st_el<T>(M, idx, ld_el<T>(M, idx) - out[i][j]);             // M - C R
+        }
+}
+
+template <typename T>
+static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int max_K, bool update) {
+    constexpr int TL = GjTile<T>::v, P = GjParts<T>::v;
+    const size_t sr = P * (GJ_NB * (GJ_NB + 1) + GJ_NB * (GJ_T + 1)) * sizeof(int2);
+    const size_t su = P * (TL * (GJ_NB + 1) + GJ_NB * (TL + 1)) * sizeof(int2);
+    cudaError_t e = cudaFuncSetAttribute(k_gj_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gj_update<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)su);
+    if (e != cudaSuccess) return e;
+    k_gj_panel<T><<<v.n_sub, 256, 0, st>>>(v, kb);
+    k_gj_rows<T><<<dim3((max_K + GJ_T - 1) / GJ_T, v.n_sub), 256, sr, st>>>(v, kb);
+    if (update) k_gj_update<T><<<dim3((max_K + TL - 1) / TL, (max_K + TL - 1) / TL, v.n_sub), 256, su, st>>>(v, kb);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ initial data
 
 // c0 = (B'1^T W f1) (x) (B'2^T W f2) for phi0 = prod_e exp(-gamma (x_e - x0_e)^2)
 // (projection of Sec. 6.1 in the orthonormal basis: c' = X^T c~).
-// out[sid] = partial PoU norm^2 of c0 (later summed per instance).
+// out[sid] = partial PoU norm^2 of c0 (later summed per instance).  The node values
+// are formed once per coordinate and a warp sums one coefficient (one thread per
+// coefficient, with its own exponentials: 430 us at kd = 24, q = 132; 23 here).
 __global__ void k_project(SwrDeviceView v, double* norm_part) {
     const int sid = blockIdx.x;
     const SubDev& s = v.sub[sid];
@@ -770,22 +974,34 @@ __global__ void k_project(SwrDeviceView v, double* norm_part) {
     T1Layout lay(q, kd);
     __shared__ double u[2][ORTH_MAX_KD * 4];
     __shared__ double nrm[2];
+    __shared__ double f[384];               // w exp(-gamma (x - x0)^2) at the nodes (q <= 384)
+    __shared__ double pu[ORTH_MAX_KD];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int d = 0; d < s.N; ++d) {
         const double* T = v.arena + s.t1[d];
-        for (int a = threadIdx.x; a < kd; a += blockDim.x) {
-            double acc = 0;
-            for (int n = 0; n < q; ++n) {
-                double r = T[lay.x() + n] - in.x0[d];
-                acc += T[lay.w() + n] * exp(-in.gamma0 * r * r) * T[lay.B() + n * kd + a];
-            }
-            u[d][a] = acc;
+        for (int n = threadIdx.x; n < q; n += blockDim.x) {
+            const double r = T[lay.x() + n] - in.x0[d];
+            f[n] = T[lay.w() + n] * exp(-in.gamma0 * r * r);
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
+        for (int a = warp; a < kd; a += nw) {
             double acc = 0;
-            for (int a = 0; a < kd; ++a)
-                for (int c = 0; c < kd; ++c) acc += u[d][a] * T[lay.mat(M_PP) + a * kd + c] * u[d][c];
-            nrm[d] = acc;
+            for (int n = lane; n < q; n += 32) acc += f[n] * T[lay.B() + n * kd + a];
+            acc = warp_sum(acc);
+            if (lane == 0) u[d][a] = acc;
+        }
+        __syncthreads();
+        for (int a = threadIdx.x; a < kd; a += blockDim.x) {
+            double acc = 0;
+            for (int c = 0; c < kd; ++c) acc += T[lay.mat(M_PP) + a * kd + c] * u[d][c];
+            pu[a] = u[d][a] * acc;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            double acc = 0;
+            for (int a = lane; a < kd; a += 32) acc += pu[a];
+            acc = warp_sum(acc);
+            if (lane == 0) nrm[d] = acc;
         }
         __syncthreads();
     }
@@ -875,7 +1091,7 @@ __global__ void k_normalize_c0(SwrDeviceView v, const double* norm_part) {
 static inline unsigned div_up(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
 // Launches of an assembly besides the e-e block (3) and the Gauss-Jordan
-// panels/updates (2 per block column): tabulate, mat1d, orth, h_kron,
+// panels, row blocks and updates (3 per block column): tabulate, mat1d, orth, h_kron,
 // symmetrize, step_matrix, project, anti_c0, normalize_c0.
 extern const int kAssembleLaunchesFixed = 9;
 
@@ -915,25 +1131,9 @@ cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, 
     k_step_matrix<<<ge, 256, 0, st>>>(v);
     int nkb = (max_K + GJ_NB - 1) / GJ_NB;
     for (int kb = 0; kb < nkb; ++kb) {
-        if (any_tdse) {
-            dim3 gu(div_up(max_K, 32), div_up(max_K, 32), v.n_sub);
-            k_gj_panel<cplx><<<v.n_sub, 256, 0, st>>>(v, kb);
-            if (tg) {
-                cudaError_t e = tg_update(tg, v, st, kb, max_K);
-                if (e != cudaSuccess) return e;
-            } else {
-                k_gj_update<cplx><<<gu, 256, 0, st>>>(v, kb);
-            }
-        } else {
-            dim3 gu(div_up(max_K, 64), div_up(max_K, 64), v.n_sub);
-            k_gj_panel<double><<<v.n_sub, 256, 0, st>>>(v, kb);
-            if (tg) {
-                cudaError_t e = tg_update(tg, v, st, kb, max_K);
-                if (e != cudaSuccess) return e;
-            } else {
-                k_gj_update<double><<<gu, 256, 0, st>>>(v, kb);
-            }
-        }
+        cudaError_t e = any_tdse ? gj_block<cplx>(v, st, kb, max_K, !tg) : gj_block<double>(v, st, kb, max_K, !tg);
+        if (e == cudaSuccess && tg) e = tg_update(tg, v, st, kb, max_K);
+        if (e != cudaSuccess) return e;
     }
     k_project<<<v.n_sub, 256, 0, st>>>(v, d_norm_part);
     k_anti_c0<<<v.n_sub, 256, 0, st>>>(v, d_norm_part);

@@ -51,6 +51,20 @@ __device__ inline double fx_unit(int emax, int eg) {
     const int e = emax - 55 + eg;  // biased
     return e > 0 && e < 0x7ff ? __hiloint2double(e << 20, 0) : 0.0;
 }
+// s 2^e, rounded to nearest, without the FP64 pipe (0 below the normal range,
+// NaN for exponents of non-finite operands).
+__device__ inline double fx_double(long long s, int e) {
+    if (s == 0) return 0.0;
+    unsigned long long m = s < 0 ? 0ULL - (unsigned long long)s : (unsigned long long)s;
+    const int z = __clzll((long long)m);
+    m <<= z;                                   // leading bit 63
+    m = (m >> 11) + ((m >> 10) & 1ULL);        // 53 bits, the next one rounds
+    const int be = 1023 + 63 - z + e;          // biased exponent of bit 52 of m
+    if (be <= 0) return 0.0;
+    if (be >= 0x7fe) return __longlong_as_double(0x7ff8000000000000LL);
+    const unsigned long long u = ((unsigned long long)(be - 1) << 52) + m;  // (a carry out of the rounding raises be)
+    return __longlong_as_double((long long)(u | (s < 0 ? 0x8000000000000000ULL : 0ULL)));
+}
 __device__ inline long long fx_fold(long long s1, long long s2) { return s1 + ((s2 + (1LL << (FX_BITS - 1))) >> FX_BITS); }
 __device__ inline void fx_mac(long long& s, int a, int b) { s += (long long)a * b; }
 // (s1, s2) += a b for limb pairs.

@@ -310,6 +310,26 @@ def test_parity_fp64_window_on_chip_edges(swr_mod, inst):
     _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE)
 
 
+@pytest.mark.parametrize("mode", [P.TISE, P.TDSE])
+@pytest.mark.parametrize("K_d", [31, 32, 33, 63, 65])
+def test_parity_step_matrix_inverse_at_block_edges(swr_mod, K_d, mode):
+    # one pivot block, one exactly, one row past it; one row short of and past a
+    # tile of the update (64 real, 32 complex)
+    inst = P.tise_1d_two_subdomains().replace(K_d=K_d, delta=P.spacing_rule_delta((-10.0, 10.0), 2, 1.0, K_d), q_p=24,
+                                              n_steps=9, ngf_tol=0.0)
+    if mode == P.TDSE:
+        inst = inst.replace(mode=mode, mu=-10j, dt=0.01, field=(0.5, 0.09, 8.0, 0.3))
+    _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE, window_variant=0 if mode == P.TDSE else 1)
+
+
+@pytest.mark.parametrize("K_d,q_p,n_mid", [(3, 5, 1), (8, 16, 2), (9, 13, 3), (16, 64, 4)])
+def test_parity_electron_repulsion_at_tile_edges(swr_mod, K_d, q_p, n_mid):
+    # q and K_d^2 on, under and past the 64 x 64 tiles and the folds every 64
+    # terms, and the largest quadrature (384 nodes)
+    _compare(swr_mod, P.small_tise_2d(L=2, K_d=K_d, q_p=q_p, n_mid=n_mid, max_steps=20), kmax=2,
+             rel_robin=REL_ROBIN_PROJECTED_EDGE, window_variant=1)
+
+
 def test_parity_classical_swr_imaginary_time(swr_mod):
     # classical SWR (Dirichlet data mu psi_j, imposed by penalty): FP64 and mixed
     inst = P.small_tise_2d().replace(tc="dirichlet", mu=50.0)
