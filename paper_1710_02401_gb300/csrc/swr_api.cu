@@ -34,6 +34,7 @@ int window_tasks_per_cta_max();
 int window_rows_per_task_max();
 cudaError_t window_occupancy(int* blocks_per_sm, size_t smem, int variant, bool df32);
 cudaError_t launch_split_df32(const SwrDeviceView& v, cudaStream_t st, int max_K, bool make_w);
+cudaError_t launch_fx_rows(const SwrDeviceView& v, cudaStream_t st, int max_K);
 cudaError_t launch_window(SweepArgs& a, int grid, size_t smem, cudaStream_t st, int n_inst, int variant, bool df32,
                           bool onep, cudaEvent_t ev_begin, cudaEvent_t ev_end);
 extern const int kAssembleLaunchesFixed, kStepLaunches;
@@ -1142,6 +1143,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     else if (c->tdse) CU(launch_split_c_df32(view(c), c->stream, c->max_K));
     if (c->robin_w) CU(launch_robin_ge(view(c), c->stream, c->max_K, c->max_J));
     if (c->oc) CU(launch_oc_make_w(view(c), c->stream, c->max_K));
+    else if (!c->df32 && !c->tdse) CU(launch_fx_rows(view(c), c->stream, c->max_K));
     CU(cudaEventRecord(c->ev1, c->stream));
     swr_status st = check_err(c);
     if (st != SWR_OK) return st;
@@ -1150,7 +1152,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     c->counters[6] += ams;
     c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 3) : 0) +
                       (c->tg ? 5 : 3) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
-                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (c->oc ? 1 : 0);
+                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (!c->df32 && !c->tdse ? 1 : 0);
     c->assembled = true;
     c->k = 0;
     c->parity = 0;
@@ -1452,7 +1454,9 @@ extern "C" swr_status swr_autotune(swr_ctx* c, int steps, swr_tune_report* out) 
     cands.push_back({c->prob.window_variant, c->prob.rows_per_task});  // the plan before tuning
     const int rows_list[] = {0, 16, 32, 64, 128, 256};
     const int variants[] = {WIN_TWO_PHASE, WIN_FUSED, WIN_SPLIT, WIN_RESIDENT, WIN_CLUSTER};
+    // (on chip, H' holds W instead of the grid windows' rows: the plan stays)
     for (int v : variants) {
+        if (c->oc) break;
         if (v == WIN_FUSED && !(c->df32 && c->has_w)) continue;
         if ((v == WIN_SPLIT || v == WIN_RESIDENT || v == WIN_CLUSTER) && !c->df32) continue;
         if (v == WIN_CLUSTER && (c->any_anti || !c->robin_w)) continue;

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_window_onchip(OcArgs A) {
     __shared__ __align__(16) double2 s_slot[2][OC_CMAX];  // partials of s_n^2 and D_{n-1} by step parity and CTA
     __shared__ int s_emax[2][OC_SUBS];                    // exponent of v per subdomain here, by step parity
     __shared__ int s_base[OC_CMAX], s_bound[OC_CMAX + 1]; // first row of y kept by each CTA; its first own row
-    __shared__ int s_sub0[OC_SUBS + 1], s_voff[OC_SUBS];  // per subdomain here: first row, offset of its limbs
+    __shared__ int s_sub0[OC_SUBS + 1];  // per subdomain here: first row
     __shared__ double s_is[2];                            // 1/s_n, 1/s_{n-1}
     __shared__ int s_stop;
     const SwrDeviceView& v = A.v;

@@ -23,14 +23,15 @@
 // Every wait is bounded; on timeout the kernel raises SWR_ERR_TIMEOUT and
 // returns.
 //
-// Precision: FP64 (DFMA), or double-single (SWR_PREC_MIXED): G = G_hi + G_lo
+// Precision: FP64 (the products in 56-bit fixed point, swr_fixed.cuh: 4.5
+// multiply-adds per clock and SM against 1.6 on the FP64 pipe), or double-single (SWR_PREC_MIXED): G = G_hi + G_lo
 // in FP32 pairs, v = v_hi + v_lo; products run on the FP32 pipes with
 // error-free TwoProduct/TwoSum accumulation into a (hi, lo) pair, which keeps
 // the FP64 accuracy of the step (~1e-14) on units with 64x the FP64 rate.
 #include <limits.h>
 #include <math.h>
 
-#include "swr_internal.cuh"
+#include "swr_fixed.cuh"
 
 namespace swr {
 
@@ -336,7 +337,7 @@ __device__ inline void prefetch_rows(const SwrDeviceView& v, const TaskCache& tc
         prefetch_l2(Gh + rb * ld, (size_t)nrow * ld * sizeof(float));
         prefetch_l2(Gh + (long long)tc.K * ld + rb * ld, (size_t)nrow * ld * sizeof(float));
     } else {
-        prefetch_l2(v.arena + tc.Gm + (long long)rb * tc.K, (size_t)nrow * tc.K * sizeof(double));
+        prefetch_l2(v.arena + v.sub[tc.sid].Hm + (long long)rb * tc.K, (size_t)nrow * tc.K * sizeof(int2));
     }
 }
 
@@ -387,35 +388,77 @@ __device__ inline void df32_rows4(const float* Gh, const float* Gl, int ld, cons
     }
 }
 
-// Rows [rb, rb + nrow), nrow <= 4, of G v in FP64: per row two accumulators
-// over columns c = lane + 64 m and c = lane + 32 + 64 m, then a shuffle sum
-// (the same order for every row whatever warp computes it); y[i] to all lanes.
-__device__ inline void fp64_rows4(const double* G, int K, const double* vs, int rb, int nrow, int lane, double* y) {
-    double a[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0};
-    int c = lane;
-    for (; c + 32 < K; c += 64) {
-        const double x0 = vs[c], x1 = vs[c + 32];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (i < nrow) {
-                const double* g = G + (long long)(rb + i) * K;
-                a[i] = fma(g[c], x0, a[i]);
-                b[i] = fma(g[c + 32], x1, b[i]);
-            }
+// Limbs of the FP64 step-matrix inverse into the space of H' (not needed after
+// the inversion), every row scaled by a power of two above its 2-norm, whose
+// exponent goes to the assembly's scratch: the two-phase FP64 window reads 8
+// bytes per element as before.  With rows and columns of norm at most 2^28 the
+// sums stay below 2^61 for K <= 1024.
+__global__ void k_fx_rows(SwrDeviceView v) {
+    const SubDev& s = v.sub[blockIdx.y];
+    const int K = s.K, lane = threadIdx.x & 31;
+    int2* L = reinterpret_cast<int2*>(v.arena + s.Hm);
+    int* ex = reinterpret_cast<int*>(v.arena + s.work);
+    for (int r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); r < K; r += gridDim.x * (blockDim.x / 32)) {
+        const double* g = v.arena + s.Gm + (long long)r * K;
+        int e = 0;
+        for (int c = lane; c < K; c += 32) e = max(e, fx_exp(g[c]));
+        e = __reduce_max_sync(0xffffffffu, e);
+        // the 2-norm over the largest entry: 2^(e - 1022) <= norm bound < 2^(e - 1022 + x)
+        const double sc = e > 0 && e < 2046 ? __hiloint2double((2045 - e) << 20, 0) : 0.0;
+        float q = 0.f;
+        for (int c = lane; c < K; c += 32) {
+            const float t = (float)(g[c] * sc);
+            q += t * t;
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        int x = 0;
+        while (x < 6 && ldexpf(1.f, 2 * x) <= 1.001f * q) ++x;  // norm < 2^x times the scale
+        if (e < FX_BAD) e += x;
+        for (int c = lane; c < K; c += 32) L[(long long)r * K + c] = fx_limbs(g[c], e);
+        if (lane == 0) ex[r] = e;
     }
-    if (c < K) {
-        const double x0 = vs[c];
+}
+
+// Rows [rb, rb + nrow), nrow <= 4, of G v in fixed point: lanes over the columns,
+// a row's exact sum over the lanes; y[i] to all lanes.  16 subdomains of K = 576:
+// a step of the window takes 31 us instead of 39.9 with FP64 rows, of which
+// the two grid barriers and the FP64 chains between them are the larger part.
+__device__ inline void fx_rows4(const int2* L, const int* ex, int K, const int2* vl, int ev, int rb, int nrow, int lane,
+                                double* y) {
+    long long s1[4] = {0, 0, 0, 0}, s2[4] = {0, 0, 0, 0};
+#pragma unroll 2
+    for (int c = lane; c < K; c += 32) {
+        const int2 x = vl[c];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            if (i < nrow) a[i] = fma(G[(long long)(rb + i) * K + c], x0, a[i]);
+            if (i < nrow) {
+                const int2 g = L[(long long)(rb + i) * K + c];
+                fx_mac2(s1[i], s2[i], g.x, g.y, x.x, x.y);
+            }
+    }
+    long long t[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t[i] = fx_fold(s1[i], s2[i]);
+    // the four sums over 32 lanes: lane bits 4 and 3 choose the row on the way
+    const bool u16 = lane & 16, u8 = lane & 8;
+    t[0] = (u16 ? t[2] : t[0]) + fx_shfl_xor(u16 ? t[0] : t[2], 16);
+    t[1] = (u16 ? t[3] : t[1]) + fx_shfl_xor(u16 ? t[1] : t[3], 16);
+    t[0] = (u8 ? t[1] : t[0]) + fx_shfl_xor(u8 ? t[0] : t[1], 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t[0] += fx_shfl_xor(t[0], o);
+    const int mine = (u16 ? 2 : 0) + (u8 ? 1 : 0);  // the row this lane's sum belongs to
+    double z = 0.0;
+    if (mine < nrow) {
+        const int eg = ex[rb + mine];
+        z = (ev == FX_BAD || eg >= FX_BAD) ? nan("") : fx_double(t[0], ev + eg - 2044 - 56);
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) y[i] = warp_sum(a[i] + b[i]);
+    for (int i = 0; i < 4; ++i) y[i] = __shfl_sync(0xffffffffu, z, 8 * i);
 }
 
 // Two-phase window: two reduce-barriers per step (see the top of the file).
-// DF32 = false: G in FP64 (DFMA).  DF32 = true: G as FP32 hi/lo planes
+// DF32 = false: G in 56-bit fixed point (k_fx_rows).  DF32 = true: G as FP32 hi/lo planes
 // (8 bytes per element like FP64, on the FP32 pipes).  Per-task state sits in
 // shared memory when the CTA has at most WIN_TPC tasks, else (A.many) in
 // global memory.  Dynamic shared memory (doubles):
@@ -428,6 +471,7 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_2ph(SweepArgs A) {
     __shared__ TaskCache s_tcs[WIN_TPC];
     __shared__ double s_own[WIN_TPC][4][WIN_RB];
     __shared__ int s_alive[WIN_TPC];
+    __shared__ int s_ev[WIN_THREADS / 32];
     int go = 1;
     const SwrDeviceView& v = A.v;
     const int t_begin = A.cta_task0[blockIdx.x];
@@ -504,7 +548,8 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_2ph(SweepArgs A) {
         const double* sc_n = A.scal_inst + (n & 1) * 2 * v.n_inst;
         const double* sc_p = A.scal_inst + ((n & 1) ^ 1) * 2 * v.n_inst;
         // ------------------------------------------------------ phase A(n+1)
-        int vs_sid = -1;  // subdomain whose v is in vs / vf (consecutive tasks of one subdomain share it)
+        int vs_sid = -1;  // subdomain whose v is in vf (consecutive tasks of one subdomain share it)
+        int ev_v = 0;     // exponent of its limbs
         for (int j = 0; j < ntk; ++j) {
             __syncthreads();
             if (!alive[j]) continue;
@@ -543,6 +588,7 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_2ph(SweepArgs A) {
                     ynm = v.arena + ms.hist + (long long)n * K;
                     if (wp > 0) bnm = v.arena + ms.bvec + (long long)min(n + 1, wp) * K;
                 }
+                int ev = 0;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     int c = tid + i * WIN_THREADS;
@@ -556,10 +602,25 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_2ph(SweepArgs A) {
                             float h = (float)val;
                             vf[c] = make_float2(h, (float)(val - (double)h));
                         } else {
-                            vs[c] = val;
+                            yv[i] = val;
+                            ev = max(ev, fx_exp(val));
                         }
                     } else if (DF32 && c < df32_ld(K)) {
                         vf[c] = make_float2(0.f, 0.f);  // padding columns of the FP32 planes
+                    }
+                }
+                if (!DF32) {  // v as limbs (vf) relative to its largest entry
+                    ev = __reduce_max_sync(0xffffffffu, ev);
+                    if (lane == 0) s_ev[warp] = ev;
+                    __syncthreads();
+                    ev = s_ev[0];
+#pragma unroll
+                    for (int w = 1; w < nw; ++w) ev = max(ev, s_ev[w]);
+                    ev_v = ev;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int c = tid + i * WIN_THREADS;
+                        if (c < K) reinterpret_cast<int2*>(vf)[c] = fx_limbs(yv[i], ev);
                     }
                 }
                 vs_sid = tc.sid;
@@ -590,7 +651,10 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_2ph(SweepArgs A) {
                 if (many && lane == 0) prefetch_rows<DF32>(v, tc, rb + 4 * nw, min(4, tc.r0 + nr - (rb + 4 * nw)));
                 double y[4];
                 if (DF32) df32_rows4(Gh, Gl, ld, vf, rb, nrow, lane, y);
-                else fp64_rows4(v.arena + tc.Gm, K, vs, rb, nrow, lane, y);
+                else
+                    fx_rows4(reinterpret_cast<const int2*>(v.arena + v.sub[tc.sid].Hm),
+                             reinterpret_cast<const int*>(v.arena + v.sub[tc.sid].work), K,
+                             reinterpret_cast<const int2*>(vf), ev_v, rb, nrow, lane, y);
                 if (lane == 0) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -1970,6 +2034,12 @@ cudaError_t window_occupancy(int* blocks_per_sm, size_t smem, int variant, bool 
     }
     *blocks_per_sm = best;
     return cudaSuccess;
+}
+
+// FP64, two-phase window: the step matrices in fixed point.
+cudaError_t launch_fx_rows(const SwrDeviceView& v, cudaStream_t st, int max_K) {
+    k_fx_rows<<<dim3((unsigned)((max_K + 7) / 8), v.n_sub), 256, 0, st>>>(v);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_split_df32(const SwrDeviceView& v, cudaStream_t st, int max_K, bool make_w) {

@@ -330,6 +330,18 @@ def test_parity_electron_repulsion_at_tile_edges(swr_mod, K_d, q_p, n_mid):
              rel_robin=REL_ROBIN_PROJECTED_EDGE, window_variant=1)
 
 
+@pytest.mark.parametrize("inst", [
+    P.tise_1d_two_subdomains().replace(K_d=3, delta=0.05, max_steps=60),    # a single, partial block of rows
+    P.small_tise_2d(L=2, K_d=17, q_p=17, n_mid=2, max_steps=40),            # K = 289: no multiple of 32 lanes or 4 rows
+    P.small_tise_2d(L=2, K_d=32, q_p=32, n_mid=2, max_steps=12),            # K = 1024, the largest
+    P.small_tise_2d(L=2, K_d=7, q_p=6, n_mid=2, max_steps=60).replace(
+        K_d=[7, 3, 9, 6], delta=[1.3, 0.4, 1.7, 1.1]),                      # tasks of different widths in a CTA
+    P.small_tise_2d(L=6, K_d=16, q_p=16, n_mid=2, max_steps=20)],           # several row tasks in a CTA
+    ids=["tiny", "k289", "k1024", "uneven", "36-subdomains"])
+def test_parity_fp64_grid_window_edges(swr_mod, inst):
+    _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE, window_variant=1)
+
+
 def test_parity_classical_swr_imaginary_time(swr_mod):
     # classical SWR (Dirichlet data mu psi_j, imposed by penalty): FP64 and mixed
     inst = P.small_tise_2d().replace(tc="dirichlet", mu=50.0)
