@@ -34,7 +34,7 @@ int window_tasks_per_cta_max();
 int window_rows_per_task_max();
 cudaError_t window_occupancy(int* blocks_per_sm, size_t smem, int variant, bool df32);
 cudaError_t launch_split_df32(const SwrDeviceView& v, cudaStream_t st, int max_K, bool make_w);
-cudaError_t launch_fx_rows(const SwrDeviceView& v, cudaStream_t st, int max_K);
+cudaError_t launch_fx_rows(const SwrDeviceView& v, cudaStream_t st, int max_K, bool w);
 cudaError_t launch_window(SweepArgs& a, int grid, size_t smem, cudaStream_t st, int n_inst, int variant, bool df32,
                           bool onep, cudaEvent_t ev_begin, cudaEvent_t ev_end);
 extern const int kAssembleLaunchesFixed, kStepLaunches;
@@ -91,6 +91,7 @@ struct swr_ctx {
     std::vector<double> cn_sweeps;       // real time: matvecs with G0 per subdomain over the whole window
     unsigned char* d_cn_need = nullptr;
     bool oc = false;                     // FP64, automatic plan: on-chip window, one cluster per instance
+    bool w1 = false;                     // FP64, automatic plan: one-pass grid window (k_window_fx)
     OcPlan oc_shape;
     int *d_oc_bounds = nullptr, *d_oc_row0 = nullptr;
     bool rt = false;                     // real time in fixed point (every precision but SWR_PREC_FP32_REFINED)
@@ -345,6 +346,10 @@ static swr_status validate(swr_ctx* c, const swr_problem* p) {
 static const int ROWS_MIN = 8;          // smallest row task
 static const int ROWS_MANY_MAX = 256;    // largest row task (task state in global memory)
 static const size_t WIN_SMEM_TASKS_MAX = 100 * 1024;  // dynamic shared memory for two CTAs per SM
+// FP64 one-pass window (k_window_fx): G and W must stay in L2 (129 MB).  us per step
+// one-pass / two-phase: 16 x 576^2 (85 MB) 18.8 / 32.2, 100 x 256^2 (105 MB) 30.4 /
+// 59.4, 25 x 576^2 (133 MB) 32.1 / 40.2, 9 x 1024^2 (151 MB) 47.2 / 38.8.
+static const double W1_BYTES_MAX = 110e6;
 static const int SPLIT_STAGES = 2;       // split window: stages of staged step-matrix rows in flight per CTA
 static const int SPLIT_STAGE_ROWS = 4;   // split window: rows of the widest subdomain per stage (at most)
 
@@ -538,6 +543,10 @@ static bool plan_window(swr_ctx* c, int variant_req, int rows_req, bool have_dev
     // FP64, nothing asked for: the two-phase recursion on chip where every
     // instance fits one cluster (2 subdomains of 40 Gaussians: 15.6 -> 2.9 us per
     // step, 9 of K = 121: 16.0 -> 6.0); the plan below is kept for its tasks
+    c->w1 = false;
+    double gw_bytes = 0;  // G and W of the subdomains that are solved
+    for (const SubDev& s : c->sub)
+        if (!(c->inst[s.inst].anti && s.N == 2 && s.idx[0] > s.idx[1])) gw_bytes += 2.0 * 8.0 * s.K * s.K;
     c->oc = variant_req == 0 && rows_req == 0 && !c->df32 && !c->tdse && !c->any_anti && have_dev &&
             oc_plan(c->inst, c->sub, nsm, &c->oc_shape);
     if (variant_req == WIN_CLUSTER) return plan_cluster(c, rows_req, have_dev);
@@ -557,6 +566,7 @@ static bool plan_window(swr_ctx* c, int variant_req, int rows_req, bool have_dev
         if (variant == WIN_SPLIT && !c->df32) return false;
         if (variant == WIN_RESIDENT && (!c->df32 || c->tdse || c->any_anti || !fits)) return false;
         c->variant = variant;
+        c->w1 = variant_req == 0 && rows_req == 0 && fits && !c->df32 && !c->tdse && !c->oc && gw_bytes <= W1_BYTES_MAX;
         c->many = (fits && variant != WIN_SPLIT) ? 0 : 1;  // the split kernel keeps task state in global memory
         const long long gres_floats = (long long)c->max_rows * df32_ld(c->max_K);
         c->g_resident = (variant == WIN_FUSED && c->tasks_per_cta == 1 &&
@@ -583,7 +593,7 @@ static bool plan_window(swr_ctx* c, int variant_req, int rows_req, bool have_dev
         c->bps = per_sm;
         if (!have_dev) return true;
         int bps = 0;
-        if (window_occupancy(&bps, c->win_smem, c->variant, c->df32) != cudaSuccess) {
+        if (window_occupancy(&bps, c->win_smem, c->w1 ? WIN_FX : c->variant, c->df32) != cudaSuccess) {
             cudaGetLastError();
             bps = 0;
         }
@@ -1142,8 +1152,8 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     if (c->rt) CU(launch_rt_pack(view(c), c->stream, c->max_K));
     else if (c->tdse) CU(launch_split_c_df32(view(c), c->stream, c->max_K));
     if (c->robin_w) CU(launch_robin_ge(view(c), c->stream, c->max_K, c->max_J));
-    if (c->oc) CU(launch_oc_make_w(view(c), c->stream, c->max_K));
-    else if (!c->df32 && !c->tdse) CU(launch_fx_rows(view(c), c->stream, c->max_K));
+    if (c->oc || c->w1) CU(launch_oc_make_w(view(c), c->stream, c->max_K));
+    if (!c->oc && !c->df32 && !c->tdse) CU(launch_fx_rows(view(c), c->stream, c->max_K, c->w1));
     CU(cudaEventRecord(c->ev1, c->stream));
     swr_status st = check_err(c);
     if (st != SWR_OK) return st;
@@ -1152,7 +1162,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     c->counters[6] += ams;
     c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 3) : 0) +
                       (c->tg ? 5 : 3) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
-                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (!c->df32 && !c->tdse ? 1 : 0);
+                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (!c->df32 && !c->tdse ? (c->w1 ? 2 : 1) : 0);
     c->assembled = true;
     c->k = 0;
     c->parity = 0;
@@ -1211,7 +1221,7 @@ static SweepArgs sweep_args(swr_ctx* c) {
 // The imaginary-time window between its two events.
 static cudaError_t run_window(swr_ctx* c, SweepArgs& a, cudaStream_t st) {
     if (!c->oc)
-        return launch_window(a, c->grid, c->win_smem, st, (int)c->inst.size(), c->variant, c->df32, fp32_phase(c), c->evw0,
+        return launch_window(a, c->grid, c->win_smem, st, (int)c->inst.size(), c->w1 ? WIN_FX : c->variant, c->df32, fp32_phase(c), c->evw0,
                              c->evw1);
     cudaError_t e = record_event(c->evw0, st);
     if (e == cudaSuccess) e = launch_oc_window(a, c->oc_shape, c->d_oc_bounds, c->d_oc_row0, st);
@@ -1470,7 +1480,7 @@ extern "C" swr_status swr_autotune(swr_ctx* c, int steps, swr_tune_report* out) 
     for (size_t i = 0; i < cands.size(); ++i) {
         if (!plan_window(c, cands[i].variant, cands[i].rows, true)) continue;
         if (c->bps < 1 || c->grid > c->bps * c->nsm) continue;
-        std::vector<int> sig = {c->variant, (int)c->tasks.size(), c->grid, c->rows_target, c->oc ? 1 : 0};
+        std::vector<int> sig = {c->variant, (int)c->tasks.size(), c->grid, c->rows_target, c->oc ? 1 : c->w1 ? 2 : 0};
         bool dup = false;
         for (const auto& x : seen) dup = dup || x == sig;
         if (dup) continue;
@@ -1482,7 +1492,7 @@ extern "C" swr_status swr_autotune(swr_ctx* c, int steps, swr_tune_report* out) 
         if (i == 0) t_default = t;
         if (t < best_t) {
             best_t = t;
-            best = c->oc ? cands[i] : Cand{c->variant, c->rows_target};  // (on chip: the automatic plan as it is)
+            best = c->oc || c->w1 ? cands[i] : Cand{c->variant, c->rows_target};  // (the automatic FP64 plan as it is)
         }
     }
     drop_graphs(c);  // captured with the old plan's launch configuration

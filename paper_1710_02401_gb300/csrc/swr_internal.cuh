@@ -260,7 +260,8 @@ struct TaskCache {
 };
 
 // Window kernel variants.
-enum WindowVariant { WIN_TWO_PHASE = 1, WIN_FUSED = 2, WIN_SPLIT = 3, WIN_RESIDENT = 4, WIN_CLUSTER = 5 };
+// (WIN_FX: the FP64 one-pass kernel of the automatic two-phase plan, not requested by number.)
+enum WindowVariant { WIN_TWO_PHASE = 1, WIN_FUSED = 2, WIN_SPLIT = 3, WIN_RESIDENT = 4, WIN_CLUSTER = 5, WIN_FX = 6 };
 
 // Event record that becomes an event-record node of the graph under stream
 // capture (external record) and is a plain record otherwise.

@@ -78,7 +78,7 @@ __global__ void k_oc_make_w(SwrDeviceView v) {
     const double* P2 = v.arena + s.t1[s.N == 2 ? 1 : 0] + lay.mat(M_PP);
     const double* G = v.arena + s.Gm;
     double* W = v.arena + s.Hm;
-    __shared__ double Y[OC_KMAX], T[OC_KMAX];
+    __shared__ double Y[1024], T[1024];  // K <= 1024
     for (int j = blockIdx.x; j < K; j += gridDim.x) {
         for (int r = threadIdx.x; r < K; r += blockDim.x) Y[r] = G[(long long)r * K + j];
         __syncthreads();

@@ -337,7 +337,7 @@ __device__ inline void prefetch_rows(const SwrDeviceView& v, const TaskCache& tc
         prefetch_l2(Gh + rb * ld, (size_t)nrow * ld * sizeof(float));
         prefetch_l2(Gh + (long long)tc.K * ld + rb * ld, (size_t)nrow * ld * sizeof(float));
     } else {
-        prefetch_l2(v.arena + v.sub[tc.sid].Hm + (long long)rb * tc.K, (size_t)nrow * tc.K * sizeof(int2));
+        prefetch_l2(v.arena + tc.Gm + (long long)rb * tc.K, (size_t)nrow * tc.K * sizeof(int2));
     }
 }
 
@@ -388,23 +388,24 @@ __device__ inline void df32_rows4(const float* Gh, const float* Gl, int ld, cons
     }
 }
 
-// Limbs of the FP64 step-matrix inverse into the space of H' (not needed after
-// the inversion), every row scaled by a power of two above its 2-norm, whose
-// exponent goes to the assembly's scratch: the two-phase FP64 window reads 8
-// bytes per element as before.  With rows and columns of norm at most 2^28 the
-// sums stay below 2^61 for K <= 1024.
+// The FP64 step-matrix inverse G (blockIdx.z = 0) and, for the one-pass window,
+// W = (Pp (x) Pp) G in the space of H' (blockIdx.z = 1) as limbs in their own
+// place, every row scaled by a power of two above its 2-norm, whose exponent goes
+// to the assembly's scratch ([2][K] ints): the FP64 grid windows read 8 bytes per
+// element as before.  With rows and columns of norm at most 2^28 the sums stay
+// below 2^61 for K <= 1024.
 __global__ void k_fx_rows(SwrDeviceView v) {
     const SubDev& s = v.sub[blockIdx.y];
     const int K = s.K, lane = threadIdx.x & 31;
-    int2* L = reinterpret_cast<int2*>(v.arena + s.Hm);
-    int* ex = reinterpret_cast<int*>(v.arena + s.work);
+    double* M = v.arena + (blockIdx.z ? s.Hm : s.Gm);
+    int* ex = reinterpret_cast<int*>(v.arena + s.work) + (long long)blockIdx.z * K;
     for (int r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); r < K; r += gridDim.x * (blockDim.x / 32)) {
-        const double* g = v.arena + s.Gm + (long long)r * K;
+        double* g = M + (long long)r * K;
         int e = 0;
         for (int c = lane; c < K; c += 32) e = max(e, fx_exp(g[c]));
         e = __reduce_max_sync(0xffffffffu, e);
-        // the 2-norm over the largest entry: 2^(e - 1022) <= norm bound < 2^(e - 1022 + x)
-        const double sc = e > 0 && e < 2046 ? __hiloint2double((2045 - e) << 20, 0) : 0.0;
+        // the 2-norm over the largest entry, as a power of two above it
+        const double sc = e > 0 && e < 2045 ? __hiloint2double((2045 - e) << 20, 0) : 0.0;
         float q = 0.f;
         for (int c = lane; c < K; c += 32) {
             const float t = (float)(g[c] * sc);
@@ -413,9 +414,9 @@ __global__ void k_fx_rows(SwrDeviceView v) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
         int x = 0;
-        while (x < 6 && ldexpf(1.f, 2 * x) <= 1.001f * q) ++x;  // norm < 2^x times the scale
+        while (x < 6 && ldexpf(1.f, 2 * x) <= 1.001f * q) ++x;
         if (e < FX_BAD) e += x;
-        for (int c = lane; c < K; c += 32) L[(long long)r * K + c] = fx_limbs(g[c], e);
+        for (int c = lane; c < K; c += 32) reinterpret_cast<int2*>(g)[c] = fx_limbs(g[c], e);
         if (lane == 0) ex[r] = e;
     }
 }
@@ -652,7 +653,7 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_2ph(SweepArgs A) {
                 double y[4];
                 if (DF32) df32_rows4(Gh, Gl, ld, vf, rb, nrow, lane, y);
                 else
-                    fx_rows4(reinterpret_cast<const int2*>(v.arena + v.sub[tc.sid].Hm),
+                    fx_rows4(reinterpret_cast<const int2*>(v.arena + tc.Gm),
                              reinterpret_cast<const int*>(v.arena + v.sub[tc.sid].work), K,
                              reinterpret_cast<const int2*>(vf), ev_v, rb, nrow, lane, y);
                 if (lane == 0) {
@@ -996,6 +997,270 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_fused(SweepArgs A) {
         if (!release_barrier(&A.bar->count, &A.bar->gen, target, gen, v.err, A.spin_limit, A.n_active, &go)) return;
         if (!go) return;
         task_sums();
+    }
+}
+
+// ------------------------------------------------------ FP64 one-pass window
+//
+// FP64, one grid barrier per step: the recursion of the fused window above with
+// G and W = (Pp (x) Pp) G in 56-bit fixed point (k_fx_rows).  The two-phase
+// window spends most of its step in two barriers and in the FP64 chains of z =
+// (Pp (x) Pp) y between them; reading W as well costs 8 more bytes per element,
+// which pays while both matrices stay in L2 (the plan's rule).  Bound by the
+// integer multiply-adds (4.5 per clock and SM, 8 us of a step below) and the L2
+// reads of both matrices.  16 subdomains of K = 576: 18.8 us per step, 32.2
+// two-phase.
+
+// Rows [rb, rb + nrow), nrow <= 4, of y = G v and z = W v: lanes over the columns,
+// the eight exact sums transposed over the lanes on the way, lane 4 k gets sum k.
+__device__ inline void fx_rows4_yz(const int2* G, const int2* W, const int* eg, const int* ew, int K, const int2* vl, int ev,
+                                   int rb, int nrow, int lane, double* ynew, double* yslot, double* zslot) {
+    long long s1[8] = {}, s2[8] = {};
+    const int2 *g[4], *w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {  // (past the last row: that row once more)
+        g[i] = G + (long long)(rb + min(i, nrow - 1)) * K;
+        w[i] = W + (long long)(rb + min(i, nrow - 1)) * K;
+    }
+#pragma unroll 2
+    for (int c = lane; c < K; c += 32) {
+        const int2 x = vl[c];
+        int2 m[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            m[i] = g[i][c];
+            m[4 + i] = w[i][c];
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) fx_mac2(s1[i], s2[i], m[i].x, m[i].y, x.x, x.y);
+    }
+    long long t[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t[i] = fx_fold(s1[i], s2[i]);
+    const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t[i] = (u16 ? t[i + 4] : t[i]) + fx_shfl_xor(u16 ? t[i] : t[i + 4], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) t[i] = (u8 ? t[i + 2] : t[i]) + fx_shfl_xor(u8 ? t[i] : t[i + 2], 8);
+    t[0] = (u4 ? t[1] : t[0]) + fx_shfl_xor(u4 ? t[0] : t[1], 4);
+    t[0] += fx_shfl_xor(t[0], 2);
+    t[0] += fx_shfl_xor(t[0], 1);
+    const int i = (lane >> 2) & 3;
+    if ((lane & 3) == 0 && i < nrow) {
+        const int em = lane < 16 ? eg[rb + i] : ew[rb + i];
+        const double x = (ev >= FX_BAD || em >= FX_BAD) ? nan("") : fx_double(t[0], ev + em - 2044 - 56);
+        if (lane < 16) {
+            ynew[i] = x;
+            yslot[i] = x;
+        } else {
+            zslot[i] = x;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(WIN_THREADS, 2) k_window_fx(SweepArgs A) {
+    extern __shared__ double sm[];
+    __shared__ double red[33];
+    __shared__ TaskCache tcs[WIN_TPC];
+    __shared__ double own[WIN_TPC][6][WIN_RB];  // y slots 0..2, z slots 3..5 (ring of 3)
+    __shared__ double is_prev[WIN_TPC], s2_sm[WIN_TPC], d2_sm[WIN_TPC];
+    __shared__ int alive[WIN_TPC];
+    __shared__ double s_sc[2];
+    __shared__ int s_stop, s_ev[WIN_THREADS / 32];
+    int go = 1;
+    const SwrDeviceView& v = A.v;
+    const int t_begin = A.cta_task0[blockIdx.x];
+    const int ntk = A.cta_task0[blockIdx.x + 1] - t_begin;
+    const int cap = A.cap;
+    const int kmax = df32_ld(A.kmax), kdmax = A.kdmax;
+    double* vs = sm;
+    int2* vl = reinterpret_cast<int2*>(sm + kmax);
+    double* tmp = sm + 2 * kmax;
+    double* Psm = tmp + A.rows_max + 2 * kdmax;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = WIN_THREADS / 32;
+    unsigned target = 0, gen = 0;
+    // partials of step m in buffer m & 1: a CTA past a barrier writes the next
+    // buffer while others still sum this one
+
+    // ------------------------------------------------------- set-up + step 0
+    for (int j = 0; j < ntk; ++j) {
+        const int t = A.cta_list[t_begin + j];
+        __syncthreads();
+        if (tid == 0) {
+            tcs[j] = make_task_cache(A, t);
+            alive[j] = 1;
+            is_prev[j] = 1.0;
+        }
+        __syncthreads();
+        const TaskCache& tc = tcs[j];
+        const int K = tc.K, nr = tc.nr;
+        const double* c0 = v.arena + tc.c0;
+        for (int c = tid; c < K; c += WIN_THREADS) vs[c] = c0[c];
+        __syncthreads();
+        double* h0 = v.arena + tc.hist;
+        for (int r = tid; r < nr; r += WIN_THREADS) {
+            h0[tc.r0 + r] = vs[tc.r0 + r];
+            own[j][0][r] = vs[tc.r0 + r];  // y^0 in slot 0
+        }
+        z_rows_staged(tc, v.arena + tc.p1, v.arena + tc.p2, vs, own[j][3], tmp, Psm);  // z^0 in slot 3
+        double acc = 0;
+        for (int r = tid; r < nr; r += WIN_THREADS) acc += own[j][0][r] * own[j][3][r];
+        acc = wblock_sum(acc, red);
+        if (tid == 0) {
+            A.part_s[t] = acc * mirror_weight(v, tc);
+            A.part_d[t] = 0.0;
+        }
+    }
+    target += gridDim.x;
+    ++gen;
+    if (!release_barrier(&A.bar->count, &A.bar->gen, target, gen, v.err, A.spin_limit, nullptr, &go)) return;
+
+    for (int n = 0;; ++n) {
+        const long long rd = (n & 1) ? A.n_tasks : 0, wr = (n & 1) ? 0 : A.n_tasks;
+        for (int j = 0; j < ntk; ++j) {
+            __syncthreads();
+            if (!alive[j]) continue;
+            const TaskCache& tc = tcs[j];
+            const int K = tc.K, nr = tc.nr, inst = tc.inst;
+            const int t = A.cta_list[t_begin + j];
+            // one round trip: y^n, b'^{n+1} and the partials of s_n^2, D_{n-1}
+            const double* yn = v.arena + tc.hist + (long long)n * K;
+            const int wp = A.win_prev[inst];
+            const double* bn = (wp > 0) ? v.arena + tc.bvec + (long long)min(n + 1, wp) * K : nullptr;
+            double yv[4], bv[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = tid + i * WIN_THREADS;
+                yv[i] = (c < K) ? __ldcg(yn + c) : 0.0;
+                bv[i] = (c < K && bn) ? __ldcg(bn + c) : 0.0;
+            }
+            const bool sum = j == 0 || tcs[j - 1].inst != inst;  // (an instance's tasks stop together)
+            if (sum) {
+                double xa = 0, xb = 0;
+                for (int u = A.inst_task0[inst] + tid; u < A.inst_task0[inst + 1]; u += WIN_THREADS) {
+                    xa += __ldcg(A.part_s + rd + u);
+                    if (n >= 2) xb += __ldcg(A.part_d + rd + u);
+                }
+                xa = warp_sum(xa);
+                xb = warp_sum(xb);
+                if (lane == 0) {
+                    red[warp] = xa;
+                    red[nw + warp] = xb;
+                }
+                __syncthreads();
+            }
+            if (warp == 0) {
+                double s2 = 0, d2 = 0;
+                if (sum) {  // the warps' sums, s^2 in lanes 0-7, D in lanes 8-15
+                    double x = red[lane & 15];
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                    s2 = __shfl_sync(0xffffffffu, x, 0);
+                    d2 = __shfl_sync(0xffffffffu, x, 8);
+                } else {
+                    s2 = s2_sm[j - 1];
+                    d2 = d2_sm[j - 1];
+                }
+                if (lane == 0) {
+                    s2_sm[j] = s2;
+                    d2_sm[j] = d2;
+                    const double is_n = tc.normalize ? rsqrt(s2) : 1.0;
+                    const double s_n = tc.normalize ? s2 * is_n : 1.0;
+                    int stop = 0, w = n;
+                    if (n >= 2 && tc.ngf_stop && sqrt(fmax(d2, 0.0)) <= tc.ngf_tol) {
+                        stop = 1;
+                        w = n - 1;
+                    } else if (n >= tc.maxs || !isfinite(s_n) || s_n <= 0.0) {
+                        stop = 1;
+                    }
+                    if (tc.first) A.snorm[(long long)inst * (cap + 1) + n] = s_n;
+                    if (stop) {
+                        alive[j] = 0;
+                        if (tc.first) {
+                            A.win[inst] = w;
+                            if (!isfinite(s_n) || s_n <= 0.0) atomicOr(v.err, SWR_ERR_NUMERIC);
+                            __threadfence();
+                            atomicSub(A.n_active, 1);
+                        }
+                    } else {
+                        s_sc[0] = is_n;
+                        s_sc[1] = is_prev[j];
+                        is_prev[j] = is_n;
+                    }
+                    s_stop = stop;
+                }
+            }
+            __syncthreads();
+            if (s_stop) continue;
+            const double is_n = s_sc[0], is_p = s_sc[1];
+            // v = y^n / s_n + kappa dt b'; antisymmetric states: its antisymmetric part on
+            // a diagonal subdomain (its own mirror)
+            const bool anti = diagonal_anti(v, tc);
+            int ev = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = tid + i * WIN_THREADS;
+                if (c < K) {
+                    double val = yv[i] * is_n + tc.kdt * bv[i];
+                    if (anti) {
+                        const int sc = swap_index(c, tc.kd);
+                        val = 0.5 * (val - (__ldcg(yn + sc) * is_n + (bn ? tc.kdt * __ldcg(bn + sc) : 0.0)));
+                    }
+                    yv[i] = val;
+                    ev = max(ev, fx_exp(val));
+                }
+            }
+            ev = __reduce_max_sync(0xffffffffu, ev);
+            if (lane == 0) s_ev[warp] = ev;
+            __syncthreads();
+            ev = s_ev[0];
+#pragma unroll
+            for (int w = 1; w < nw; ++w) ev = max(ev, s_ev[w]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = tid + i * WIN_THREADS;
+                if (c < K) vl[c] = fx_limbs(yv[i], ev);
+            }
+            __syncthreads();
+            double* ynew = v.arena + tc.hist + (long long)(n + 1) * K;
+            double* yslot = own[j][(n + 1) % 3];
+            double* zslot = own[j][3 + (n + 1) % 3];
+            const SubDev& sd = v.sub[tc.sid];
+            const int* eg = reinterpret_cast<const int*>(v.arena + sd.work);
+            for (int rb = 4 * warp; rb < nr; rb += 4 * nw)
+                fx_rows4_yz(reinterpret_cast<const int2*>(v.arena + sd.Gm), reinterpret_cast<const int2*>(v.arena + sd.Hm), eg,
+                            eg + K, K, vl, ev, tc.r0 + rb, min(4, nr - rb), lane, ynew + tc.r0 + rb, yslot + rb, zslot + rb);
+            __syncthreads();
+            // partials of s_{n+1}^2 and of D_n = ||y^n/s_n - y^{n-1}/s_{n-1}||^2_chi: the own
+            // rows' (WIN_RB = 64) in the first two warps
+            const bool dn = (n >= 1 && tc.ngf_stop);
+            if (warp < 2) {
+                double acc = 0, accd = 0;
+                if (tid < nr) {
+                    acc = yslot[tid] * zslot[tid];
+                    if (dn)
+                        accd = (own[j][n % 3][tid] * is_n - own[j][(n + 2) % 3][tid] * is_p) *
+                               (own[j][3 + n % 3][tid] * is_n - own[j][3 + (n + 2) % 3][tid] * is_p);
+                }
+                acc = warp_sum(acc);
+                accd = warp_sum(accd);
+                if (lane == 0) {
+                    red[2 * nw + warp] = acc;
+                    red[2 * nw + 2 + warp] = accd;
+                }
+            }
+            __syncthreads();
+            if (tid == 0) {
+                const double mw = mirror_weight(v, tc);
+                A.part_s[wr + t] = (red[2 * nw] + red[2 * nw + 1]) * mw;
+                if (dn) A.part_d[wr + t] = (red[2 * nw + 2] + red[2 * nw + 3]) * mw;
+            }
+        }
+        __syncthreads();
+        target += gridDim.x;
+        ++gen;
+        if (!release_barrier(&A.bar->count, &A.bar->gen, target, gen, v.err, A.spin_limit, A.n_active, &go)) return;
+        if (!go) return;
     }
 }
 
@@ -2013,6 +2278,7 @@ int window_rows_per_task_max() { return WIN_RB; }
 static const void* window_kernel(int variant, bool df32, bool onep) {
     if (variant == WIN_RESIDENT)
         return onep ? (const void*)k_window_resident<true> : (const void*)k_window_resident<false>;
+    if (variant == WIN_FX) return (const void*)k_window_fx;
     if (variant == WIN_FUSED) return onep ? (const void*)k_window_fused<true> : (const void*)k_window_fused<false>;
     if (variant == WIN_SPLIT) return onep ? (const void*)k_window_split<true> : (const void*)k_window_split<false>;
     return df32 ? (const void*)k_window_2ph<true> : (const void*)k_window_2ph<false>;
@@ -2036,9 +2302,9 @@ cudaError_t window_occupancy(int* blocks_per_sm, size_t smem, int variant, bool 
     return cudaSuccess;
 }
 
-// FP64, two-phase window: the step matrices in fixed point.
-cudaError_t launch_fx_rows(const SwrDeviceView& v, cudaStream_t st, int max_K) {
-    k_fx_rows<<<dim3((unsigned)((max_K + 7) / 8), v.n_sub), 256, 0, st>>>(v);
+// FP64 grid windows: the step matrices (and W) in fixed point.
+cudaError_t launch_fx_rows(const SwrDeviceView& v, cudaStream_t st, int max_K, bool w) {
+    k_fx_rows<<<dim3((unsigned)((max_K + 7) / 8), v.n_sub, w ? 2 : 1), 256, 0, st>>>(v);
     return cudaGetLastError();
 }
 

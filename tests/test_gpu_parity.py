@@ -338,8 +338,9 @@ def test_parity_electron_repulsion_at_tile_edges(swr_mod, K_d, q_p, n_mid):
         K_d=[7, 3, 9, 6], delta=[1.3, 0.4, 1.7, 1.1]),                      # tasks of different widths in a CTA
     P.small_tise_2d(L=6, K_d=16, q_p=16, n_mid=2, max_steps=20)],           # several row tasks in a CTA
     ids=["tiny", "k289", "k1024", "uneven", "36-subdomains"])
-def test_parity_fp64_grid_window_edges(swr_mod, inst):
-    _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE, window_variant=1)
+@pytest.mark.parametrize("variant", [1, 0])  # 0: one pass over G and W where the problem is too large for one cluster
+def test_parity_fp64_grid_window_edges(swr_mod, inst, variant):
+    _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE, window_variant=variant)
 
 
 def test_parity_classical_swr_imaginary_time(swr_mod):
