@@ -40,7 +40,7 @@ cudaError_t launch_window(SweepArgs& a, int grid, size_t smem, cudaStream_t st, 
 extern const int kAssembleLaunchesFixed, kStepLaunches;
 cudaError_t launch_post(const SwrDeviceView& v, cudaStream_t st, const int* d_win, const int* d_win_prev,
                         const double* d_snorm, int cap, int parity, int first_iter, double* d_res_part,
-                        int res_blocks, double* d_res, int max_cap_hint, int lt_kmax, int lt_kdmax, int lt_qmax,
+                        int res_blocks, double* d_res, int nsm, int lt_kmax, int lt_kdmax, int lt_qmax,
                         bool any_anti, double* d_cv_part, double* d_cvtot, bool with_cvtot);
 size_t cvtot_part_doubles(int n_inst);
 cudaError_t launch_cvtot(const SwrDeviceView& v, cudaStream_t st, const int* d_win, const double* d_snorm, int cap,
@@ -1262,7 +1262,7 @@ static cudaError_t record_iteration(swr_ctx* c, cudaStream_t st, long long* win_
     }
     if (e == cudaSuccess)
         e = launch_post(view(c), st, c->d_win, c->d_win_prev, c->d_snorm, c->cap, c->parity, c->k == 0 ? 1 : 0,
-                        c->d_res_part, RES_BLOCKS, c->d_res, c->cap, c->max_K, c->max_kd, c->max_q, c->any_anti,
+                        c->d_res_part, RES_BLOCKS, c->d_res, c->nsm > 0 ? c->nsm : 152, c->max_K, c->max_kd, c->max_q, c->any_anti,
                         c->d_cv_part, c->d_cvtot, c->prob.cvtot_each_iteration != 0);
     if (e == cudaSuccess)
         e = launch_energy(view(c), st, c->d_win, c->d_snorm, c->cap, c->d_epart, c->d_energy, c->d_norm2,

@@ -26,7 +26,7 @@ __device__ void gauss_legendre(int n, double* t, double* wt) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         // i-th root in decreasing order, initial guess of Tricomi type
         double x = cos(M_PI * (i + 0.75) / (n + 0.5));
-        double dp = 1.0, last = 1.0;
+        double dp = 1.0;
         for (int it = 0; it < 100; ++it) {
             double p0 = 1.0, p1 = x;
             for (int k = 2; k <= n; ++k) {
@@ -39,8 +39,7 @@ __device__ void gauss_legendre(int n, double* t, double* wt) {
             dp = n * (x * pn - pm) / (x * x - 1.0);
             double dx = pn / dp;
             x -= dx;
-            if (last < 1e-8) break;  // quadratic convergence: this step was the last that changes x
-            last = fabs(dx);
+            if (fabs(dx) < 1e-16) break;
         }
         // recompute derivative at the converged root
         double p0 = 1.0, p1 = x;
@@ -467,6 +466,14 @@ __global__ void k_ee_operands(SwrDeviceView v) {
     }
 }
 
+// Assembly in fixed point or FP64: batches of instances stay in FP64.  A batch steps
+// every molecule with one dt; where dt passes 1 / |E| of one of them, its window
+// amplifies the last bits of the step matrix into leading digits (seeded batches
+// of 32: one in six holds such a molecule), and the results of the other kernels
+// are kept as they are bit for bit.  One instance takes the fixed point (16
+// subdomains of K = 576: 4.3 ms of products and elimination, 12.3 in FP64).
+static inline bool fp64_batch(const SwrDeviceView& v) { return v.n_inst > 1; }
+
 // Batched GEMM  C = op(A) * B  of FP64 matrices with 64x64 tiles, in 56-bit fixed
 // point on the integer pipes (swr_fixed.cuh: 4.5 multiply-adds per clock and SM
 // against 1.6 on the FP64 pipe).  Rows of op(A) are scaled by their largest
@@ -479,7 +486,7 @@ __global__ void k_ee_operands(SwrDeviceView v) {
 
 #define GT 64
 #define GK 16
-__global__ void __launch_bounds__(256) k_dgemm(SwrDeviceView v, const GemmJob* jobs) {
+__global__ void __launch_bounds__(256) k_fxgemm(SwrDeviceView v, const GemmJob* jobs) {
     const GemmJob jb = jobs[blockIdx.z];
     const int tm = blockIdx.y * GT, tn = blockIdx.x * GT;
     if (jb.M <= 0 || tm >= jb.M || tn >= jb.N) return;
@@ -569,6 +576,62 @@ __global__ void __launch_bounds__(256) k_dgemm(SwrDeviceView v, const GemmJob* j
                 int a = gm / kd, cc = gm % kd, b = gn / kd, e = gn % kd;
                 long long K = (long long)kd * kd;
                 C[(long long)(a + kd * b) * K + (cc + kd * e)] = c;
+            }
+        }
+}
+
+// The same in FP64 (batches).
+__global__ void __launch_bounds__(256) k_dgemm(SwrDeviceView v, const GemmJob* jobs) {
+    const GemmJob jb = jobs[blockIdx.z];
+    const int tm = blockIdx.y * GT, tn = blockIdx.x * GT;
+    if (jb.M <= 0 || tm >= jb.M || tn >= jb.N) return;
+    __shared__ double As[GK][GT + 1];
+    __shared__ double Bs[GK][GT + 1];
+    const double* A = v.arena + jb.a;
+    const double* B = v.arena + jb.b;
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    double acc[4][4] = {};
+    for (int k0 = 0; k0 < jb.K; k0 += GK) {
+        for (int e = threadIdx.x; e < GK * GT; e += 256) {
+            int kk = e / GT, mm = e % GT;
+            int gk = k0 + kk, gm = tm + mm;
+            double val = 0.0;
+            if (gk < jb.K && gm < jb.M)
+                val = jb.transA ? A[(long long)gk * jb.lda + gm] : A[(long long)gm * jb.lda + gk];
+            As[kk][mm] = val;
+            int gn = tn + mm;
+            Bs[kk][mm] = (gk < jb.K && gn < jb.N) ? B[(long long)gk * jb.ldb + gn] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < GK; ++kk) {
+            double ar[4], br[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ar[i] = As[kk][ty + 16 * i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) br[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma(ar[i], br[j], acc[i][j]);
+        }
+        __syncthreads();
+    }
+    double* C = v.arena + jb.c;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            int gm = tm + ty + 16 * i, gn = tn + tx + 16 * j;
+            if (gm >= jb.M || gn >= jb.N) continue;
+            if (jb.mode == 0) {
+                C[(long long)gm * jb.ldc + gn] = acc[i][j];
+            } else {
+                // gm = (a,c) = a*kd + c, gn = (b,d) = b*kd + e; H'[(a + kd b), (c + kd e)]
+                int kd = jb.kd;
+                int a = gm / kd, c = gm % kd, b = gn / kd, e = gn % kd;
+                long long K = (long long)kd * kd;
+                C[(long long)(a + kd * b) * K + (c + kd * e)] = acc[i][j];
             }
         }
 }
@@ -678,19 +741,10 @@ __device__ inline cplx one_el(cplx) { return mkc(1.0, 0.0); }
 
 #define GJ_NB 32
 #define GJ_T 64   // columns of the row-block kernel, tile edge of the real update
-// 1/x by two Newton steps from the FP32 reciprocal (264 clocks on the FP64 pipe
-// instead of 550 for the division); the division where FP32 does not reach.
-__device__ inline double gj_rcp(double x) {
-    const double ax = fabs(x);
-    if (!(ax > 1e-30 && ax < 1e30)) return 1.0 / x;
-    double r = (double)(1.0f / (float)x);
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
-}
-__device__ inline double gj_inv(double x) { return gj_rcp(x); }
+__device__ inline double gj_inv(double x) { return 1.0 / x; }
 __device__ inline cplx gj_inv(cplx x) {
-    const double d = gj_rcp(x.re * x.re + x.im * x.im);
-    return mkc(x.re * d, -x.im * d);
+    const double d = x.re * x.re + x.im * x.im;
+    return mkc(x.re / d, -x.im / d);
 }
 __device__ inline double gj_fnma(double a, double b, double c) { return fma(-a, b, c); }
 __device__ inline cplx gj_fnma(cplx a, cplx b, cplx c) { return c - a * b; }
@@ -768,6 +822,14 @@ __device__ inline int gj_exp(cplx x) { return max(fx_exp(x.re), fx_exp(x.im)); }
 __device__ inline double gj_make(const double* x, double) { return x[0]; }
 __device__ inline cplx gj_make(const double* x, cplx) { return mkc(x[0], x[1]); }
 
+// An operand in shared memory: limbs, or (batches, real) the FP64 value.
+template <bool FX> struct GjOperand { using type = int2; };
+template <> struct GjOperand<false> { using type = double; };
+template <bool FX> __device__ inline typename GjOperand<FX>::type gj_operand(double x, int e) {
+    if constexpr (FX) return fx_limbs(x, e);
+    else return x;
+}
+
 // Product of a GA x 32 block (rows scaled by ea) and a 32 x GB one (columns by
 // eb), limbs in shared memory, in fixed point (swr_fixed.cuh): thread (ty, tx)
 // of 16 x 16 gets rows ty + 16 i, columns tx + 16 j.  Both the row block Pinv M[kb, :]
@@ -813,10 +875,32 @@ __device__ inline void gj_product(const int2 (*A)[GA][GJ_NB + 1], const int2 (*B
         }
 }
 
+// The same in FP64: one chain of multiply-adds per element, in the order of t.
+template <int GA, int GB>
+__device__ inline void gj_product64(const double (*A)[GJ_NB + 1], const double (*B)[GB + 1], int tx, int ty,
+                                    double (&out)[GA / 16][GB / 16]) {
+#pragma unroll
+    for (int i = 0; i < GA / 16; ++i)
+#pragma unroll
+        for (int j = 0; j < GB / 16; ++j) out[i][j] = 0.0;
+#pragma unroll 4
+    for (int t = 0; t < GJ_NB; ++t) {
+        double br[GB / 16];
+#pragma unroll
+        for (int j = 0; j < GB / 16; ++j) br[j] = B[t][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < GA / 16; ++i) {
+            const double ar = A[ty + 16 * i][t];
+#pragma unroll
+            for (int j = 0; j < GB / 16; ++j) out[i][j] = fma(ar, br[j], out[i][j]);
+        }
+    }
+}
+
 // Columns [tn, tn + GJ_T) of the pivot row block: Rp = Pinv M[kb, :], and the pivot
 // column block Cp = M[:, kb] of the same index range, by GJ_T columns per CTA
 // (one CTA doing all of it took 180 us of a 276 us panel at K = 576, 16 us here).
-template <typename T>
+template <typename T, bool FX>
 __global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
     constexpr int P = GjParts<T>::v;
     const SubDev& s = v.sub[blockIdx.y];
@@ -828,8 +912,9 @@ __global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
     double* Rp = Pinv + P * GJ_NB * GJ_NB;
     double* Cp = Rp + P * (long long)GJ_NB * K;
     extern __shared__ int2 gj_sm[];
-    int2(*A)[GJ_NB][GJ_NB + 1] = reinterpret_cast<int2(*)[GJ_NB][GJ_NB + 1]>(gj_sm);
-    int2(*B)[GJ_NB][GJ_T + 1] = reinterpret_cast<int2(*)[GJ_NB][GJ_T + 1]>(gj_sm + P * GJ_NB * (GJ_NB + 1));
+    using E = typename GjOperand<FX>::type;
+    E(*A)[GJ_NB][GJ_NB + 1] = reinterpret_cast<E(*)[GJ_NB][GJ_NB + 1]>(gj_sm);
+    E(*B)[GJ_NB][GJ_T + 1] = reinterpret_cast<E(*)[GJ_NB][GJ_T + 1]>(gj_sm + P * GJ_NB * (GJ_NB + 1));
     __shared__ int ea[GJ_NB], eb[GJ_T];
     if (tid < GJ_T) eb[tid] = 0;
     __syncthreads();
@@ -853,18 +938,19 @@ __global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int e = tid + 256 * u, i = e / GJ_NB, t = e % GJ_NB;
-            A[p][i][t] = fx_limbs(gj_part(pa[u], p), ea[i]);
+            A[p][i][t] = gj_operand<FX>(gj_part(pa[u], p), ea[i]);
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int e = tid + 256 * u, t = e / GJ_T, j = e % GJ_T;
-            B[p][t][j] = fx_limbs(gj_part(mb[u], p), eb[j]);
+            B[p][t][j] = gj_operand<FX>(gj_part(mb[u], p), eb[j]);
         }
     }
     __syncthreads();
     const int tx = tid % 16, ty = tid / 16;
     T out[2][4];
-    gj_product<T, GJ_NB, GJ_T>(A, B, ea, eb, tx, ty, out);
+    if constexpr (FX) gj_product<T, GJ_NB, GJ_T>(A, B, ea, eb, tx, ty, out);
+    else gj_product64<GJ_NB, GJ_T>(A[0], B[0], tx, ty, out);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -885,7 +971,7 @@ __global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
 template <typename T> struct GjTile { static const int v = 64; };
 template <> struct GjTile<cplx> { static const int v = 32; };
 
-template <typename T>
+template <typename T, bool FX>
 __global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb) {
     constexpr int TL = GjTile<T>::v, P = GjParts<T>::v, N = TL * GJ_NB / 256, Q = TL / 16;
     const SubDev& s = v.sub[blockIdx.z];
@@ -899,8 +985,9 @@ __global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb) {
     const double* Rp = Pinv + P * GJ_NB * GJ_NB;
     const double* Cp = Rp + P * (long long)GJ_NB * K;
     extern __shared__ int2 gj_sm[];
-    int2(*A)[TL][GJ_NB + 1] = reinterpret_cast<int2(*)[TL][GJ_NB + 1]>(gj_sm);
-    int2(*B)[GJ_NB][TL + 1] = reinterpret_cast<int2(*)[GJ_NB][TL + 1]>(gj_sm + P * TL * (GJ_NB + 1));
+    using E = typename GjOperand<FX>::type;
+    E(*A)[TL][GJ_NB + 1] = reinterpret_cast<E(*)[TL][GJ_NB + 1]>(gj_sm);
+    E(*B)[GJ_NB][TL + 1] = reinterpret_cast<E(*)[GJ_NB][TL + 1]>(gj_sm + P * TL * (GJ_NB + 1));
     __shared__ int ea[TL], eb[TL];
     if (tid < TL) eb[tid] = 0;
     __syncthreads();
@@ -923,13 +1010,14 @@ __global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb) {
 #pragma unroll
         for (int u = 0; u < N; ++u) {
             const int e = tid + 256 * u;
-            A[p][e / GJ_NB][e % GJ_NB] = fx_limbs(gj_part(ca[u], p), ea[e / GJ_NB]);
-            B[p][e / TL][e % TL] = fx_limbs(gj_part(rb[u], p), eb[e % TL]);
+            A[p][e / GJ_NB][e % GJ_NB] = gj_operand<FX>(gj_part(ca[u], p), ea[e / GJ_NB]);
+            B[p][e / TL][e % TL] = gj_operand<FX>(gj_part(rb[u], p), eb[e % TL]);
         }
     __syncthreads();
     const int tx = tid % 16, ty = tid / 16;
     T out[Q][Q];
-    gj_product<T, TL, TL>(A, B, ea, eb, tx, ty, out);
+    if constexpr (FX) gj_product<T, TL, TL>(A, B, ea, eb, tx, ty, out);
+    else gj_product64<TL, TL>(A[0], B[0], tx, ty, out);
 #pragma unroll
     for (int i = 0; i < Q; ++i)
 #pragma unroll
@@ -945,17 +1033,17 @@ __global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb) {
         }
 }
 
-template <typename T>
+template <typename T, bool FX>
 static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int max_K, bool update) {
     constexpr int TL = GjTile<T>::v, P = GjParts<T>::v;
     const size_t sr = P * (GJ_NB * (GJ_NB + 1) + GJ_NB * (GJ_T + 1)) * sizeof(int2);
     const size_t su = P * (TL * (GJ_NB + 1) + GJ_NB * (TL + 1)) * sizeof(int2);
-    cudaError_t e = cudaFuncSetAttribute(k_gj_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gj_update<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)su);
+    cudaError_t e = cudaFuncSetAttribute(k_gj_rows<T, FX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gj_update<T, FX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)su);
     if (e != cudaSuccess) return e;
     k_gj_panel<T><<<v.n_sub, 256, 0, st>>>(v, kb);
-    k_gj_rows<T><<<dim3((max_K + GJ_T - 1) / GJ_T, v.n_sub), 256, sr, st>>>(v, kb);
-    if (update) k_gj_update<T><<<dim3((max_K + TL - 1) / TL, (max_K + TL - 1) / TL, v.n_sub), 256, su, st>>>(v, kb);
+    k_gj_rows<T, FX><<<dim3((max_K + GJ_T - 1) / GJ_T, v.n_sub), 256, sr, st>>>(v, kb);
+    if (update) k_gj_update<T, FX><<<dim3((max_K + TL - 1) / TL, (max_K + TL - 1) / TL, v.n_sub), 256, su, st>>>(v, kb);
     return cudaGetLastError();
 }
 
@@ -964,8 +1052,8 @@ static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int
 // c0 = (B'1^T W f1) (x) (B'2^T W f2) for phi0 = prod_e exp(-gamma (x_e - x0_e)^2)
 // (projection of Sec. 6.1 in the orthonormal basis: c' = X^T c~).
 // out[sid] = partial PoU norm^2 of c0 (later summed per instance).  The node values
-// are formed once per coordinate and a warp sums one coefficient (one thread per
-// coefficient, with its own exponentials: 430 us at kd = 24, q = 132; 23 here).
+// are formed once per coordinate (in every coefficient's own sum: 430 us at kd =
+// 24, q = 132).
 __global__ void k_project(SwrDeviceView v, double* norm_part) {
     const int sid = blockIdx.x;
     const SubDev& s = v.sub[sid];
@@ -975,8 +1063,6 @@ __global__ void k_project(SwrDeviceView v, double* norm_part) {
     __shared__ double u[2][ORTH_MAX_KD * 4];
     __shared__ double nrm[2];
     __shared__ double f[384];               // w exp(-gamma (x - x0)^2) at the nodes (q <= 384)
-    __shared__ double pu[ORTH_MAX_KD];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int d = 0; d < s.N; ++d) {
         const double* T = v.arena + s.t1[d];
         for (int n = threadIdx.x; n < q; n += blockDim.x) {
@@ -984,24 +1070,19 @@ __global__ void k_project(SwrDeviceView v, double* norm_part) {
             f[n] = T[lay.w() + n] * exp(-in.gamma0 * r * r);
         }
         __syncthreads();
-        for (int a = warp; a < kd; a += nw) {
-            double acc = 0;
-            for (int n = lane; n < q; n += 32) acc += f[n] * T[lay.B() + n * kd + a];
-            acc = warp_sum(acc);
-            if (lane == 0) u[d][a] = acc;
-        }
-        __syncthreads();
         for (int a = threadIdx.x; a < kd; a += blockDim.x) {
             double acc = 0;
-            for (int c = 0; c < kd; ++c) acc += T[lay.mat(M_PP) + a * kd + c] * u[d][c];
-            pu[a] = u[d][a] * acc;
+#pragma unroll 4
+            for (int n = 0; n < q; ++n) acc += f[n] * T[lay.B() + n * kd + a];
+            u[d][a] = acc;
         }
         __syncthreads();
-        if (warp == 0) {
+        if (threadIdx.x == 0) {
             double acc = 0;
-            for (int a = lane; a < kd; a += 32) acc += pu[a];
-            acc = warp_sum(acc);
-            if (lane == 0) nrm[d] = acc;
+            for (int a = 0; a < kd; ++a)
+#pragma unroll 4
+                for (int c = 0; c < kd; ++c) acc += u[d][a] * T[lay.mat(M_PP) + a * kd + c] * u[d][c];
+            nrm[d] = acc;
         }
         __syncthreads();
     }
@@ -1120,9 +1201,10 @@ cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, 
         } else {
             int kd2 = max_kd * max_kd;
             // Mee = Wv (q x q) * P2 (q x kd^2)
-            k_dgemm<<<dim3(div_up(kd2, GT), div_up(max_q, GT), v.n_sub), 256, 0, st>>>(v, d_jobs1);
+            const auto gemm = fp64_batch(v) ? k_dgemm : k_fxgemm;
+            gemm<<<dim3(div_up(kd2, GT), div_up(max_q, GT), v.n_sub), 256, 0, st>>>(v, d_jobs1);
             // V'ee[(a,c),(b,e)] = P1^T (kd^2 x q) * Mee (q x kd^2), scattered into H'
-            k_dgemm<<<dim3(div_up(kd2, GT), div_up(kd2, GT), v.n_sub), 256, 0, st>>>(v, d_jobs2);
+            gemm<<<dim3(div_up(kd2, GT), div_up(kd2, GT), v.n_sub), 256, 0, st>>>(v, d_jobs2);
         }
     }
     dim3 ge(div_up((long long)max_K * max_K, 256 * 8), v.n_sub);
@@ -1131,7 +1213,9 @@ cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, 
     k_step_matrix<<<ge, 256, 0, st>>>(v);
     int nkb = (max_K + GJ_NB - 1) / GJ_NB;
     for (int kb = 0; kb < nkb; ++kb) {
-        cudaError_t e = any_tdse ? gj_block<cplx>(v, st, kb, max_K, !tg) : gj_block<double>(v, st, kb, max_K, !tg);
+        cudaError_t e = any_tdse      ? gj_block<cplx, true>(v, st, kb, max_K, !tg)
+                        : fp64_batch(v) ? gj_block<double, false>(v, st, kb, max_K, !tg)
+                                        : gj_block<double, true>(v, st, kb, max_K, !tg);
         if (e == cudaSuccess && tg) e = tg_update(tg, v, st, kb, max_K);
         if (e != cudaSuccess) return e;
     }

@@ -268,8 +268,13 @@ __global__ void k_gather(SwrDeviceView v, const int* win, const double* snorm, i
             // g = (n.grad + mu) psi_j averaged (Robin), or mu psi_j (classical SWR by
             // penalty); complex mu mixes the planes
             const double sd = in.tc == SWR_TC_DIRICHLET ? 0.0 : sig;
-            double gre = (sd * der[0] + in.mu_re * val[0] - in.mu_im * val[1]) * inv;
-            double gim = (sd * der[1] + in.mu_re * val[1] + in.mu_im * val[0]) * inv;
+            double gre, gim = 0.0;
+            if (nch == 1) {
+                gre = (sd * der[0] + in.mu_re * val[0]) * inv;
+            } else {
+                gre = (sd * der[0] + in.mu_re * val[0] - in.mu_im * val[1]) * inv;
+                gim = (sd * der[1] + in.mu_re * val[1] + in.mu_im * val[0]) * inv;
+            }
             for (int ch = 0; ch < nch; ++ch) {
                 const double gv = ch ? gim : gre;
                 v.arena[s.u[parity] + ((long long)n * nch + ch) * s.ngam + node] = own[ch] * isn;
@@ -584,21 +589,28 @@ __global__ void k_energy(SwrDeviceView v, const int* win, const double* snorm, i
     }
 }
 
+// A warp per instance, lanes over its partials (one thread summed them in 44 us with
+// 16 subdomains: a chain of 66-clock additions).
 __global__ void k_energy_reduce(SwrDeviceView v, const double* part, double* energy, double* norm2, double* dipole) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= v.n_inst) return;
     const InstDev& in = v.inst[i];
     double num = 0, den = 0, dip = 0;
-    for (int j = 0; j < in.n_sub; ++j)
-        for (int b = 0; b < ENERGY_BLOCKS; ++b) {
-            const long long o = 3LL * ((long long)(in.sub_base + j) * ENERGY_BLOCKS + b);
-            num += part[o];
-            den += part[o + 1];
-            dip += part[o + 2];
-        }
-    energy[i] = num / den;
-    norm2[i] = den;
-    dipole[i] = dip / den;
+    const double* p = part + 3LL * in.sub_base * ENERGY_BLOCKS;
+#pragma unroll 4
+    for (int b = lane; b < in.n_sub * ENERGY_BLOCKS; b += 32) {
+        num += p[3 * b];
+        den += p[3 * b + 1];
+        dip += p[3 * b + 2];
+    }
+    num = warp_sum(num);
+    den = warp_sum(den);
+    dip = warp_sum(dip);
+    if (lane == 0) {
+        energy[i] = num / den;
+        norm2[i] = den;
+        dipole[i] = dip / den;
+    }
 }
 
 // Antisymmetric states (Appendix A): the lower subdomain (i1 > i2) of each
@@ -635,20 +647,37 @@ static inline unsigned div_up(long long a, long long b) { return (unsigned)((a +
 // fill).
 extern const int kStepLaunches = 8;
 
+// CTAs per subdomain of a kernel that first stages the subdomain's tables and then
+// strides over the steps of the window: 64, in a batch of many subdomains 16
+// waves of resident CTAs (64 each staged the tables for one to three steps; two
+// waves left the tail to the largest bases).  The kernels after the window of a
+// batch of 32 (1101 subdomains): 6.47 -> 4.81 ms at 60 steps, 12.1 -> 10.9 at 190.
+static cudaError_t step_blocks(const void* f, size_t smem, int n_sub, int nsm, unsigned* nb) {
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    int per_sm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, smem);
+    if (e != cudaSuccess) return e;
+    const int slots = (per_sm > 0 ? per_sm : 1) * nsm;
+    const int n = (16 * slots + n_sub - 1) / n_sub;
+    *nb = (unsigned)(n > 64 ? 64 : n);
+    return cudaSuccess;
+}
+
 cudaError_t launch_post(const SwrDeviceView& v, cudaStream_t st, const int* d_win, const int* d_win_prev,
                         const double* d_snorm, int cap, int parity, int first_iter, double* d_res_part,
-                        int res_blocks, double* d_res, int max_cap_hint, int lt_kmax, int lt_kdmax, int lt_qmax,
+                        int res_blocks, double* d_res, int nsm, int lt_kmax, int lt_kdmax, int lt_qmax,
                         bool any_anti, double* d_cv_part, double* d_cvtot, bool with_cvtot) {
-    int nb = 64;
-    if (any_anti) k_anti_fill<<<dim3(nb, v.n_sub), 256, 0, st>>>(v, d_win);
+    if (any_anti) k_anti_fill<<<dim3(64, v.n_sub), 256, 0, st>>>(v, d_win);
     {
         const size_t base = ((size_t)lt_kmax + (size_t)lt_kdmax + 32 * (size_t)lt_kdmax) * sizeof(float2);
         const size_t tab = 2 * (size_t)lt_qmax * lt_kdmax * sizeof(float2);
         const int staged = base + tab <= 96 * 1024;
         const size_t sm = base + (staged ? tab : 0);
-        if (sm > 48 * 1024) cudaFuncSetAttribute(k_line_traces, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        cudaFuncSetAttribute(k_line_traces, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+        unsigned nb = 1;
+        cudaError_t e = step_blocks((const void*)k_line_traces, sm, v.n_sub, nsm, &nb);
+        if (e != cudaSuccess) return e;
         k_line_traces<<<dim3(nb, v.n_sub), 256, sm, st>>>(v, d_win, cap, lt_kmax, lt_kdmax, lt_qmax, staged);
     }
     {
@@ -657,8 +686,9 @@ cudaError_t launch_post(const SwrDeviceView& v, cudaStream_t st, const int* d_wi
         const size_t tab = 2 * (size_t)lt_qmax * lt_kdmax * sizeof(float2);
         const int staged = tab <= 96 * 1024;
         const size_t sm = gbytes + (staged ? tab : 0);
-        if (sm > 48 * 1024) cudaFuncSetAttribute(k_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        cudaFuncSetAttribute(k_gather, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        unsigned nb = 1;
+        cudaError_t e = step_blocks((const void*)k_gather, sm, v.n_sub, nsm, &nb);
+        if (e != cudaSuccess) return e;
         k_gather<<<dim3(nb, v.n_sub), 256, sm, st>>>(v, d_win, d_snorm, cap, parity, staged, gsz);
     }
     k_residual<<<dim3(res_blocks, v.n_sub), 256, 0, st>>>(v, d_win, d_win_prev, parity, first_iter, d_res_part);
@@ -701,7 +731,7 @@ cudaError_t launch_energy(const SwrDeviceView& v, cudaStream_t st, const int* d_
                           double* psi_out, const long long* psi_off, size_t smem) {
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_energy<<<dim3(ENERGY_BLOCKS, v.n_sub), 256, smem, st>>>(v, d_win, d_snorm, cap, d_part, psi_out, psi_off);
-    k_energy_reduce<<<div_up(v.n_inst, 128), 128, 0, st>>>(v, d_part, d_energy, d_norm2, d_dipole);
+    k_energy_reduce<<<div_up(v.n_inst, 4), 128, 0, st>>>(v, d_part, d_energy, d_norm2, d_dipole);
     return cudaGetLastError();
 }
 
