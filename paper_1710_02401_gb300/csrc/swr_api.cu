@@ -441,6 +441,33 @@ static void plan_tasks(swr_ctx* c, int target_rows, int ctas, bool by_bytes = fa
     }
 }
 
+// Split window, one instance, automatic plan: the finest blocks that give every
+// CTA at most one task, counting the subdomains that are solved (0, the total over
+// the CTAs: none up to 128 rows).  An SM with one task more than the others sets
+// the time of a step; us per step, total over the CTAs / one wave: triplet on 4 x 4
+// subdomains of K = 576 32.1 / 28.5, K = 1024 52.8 / 45.0, K = 256 21.3 / 21.3;
+// 36 subdomains of K = 576 57.1 / 40.3.  Batches keep blocks of at most 64 rows (96
+// would give a batch of 32 6 % and take 3 % from one of 8).
+static int one_wave_rows(const swr_ctx* c, int ctas) {
+    const auto fits = [&](int r) {
+        long long n = 0;
+        for (const SubDev& s : c->sub) {
+            if (c->inst[s.inst].anti && s.N == 2 && s.idx[0] > s.idx[1]) continue;
+            const long long t = std::min<long long>((r * (long long)c->max_K + s.K / 2) / s.K, ROWS_MANY_MAX);
+            n += (s.K + t - 1) / t;
+        }
+        return n <= ctas;
+    };
+    int lo = ROWS_MIN, hi = 128;
+    if (!fits(hi)) return 0;
+    while (lo < hi) {
+        const int r = (lo + hi) / 2;
+        if (fits(r)) hi = r;
+        else lo = r + 1;
+    }
+    return lo;
+}
+
 // Task capacity of the auxiliary arrays: the finest row target.
 static long long task_capacity(const swr_ctx* c) {
     long long n = 0;
@@ -556,7 +583,8 @@ static bool plan_window(swr_ctx* c, int variant_req, int rows_req, bool have_dev
     if (variant_req == 0 && rows_req == 0 && plan_cluster(c, 0, have_dev)) return true;
     for (int per_sm = 2; per_sm >= 1; --per_sm) {
         plan_tasks(c, rows_req, per_sm * nsm, variant_req == WIN_SPLIT);
-        if (variant_req == 0 && c->df32 && !c->tdse && !c->has_w) plan_tasks(c, rows_req, per_sm * nsm, true);
+        if (variant_req == 0 && c->df32 && !c->tdse && !c->has_w)
+            plan_tasks(c, rows_req == 0 && c->inst.size() == 1 ? one_wave_rows(c, per_sm * nsm) : rows_req, per_sm * nsm, true);
         const bool fits = c->tasks_per_cta <= window_tasks_per_cta_max() && c->max_rows <= window_rows_per_task_max() &&
                           window_smem(c->max_K, c->max_kd, c->max_rows, c->tasks_per_cta, 0) <= WIN_SMEM_TASKS_MAX;
         int variant = variant_req;

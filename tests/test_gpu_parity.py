@@ -343,6 +343,17 @@ def test_parity_fp64_grid_window_edges(swr_mod, inst, variant):
     _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE, window_variant=variant)
 
 
+@pytest.mark.parametrize("L,K_d", [(2, 3), (4, 11), (8, 6), (2, 20)])
+def test_parity_split_window_one_task_per_cta(swr_mod, L, K_d):
+    # automatic row blocks of the split window: smallest, K no multiple of the
+    # block, more subdomains than fit 8-row blocks in one wave, large blocks
+    s, _ = _compare(swr_mod, P.small_tise_2d(L=L, K_d=K_d, q_p=max(6, K_d), n_mid=2, max_steps=20).replace(
+        symmetry="antisymmetric", phi0_center=(0.8, -0.8)), kmax=2, precision=swr_mod.PREC_MIXED,
+        rel_robin=REL_ROBIN_PROJECTED_EDGE)
+    plan = s.window_plan()
+    assert plan["variant"] == 3 and plan["tasks"] <= plan["ctas"]
+
+
 def test_parity_classical_swr_imaginary_time(swr_mod):
     # classical SWR (Dirichlet data mu psi_j, imposed by penalty): FP64 and mixed
     inst = P.small_tise_2d().replace(tc="dirichlet", mu=50.0)
