@@ -38,8 +38,10 @@ KMAX = 200
 METRIC = "SWR time-to-1e-8 interface residual; subdomain solves/s vs plain FP64 GPU path"
 # FP64 and FP32 (non-tensor) FMA rates of one GB300, measured on this machine with
 # independent FMA chains over all SMs (the ceilings of the window kernel)
-FP64_PEAK_TFLOPS = 1.01
 FP32_PEAK_TFLOPS = 67.7
+# 56-bit fixed-point products on the integer pipes: 4.5 multiply-adds per clock
+# and SM (FP64 quality), 152 SMs at 1.92 GHz
+FIXED_PEAK_TFLOPS = 2.6
 # DRAM traffic of the window kernels from one ncu capture each (profiles/): bytes per
 # launch, or for the batched case bytes per algorithmic byte, valid only while the
 # source of the kernel and of the device functions it calls is the one that was
@@ -47,9 +49,6 @@ FP32_PEAK_TFLOPS = 67.7
 KERNEL_FUNCS = {
     "k_window_fused": ["release_barrier", "block_sums2", "two_sum", "make_task_cache", "z_rows_sm", "df32_acc",
                        "k_window_fused"],
-    "k_window_2ph<false>": ["reduce_barrier", "make_task_cache", "mirror_sid", "swap_index", "mirror_weight",
-                            "diagonal_anti", "z_rows_sm", "z_rows_staged", "prefetch_l2", "prefetch_rows",
-                            "fp64_rows4", "k_window_2ph"],
     "k_window_2ph<true>": ["reduce_barrier", "two_sum", "make_task_cache", "mirror_sid", "swap_index",
                            "mirror_weight", "diagonal_anti", "z_rows_sm", "z_rows_staged", "prefetch_l2",
                            "prefetch_rows", "df32_acc", "df32_rows4", "k_window_2ph"],
@@ -61,9 +60,10 @@ KERNEL_FUNCS["k_window_split"] = ["mbar_wait", "split_stage_rows", "reduce_barri
 KERNEL_FUNCS["k_window_2ph<true>@batched"] = KERNEL_FUNCS["k_window_2ph<true>"]
 KERNEL_FUNCS["k_window_split@batched"] = KERNEL_FUNCS["k_window_split"]
 KERNEL_FUNCS["k_window_cluster"] = ["cl_rsqrt", "k_window_cluster"]
+# FP64 plans: on chip (one cluster per instance), one pass over the grid, or two phases.
+FP64_WINDOW = "k_window_onchip / k_window_fx / k_window_2ph<false>"
 PROFILED_TRAFFIC = {
     "k_window_fused": ("123b4a784de2ee96", 329.5e6, "profiles/k_window_fused_tise_2e_16sd.md"),
-    "k_window_2ph<false>": ("6fd9a352bcfedf25", 279.0e6, "profiles/k_window_2ph_fp64_tise_2e_16sd.md"),
     "k_window_2ph<true>@batched": ("cbd72ea8633a4ed0", 1.192, "profiles/k_window_2ph_df32_batched_uneven.md"),
     "k_window_split@batched": ("e908166e69fb5910", 1.030, "profiles/k_window_split_batched_uneven.md"),
     # the captured launch is a 1723-step window; the traffic is the history rows and
@@ -447,6 +447,11 @@ def extra_batched(args, env):
                     "is set up, assembled and autotuned untimed); step matrices stream from HBM"}
 
 
+# Real time: the persistent fixed-point window, or the host-launched sweeps of the
+# FP32-rounded matrices.
+RT_KERNEL = {"fp32": "k_cmv_df32 + Crank-Nicolson element-wise kernels"}
+
+
 def extra_real_time(args, env):
     """Bounded measurement of the 64-subdomain real-time workload (K = 1024
     complex, 1000 Crank-Nicolson steps): one warm-up and one timed Schwarz
@@ -475,12 +480,12 @@ def extra_real_time(args, env):
                    "ms_per_schwarz_iteration": ms, "window_ms": w_ms, "fp32_matrices": rep.fp32_matrices,
                    "norm2": float(s.norm2()[0]), "dipole": float(s.dipole()[0]),
                    "tensor_contractions": s.window_plan()["tensor_contractions"],
-                   "roofline": {"kernel": "k_cmv_df32 + Crank-Nicolson element-wise kernels" if pn != "fp64"
-                                else "k_cmv + Crank-Nicolson element-wise kernels", "bound": "hbm",
+                   "roofline": {"kernel": RT_KERNEL.get(pn, "k_rt_window"), "bound": "hbm",
                                 "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                                 "peak_source": src,
-                                "algorithmic": "step-matrix bytes per complex element (16 double-single or FP64, 8 "
-                                               "FP32-rounded) per sweep, (1 + m) sweeps per step"}}
+                                "algorithmic": "8 bytes per complex element of the symmetric step matrix (its lower "
+                                               "triangle in fixed point, or FP32-rounded) per sweep, 16 "
+                                               "double-single, (1 + m) sweeps per step"}}
         s.close()
     out[args.precision]["speedup_vs_fp64"] = out[args.precision]["value"] / out["fp64"]["value"]
     out["note"] = "second Schwarz iteration (the first is the warm-up), 1000 Crank-Nicolson steps, L2 flushed"
@@ -847,15 +852,19 @@ def main():
     bpe = {"mixed": "8 bytes (FP32 hi/lo pair)", "fp64": "8 bytes (FP64)",
            "fp32": "4 bytes (FP32-rounded, hi plane) before the switch to the refinement, 8 after"}[args.precision]
     if inst.mode == "tdse":
-        kname = {"fp64": "k_cmv"}.get(args.precision, "k_cmv_df32") + " + Crank-Nicolson element-wise kernels"
-        alg = (f"2 x {bpe} of G0 per complex element and sweep, (1 + m) sweeps per Crank-Nicolson step; "
-               "G0 (1.07 GB) does not fit in L2")
-        alu = {"achieved": tflops, "peak": FP64_PEAK_TFLOPS if args.precision == "fp64" else FP32_PEAK_TFLOPS / 6.0,
+        kname = RT_KERNEL.get(args.precision, "k_rt_window")
+        if args.precision == "fp32":
+            alg = (f"2 x {bpe} of G0 per complex element and sweep, (1 + m) sweeps per Crank-Nicolson step; "
+                   "G0 (1.07 GB) does not fit in L2")
+        else:
+            alg = ("8 bytes of the symmetric G0 per complex element and sweep (its lower triangle, 28 + 28 bits per "
+                   "component), (1 + m) sweeps per Crank-Nicolson step; the kernel is bound by its integer products")
+        alu = {"achieved": tflops, "peak": FP32_PEAK_TFLOPS / 6.0 if args.precision == "fp32" else FIXED_PEAK_TFLOPS,
                "unit": "TFLOP/s", "algorithmic": "8 K^2 FP64-equivalent flops per complex sweep"}
     else:
         kname = {S.WINDOW_FUSED: "k_window_fused", S.WINDOW_SPLIT: "k_window_split",
                  S.WINDOW_RESIDENT: "k_window_resident", S.WINDOW_CLUSTER: "k_window_cluster"}.get(
-            main_run["plan"]["variant"], "k_window_2ph<true>" if args.precision != "fp64" else "k_window_2ph<false>")
+            main_run["plan"]["variant"], "k_window_2ph<true>" if args.precision != "fp64" else FP64_WINDOW)
         if kname == "k_window_cluster":
             alg = (f"{bpe} of the step-matrix inverse per element, K^2 elements per local step solve (the "
                    "factor-apply); the cluster window keeps every subdomain's 2.65 MB of step matrix on chip "
@@ -865,9 +874,10 @@ def main():
             alg = (f"{bpe} of the step-matrix inverse per element, K^2 elements per local step solve (the "
                    "factor-apply); the 2-electron workload's 42.5 MB of step matrices stay in L2, so the kernel is "
                    "bounded by its per-step grid barrier and L2 latency, not by HBM")
-        alu = {"achieved": tflops, "peak": FP64_PEAK_TFLOPS if args.precision == "fp64" else FP32_PEAK_TFLOPS / 6.0,
+        alu = {"achieved": tflops, "peak": FIXED_PEAK_TFLOPS if args.precision == "fp64" else FP32_PEAK_TFLOPS / 6.0,
                "unit": "TFLOP/s", "algorithmic": "2 K^2 FP64-equivalent flops per local step solve",
-               "peak_source": "FP64 FMA rate (1.01 TFLOP/s) or FP32 FMA rate / 6 (67.7 TFLOP/s / 6: a double-single "
+               "peak_source": "56-bit fixed-point products on the integer pipes (2.6 TFLOP/s FP64-equivalent; the FP64 "
+                              "FMA rate is 1.01 TFLOP/s) or FP32 FMA rate / 6 (67.7 TFLOP/s / 6: a double-single "
                               "product-sum spends 12 FP32 operations per 2 FP64-equivalent flops), measured on this "
                               "pool's GB300 with independent FMA chains"}
     roof = {"kernel": kname, "bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,

@@ -55,13 +55,14 @@ typedef enum swr_mode {
 } swr_mode;
 
 typedef enum swr_precision {
-    SWR_PREC_FP64 = 0,   /* plain FP64 everywhere                                */
-    SWR_PREC_MIXED = 1,  /* step matrices stored as FP32 hi/lo pairs (four planes for
-                            the complex real-time G0) with error-free FP32
-                            accumulation: FP64-level accuracy on the FP32 pipes;
-                            FP64 reductions, norms, orthogonalisation, inversion.
-                            Real time runs the same fixed-point window as
-                            SWR_PREC_FP64 (56-bit matrices and vectors)          */
+    SWR_PREC_FP64 = 0,   /* FP64; the products with the step matrices in 56-bit fixed
+                            point (matrix rows and vectors scaled by powers of two,
+                            exact integer sums): FP64 accuracy on the integer pipes */
+    SWR_PREC_MIXED = 1,  /* imaginary time: step matrices stored as FP32 hi/lo pairs
+                            with error-free FP32 accumulation: FP64-level accuracy
+                            on the FP32 pipes; FP64 reductions, norms,
+                            orthogonalisation.  Real time runs the same fixed-point
+                            window as SWR_PREC_FP64 (56-bit matrices and vectors)  */
     SWR_PREC_FP32_REFINED = 2 /* the Schwarz iterations first run with the step
                             matrices rounded to FP32 (only the hi plane of
                             SWR_PREC_MIXED is read: 4 bytes per real element, 8
@@ -94,7 +95,9 @@ typedef enum swr_launch_mode {
 typedef enum swr_window_variant {
     SWR_WINDOW_AUTO = 0,       /* mixed precision: cluster when it fits (and no
                                   row target is given), else fused when it fits,
-                                  else split; FP64: two-phase                    */
+                                  else split; FP64: two-phase, as one cluster per
+                                  instance on chip or as one pass over G and W =
+                                  (Pp (x) Pp) G per step where these fit          */
     SWR_WINDOW_TWO_PHASE = 1,  /* y = G v, grid barrier, z = (Pp (x) Pp) y, grid
                                   barrier: G read once per step (8 bytes per
                                   element in both precisions); any batch size
@@ -141,7 +144,8 @@ typedef enum swr_window_variant {
  * local Hamiltonians (Sec. 5.1: B^T diag(w V_ee) B, sum-factorised into two
  * products per subdomain) and the rank-32 trailing updates of the blocked
  * Gauss-Jordan inversion of the step matrices (Sec. 5.4 step 2: the local
- * systems I + dt H' and I + i dt/2 H').  Either in FP64 on the FP64 pipe, or
+ * systems I + dt H' and I + i dt/2 H').  Either on the integer pipes in 56-bit
+ * fixed point (FP64 on the FP64 pipe for a batch of imaginary-time instances), or
  * on the 5th-generation tensor cores with FP64 emulated by exact BF16 slices:
  * every operand row / column scaled by a power of two and cut into integer
  * slices that BF16 holds exactly (9 slices of 7 bits for the inversion's
