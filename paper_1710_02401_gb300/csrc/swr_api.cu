@@ -418,6 +418,15 @@ static void plan_tasks(swr_ctx* c, int target_rows, int ctas, bool by_bytes = fa
     // whole GPU after the others have stopped
     const int nt = (int)c->tasks.size();
     const int g = nt < ctas ? nt : ctas;
+    if (nt <= ctas) {  // one each, in order
+        c->grid = g;
+        c->cta_list.resize(nt);
+        c->cta_task0.resize(nt + 1);
+        for (int t = 0; t < nt; ++t) c->cta_list[t] = c->cta_task0[t] = t;
+        c->cta_task0[nt] = nt;
+        c->tasks_per_cta = 1;
+        return;
+    }
     typedef std::pair<double, int> Load;
     std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
     for (int b = 0; b < g; ++b) heap.push(Load(0.0, b));
@@ -582,9 +591,9 @@ static bool plan_window(swr_ctx* c, int variant_req, int rows_req, bool have_dev
     // subdomain), else the fused, split or two-phase window below
     if (variant_req == 0 && rows_req == 0 && plan_cluster(c, 0, have_dev)) return true;
     for (int per_sm = 2; per_sm >= 1; --per_sm) {
-        plan_tasks(c, rows_req, per_sm * nsm, variant_req == WIN_SPLIT);
-        if (variant_req == 0 && c->df32 && !c->tdse && !c->has_w)
-            plan_tasks(c, rows_req == 0 && c->inst.size() == 1 ? one_wave_rows(c, per_sm * nsm) : rows_req, per_sm * nsm, true);
+        const bool auto_split = variant_req == 0 && c->df32 && !c->tdse && !c->has_w;
+        plan_tasks(c, auto_split && rows_req == 0 && c->inst.size() == 1 ? one_wave_rows(c, per_sm * nsm) : rows_req,
+                   per_sm * nsm, auto_split || variant_req == WIN_SPLIT);
         const bool fits = c->tasks_per_cta <= window_tasks_per_cta_max() && c->max_rows <= window_rows_per_task_max() &&
                           window_smem(c->max_K, c->max_kd, c->max_rows, c->tasks_per_cta, 0) <= WIN_SMEM_TASKS_MAX;
         int variant = variant_req;
@@ -912,8 +921,11 @@ static bool plan_for_device(swr_ctx* c, const swr_problem* p) {
         c->nsm = 152;
     }
     plan(c);  // descriptors and arena
-    // automatic: the tensor-core contractions where they measured faster, when
-    // every subdomain has K >= 768 (K = 1024: 1.8x the FP64 assembly; K = 576: 0.8x)
+    // automatic: the tensor-core contractions when every subdomain has K >= 768, where
+    // they were 1.8x the FP64 assembly.  In fixed point the other path is the faster
+    // one at every size tried (16 subdomains of K = 1024: 15 ms against 44, 64 complex
+    // ones: 91 against 410); callers select it with SWR_CONTRACT_FP64, the automatic
+    // choice is what the reported plan has always been
     bool all_large = !c->sub.empty();
     for (const SubDev& sd : c->sub) all_large = all_large && sd.K >= 768;
     c->use_tg = p->contraction_path == SWR_CONTRACT_TENSOR || (p->contraction_path == SWR_CONTRACT_AUTO && all_large);
@@ -1190,6 +1202,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     c->counters[6] += ams;
     c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 3) : 0) +
                       (c->tg ? 5 : 3) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
+                      (!c->tg && (c->tdse || c->inst.size() == 1) ? 1 : 0) +
                       (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (!c->df32 && !c->tdse ? (c->w1 ? 2 : 1) : 0);
     c->assembled = true;
     c->k = 0;

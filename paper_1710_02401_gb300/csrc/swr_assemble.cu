@@ -472,7 +472,7 @@ __global__ void k_ee_operands(SwrDeviceView v) {
 // of 32: one in six holds such a molecule), and the results of the other kernels
 // are kept as they are bit for bit.  One instance takes the fixed point (16
 // subdomains of K = 576: 4.3 ms of products and elimination, 12.3 in FP64).
-static inline bool fp64_batch(const SwrDeviceView& v) { return v.n_inst > 1; }
+__host__ __device__ static inline bool fp64_batch(const SwrDeviceView& v) { return v.n_inst > 1; }
 
 // Batched GEMM  C = op(A) * B  of FP64 matrices with 64x64 tiles, in 56-bit fixed
 // point on the integer pipes (swr_fixed.cuh: 4.5 multiply-adds per clock and SM
@@ -901,7 +901,7 @@ __device__ inline void gj_product64(const double (*A)[GJ_NB + 1], const double (
 // column block Cp = M[:, kb] of the same index range, by GJ_T columns per CTA
 // (one CTA doing all of it took 180 us of a 276 us panel at K = 576, 16 us here).
 template <typename T, bool FX>
-__global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
+__global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb, int sym) {
     constexpr int P = GjParts<T>::v;
     const SubDev& s = v.sub[blockIdx.y];
     const int K = s.K, k0 = kb * GJ_NB, tn = blockIdx.x * GJ_T;
@@ -929,7 +929,10 @@ __global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         const int e = tid + 256 * u, t = e / GJ_T, j = e % GJ_T;
-        mb[u] = t < nb && tn + j < K ? ld_el<T>(M, (long long)(k0 + t) * K + tn + j) : zero_el(T());
+        const bool up = sym && tn + j >= k0 + nb;  // not stored: its transpose (eliminated last)
+        mb[u] = t < nb && tn + j < K
+                    ? ld_el<T>(M, up ? (long long)(tn + j) * K + k0 + t : (long long)(k0 + t) * K + tn + j)
+                    : zero_el(T());
         atomicMax(&eb[j], gj_exp(mb[u]));
     }
     __syncthreads();
@@ -960,25 +963,27 @@ __global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb) {
         }
     for (int e = tid; e < GJ_T * nb; e += 256) {
         const int i = tn + e / nb, t = e % nb;
-        if (i < K) st_el<T>(Cp, (long long)i * GJ_NB + t, ld_el<T>(M, (long long)i * K + k0 + t));
+        if (i < K)
+            st_el<T>(Cp, (long long)i * GJ_NB + t,
+                     sym && i < k0 ? neg(ld_el<T>(M, (long long)(k0 + t) * K + i)) : ld_el<T>(M, (long long)i * K + k0 + t));
     }
 }
 
 // Rank-nb update of the whole matrix for block column kb (TILE x TILE tiles: 64 for
 // real, 32 for complex data: larger ones spill).  K = 576, 16 subdomains: 321 us
-// per block column in FP64, 131 here, bound by the integer products (4.5
-// multiply-adds per clock and SM).
+// per block column in FP64, 131 in fixed point, bound by the integer products (4.5
+// multiply-adds per clock and SM), 86 for the lower triangle only.
 template <typename T> struct GjTile { static const int v = 64; };
 template <> struct GjTile<cplx> { static const int v = 32; };
 
 template <typename T, bool FX>
-__global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb) {
+__global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb, int sym) {
     constexpr int TL = GjTile<T>::v, P = GjParts<T>::v, N = TL * GJ_NB / 256, Q = TL / 16;
     const SubDev& s = v.sub[blockIdx.z];
     const int K = s.K, k0 = kb * GJ_NB;
     if (k0 >= K) return;
     const int tm = blockIdx.y * TL, tn = blockIdx.x * TL;
-    if (tm >= K || tn >= K) return;
+    if (tm >= K || tn >= K || (sym && tn > tm)) return;
     const int nb = min(GJ_NB, K - k0), tid = threadIdx.x;
     double* M = v.arena + s.Gm;
     const double* Pinv = v.arena + s.work;
@@ -1033,8 +1038,30 @@ __global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb) {
         }
 }
 
+// Upper triangle of the inverse from its lower one (symmetric elimination).
+template <typename T>
+__global__ void k_gj_mirror(SwrDeviceView v) {
+    const SubDev& s = v.sub[blockIdx.z];
+    const int K = s.K, r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (r0 >= K || c0 > r0) return;
+    double* M = v.arena + s.Gm;
+    __shared__ T t[32][33];
+    for (int i = w; i < 32; i += 8)
+        if (r0 + i < K && c0 + lane < K) t[i][lane] = ld_el<T>(M, (long long)(r0 + i) * K + c0 + lane);
+    __syncthreads();
+    for (int i = w; i < 32; i += 8) {
+        const int r = c0 + i, c = r0 + lane;
+        if (c > r && c < K) st_el<T>(M, (long long)r * K + c, t[lane][i]);
+    }
+}
+
+// Fixed point: the step matrices are symmetric (k_symmetrize), so only tiles on and
+// under the diagonal are updated: with p eliminated and u remaining indices, M[p, u]
+// = -M[u, p]^T, the other two blocks are symmetric.  K = 576, 16 subdomains: 131 -> 86
+// us per block column; the other half follows the last one (k_gj_mirror).
 template <typename T, bool FX>
 static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int max_K, bool update) {
+    const int sym = FX && update;
     constexpr int TL = GjTile<T>::v, P = GjParts<T>::v;
     const size_t sr = P * (GJ_NB * (GJ_NB + 1) + GJ_NB * (GJ_T + 1)) * sizeof(int2);
     const size_t su = P * (TL * (GJ_NB + 1) + GJ_NB * (TL + 1)) * sizeof(int2);
@@ -1042,8 +1069,10 @@ static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gj_update<T, FX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)su);
     if (e != cudaSuccess) return e;
     k_gj_panel<T><<<v.n_sub, 256, 0, st>>>(v, kb);
-    k_gj_rows<T, FX><<<dim3((max_K + GJ_T - 1) / GJ_T, v.n_sub), 256, sr, st>>>(v, kb);
-    if (update) k_gj_update<T, FX><<<dim3((max_K + TL - 1) / TL, (max_K + TL - 1) / TL, v.n_sub), 256, su, st>>>(v, kb);
+    k_gj_rows<T, FX><<<dim3((max_K + GJ_T - 1) / GJ_T, v.n_sub), 256, sr, st>>>(v, kb, sym);
+    if (update) k_gj_update<T, FX><<<dim3((max_K + TL - 1) / TL, (max_K + TL - 1) / TL, v.n_sub), 256, su, st>>>(v, kb, sym);
+    if (sym && (kb + 1) * GJ_NB >= max_K)
+        k_gj_mirror<T><<<dim3((max_K + 31) / 32, (max_K + 31) / 32, v.n_sub), 256, 0, st>>>(v);
     return cudaGetLastError();
 }
 
@@ -1053,7 +1082,7 @@ static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int
 // (projection of Sec. 6.1 in the orthonormal basis: c' = X^T c~).
 // out[sid] = partial PoU norm^2 of c0 (later summed per instance).  The node values
 // are formed once per coordinate (in every coefficient's own sum: 430 us at kd =
-// 24, q = 132).
+// 24, q = 132) and the norm is summed over the block (216 us by one thread).
 __global__ void k_project(SwrDeviceView v, double* norm_part) {
     const int sid = blockIdx.x;
     const SubDev& s = v.sub[sid];
@@ -1063,6 +1092,8 @@ __global__ void k_project(SwrDeviceView v, double* norm_part) {
     __shared__ double u[2][ORTH_MAX_KD * 4];
     __shared__ double nrm[2];
     __shared__ double f[384];               // w exp(-gamma (x - x0)^2) at the nodes (q <= 384)
+    __shared__ double pu[ORTH_MAX_KD * 4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int d = 0; d < s.N; ++d) {
         const double* T = v.arena + s.t1[d];
         for (int n = threadIdx.x; n < q; n += blockDim.x) {
@@ -1077,10 +1108,23 @@ __global__ void k_project(SwrDeviceView v, double* norm_part) {
             u[d][a] = acc;
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (!fp64_batch(v)) {  // rows of the quadratic form, then their sum, over lanes
+            for (int a = warp; a < kd; a += nw) {
+                double acc = 0;
+                for (int c = lane; c < kd; c += 32) acc += T[lay.mat(M_PP) + a * kd + c] * u[d][c];
+                acc = warp_sum(acc);
+                if (lane == 0) pu[a] = u[d][a] * acc;
+            }
+            __syncthreads();
+            if (warp == 0) {
+                double acc = 0;
+                for (int a = lane; a < kd; a += 32) acc += pu[a];
+                acc = warp_sum(acc);
+                if (lane == 0) nrm[d] = acc;
+            }
+        } else if (threadIdx.x == 0) {
             double acc = 0;
             for (int a = 0; a < kd; ++a)
-#pragma unroll 4
                 for (int c = 0; c < kd; ++c) acc += u[d][a] * T[lay.mat(M_PP) + a * kd + c] * u[d][c];
             nrm[d] = acc;
         }
