@@ -1006,10 +1006,10 @@ __global__ void __launch_bounds__(WIN_THREADS, 2) k_window_fused(SweepArgs A) {
 // G and W = (Pp (x) Pp) G in 56-bit fixed point (k_fx_rows).  The two-phase
 // window spends most of its step in two barriers and in the FP64 chains of z =
 // (Pp (x) Pp) y between them; reading W as well costs 8 more bytes per element,
-// which pays while both matrices stay in L2 (the plan's rule).  Bound by the
-// integer multiply-adds (4.5 per clock and SM, 8 us of a step below) and the L2
-// reads of both matrices.  16 subdomains of K = 576: 18.8 us per step, 32.2
-// two-phase.
+// which pays while both matrices stay in L2 (the plan's rule).  The integer
+// products take 8 us of a step, L2 and the barrier with its FP64 sums the rest.
+// 16 subdomains of K = 576: 18.8 us per step, 32.2 two-phase.  Loading a batch of
+// columns ahead of the products gained nothing.
 
 // Rows [rb, rb + nrow), nrow <= 4, of y = G v and z = W v: lanes over the columns,
 // the eight exact sums transposed over the lanes on the way, lane 4 k gets sum k.
