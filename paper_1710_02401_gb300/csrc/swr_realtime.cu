@@ -50,9 +50,13 @@
 // in registers over a block column.  Integer sums are exact, so partial results
 // may be added in any order.
 //
-// Every wait of a bulk copy is bounded; a CTA that gives up raises
-// SWR_ERR_TIMEOUT and tells its cluster through the norm exchange, after which
-// all leave together.
+// Every wait of a bulk copy is bounded: spin_limit / 16 polls, since a poll
+// suspends for about 16 polls of an ordinary flag.  A warp that gives up raises
+// SWR_ERR_TIMEOUT, reads no further stage and issues no further copy, and its CTA
+// tells the cluster through the norm exchange, after which all leave together,
+// each once its own copies in flight have landed (a wait that does not follow the
+// caller's limit: a CTA must not exit while a copy still writes its shared
+// memory, and a copy of 8 KB completes within microseconds).
 #include <math.h>
 
 #include "swr_fixed.cuh"
@@ -279,7 +283,8 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rt_window(RtArgs A) {
         dp = reinterpret_cast<double2*>(v.arena + A.boff[3 * sid + 2]) + ra;
     }
     const unsigned char* G = reinterpret_cast<const unsigned char*>(v.arena + s.Gm);
-    const long long limit = A.spin_limit;
+    const long long limit = A.spin_limit >> 4;
+    const long long copy_limit = limit > (1LL << 20) ? limit : (1LL << 20);
 
     // ------------------------------------------------------------ the ring
     const int nt = T * (T + 1) / 2, t0 = (int)((long long)nt * rank / CS), t1 = (int)((long long)nt * (rank + 1) / CS);
@@ -308,7 +313,6 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rt_window(RtArgs A) {
         cp = ld;
     }
     unsigned qload = 0, qcomp = 0;
-    bool ok = true;
     // strip w of the tile under the load cursor into the next stage
     auto issue = [&]() {
         const unsigned st = qload % nst, bar = rt_smem(&s_bar[warp][st]);
@@ -445,10 +449,10 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rt_window(RtArgs A) {
                     cs[3 * j] = cs[3 * j + 1] = cs[3 * j + 2] = 0;
                 }
             }
-            if (ok && !rt_wait(rt_smem(&s_bar[warp][st]), par, limit)) {
-                ok = false;
+            if (!__all_sync(0xffffffffu, rt_wait(rt_smem(&s_bar[warp][st]), par, limit))) {
                 s_fail = 1;
-                atomicOr(v.err, SWR_ERR_TIMEOUT);
+                if (lane == 0) atomicOr(v.err, SWR_ERR_TIMEOUT);
+                break;
             }
             const int4* g = reinterpret_cast<const int4*>(ring + (size_t)st * RT_CHUNK) + lc;
             const int rr0 = warp * RT_S + lr * RT_LR;
@@ -603,7 +607,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rt_window(RtArgs A) {
         }
     }
     // copies in flight (the next sweep's first chunks) before the CTA leaves
-    for (unsigned q = resident ? 0u : qcomp; q < qload; ++q) rt_wait(rt_smem(&s_bar[warp][q % nst]), (q / nst) & 1u, limit);
+    for (unsigned q = resident ? 0u : qcomp; q < qload; ++q) rt_wait(rt_smem(&s_bar[warp][q % nst]), (q / nst) & 1u, copy_limit);
     if (rank == 0 && tid == 0) A.sweeps[sid] = nsweeps;
 }
 

@@ -90,6 +90,37 @@ def test_barrier_timeout_is_reported_and_the_context_recovers(S, precision, vari
     np.testing.assert_array_equal(s.energy(), want_e)
 
 
+@pytest.mark.parametrize("inst", [
+    P.small_tdse_2d(n_steps=6),                                     # matrices kept on chip
+    P.small_tdse_2d(L=2, K_d=32, q_p=32, n_mid=2, n_steps=4)],      # K = 1024: chunks streamed in every sweep
+    ids=["on-chip", "streamed"])
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("polls", [1, 15])
+def test_real_time_timeout_is_reported_and_the_context_recovers(S, inst, precision, polls):
+    # the waits for bulk copies suspend, so a limit below 16 polls of a flag is no poll of
+    # theirs: the first sweep gives up, with copies in flight, and the copies land
+    # before the kernel ends
+    ref = S.SWR(inst, precision=precision, contraction_path=S.CONTRACT_FP64)
+    ref.assemble()
+    ref.step()
+    ref.step()
+    want_res, want_psi = ref.residual().copy(), ref.get(S.FIELD_PSI_NODES).copy()
+
+    s = S.SWR(inst, precision=precision, contraction_path=S.CONTRACT_FP64)
+    s.assemble()
+    s.step()
+    ckpt = s.traces_get()
+    s.set_spin_limit(polls)
+    with pytest.raises(S.SWRError) as e:
+        s.step()
+    assert e.value.status == S.SWR_ETIMEOUT
+    s.set_spin_limit(0)
+    s.traces_set(ckpt)
+    s.step()
+    np.testing.assert_array_equal(s.residual(), want_res)
+    np.testing.assert_array_equal(s.get(S.FIELD_PSI_NODES), want_psi)
+
+
 def test_timeout_limit_is_validated(S):
     with pytest.raises(S.SWRError) as e:
         S.SWR(P.small_tise_2d(), spin_limit=-1)
