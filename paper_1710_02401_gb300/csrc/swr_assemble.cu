@@ -1234,7 +1234,8 @@ cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, 
     k_tabulate<<<g2, 256, 0, st>>>(v);
     k_mat1d<<<g2, 256, 0, st>>>(v);
     size_t sm = (2 * (size_t)max_kd * max_kd + 8 * (size_t)max_kd) * sizeof(double);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_orth, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t eo = allow_dynamic_smem((const void*)k_orth);
+    if (eo != cudaSuccess) return eo;
     k_orth<<<g2, 256, sm, st>>>(v);
     if (any_ee) {
         k_ee_operands<<<dim3(v.n_sub, 16), 256, 0, st>>>(v);

@@ -600,8 +600,8 @@ int cluster_tmem_cols(int kmax, int rows_max, int hs) {
     return cols <= 512 ? cols : 0;
 }
 
-static cudaError_t cluster_config(const void* f, size_t smem, int cs) {
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+static cudaError_t cluster_config(const void* f, int cs) {
+    cudaError_t e = allow_dynamic_smem(f);
     if (e == cudaSuccess && cs > 8) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
@@ -613,7 +613,7 @@ cudaError_t cluster_occupancy(int* clusters, int rows_max, size_t smem, int cs, 
     for (int o = 0; o < 2; ++o) {
         const void* f = cluster_kernel(rows_max, o == 1);
         if (!f) return cudaErrorInvalidValue;
-        cudaError_t e = cluster_config(f, smem, cs);
+        cudaError_t e = cluster_config(f, cs);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
@@ -638,7 +638,7 @@ cudaError_t cluster_occupancy(int* clusters, int rows_max, size_t smem, int cs, 
 cudaError_t launch_cluster_window(SweepArgs& a, int grid, int cs, size_t smem, cudaStream_t st, bool onep) {
     const void* f = cluster_kernel(a.rows_max, onep);
     if (!f) return cudaErrorInvalidValue;
-    cudaError_t e = cluster_config(f, smem, cs);
+    cudaError_t e = cluster_config(f, cs);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];

@@ -259,6 +259,19 @@ struct TaskCache {
     double kdt, ngf_tol;
 };
 
+// Opens all of a CTA's shared memory beside kernel f's static arrays (227 KB in
+// all) to its launches.  The attribute belongs to the process, not to a context:
+// set to what one problem needs, it would be lowered under another context, in
+// another thread between its own setting and its launch.
+static inline cudaError_t allow_dynamic_smem(const void* f) {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, f);
+    const int most = 227 * 1024 - (int)a.sharedSizeBytes;
+    if (e == cudaSuccess && a.maxDynamicSharedSizeBytes != most)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e;
+}
+
 // Window kernel variants.
 // (WIN_FX: the FP64 one-pass kernel of the automatic two-phase plan, not requested by number.)
 enum WindowVariant { WIN_TWO_PHASE = 1, WIN_FUSED = 2, WIN_SPLIT = 3, WIN_RESIDENT = 4, WIN_CLUSTER = 5, WIN_FX = 6 };

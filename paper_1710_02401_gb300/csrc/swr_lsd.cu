@@ -791,7 +791,7 @@ extern "C" swr_status swr_lsd_build(const swr_lsd_problem* p, swr_lsd_result* ou
         k_lsd_nodes<<<(nn + 255) / 256, 256>>>(db.at<double>(o_edges), db.at<int>(o_ebase), np, dt, dw, p->q_p, dx, dwx);
         const int nt = 256;
         const size_t smem = (4 * (size_t)n * n + 64) * sizeof(double);
-        LSD_CU(cudaFuncSetAttribute(k_lsd_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        LSD_CU(allow_dynamic_smem((const void*)k_lsd_local));
         k_lsd_local_tab<<<dim3((nn_max * (p->kd + 1) + 255) / 256, p->L), 256>>>(d, dx, dwx, dnbase, db.at<double>(o_gtab));
         k_lsd_local_mat<<<dim3((p->kd * (p->kd + 1) + 7) / 8, p->L), 256>>>(d, dnbase, db.at<double>(o_gtab),
                                                                            db.at<double>(o_mat));

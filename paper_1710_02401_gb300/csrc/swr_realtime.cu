@@ -675,7 +675,7 @@ bool rt_plan(int n_sub, int kmax, int qel, RtPlan* out) {
 cudaError_t launch_rt_pack(const SwrDeviceView& v, cudaStream_t st, int max_K) {
     const int T = (max_K + RT_T - 1) / RT_T;
     const size_t smem = (size_t)T * RT_S * RT_T * sizeof(int4);
-    cudaError_t e = cudaFuncSetAttribute(k_rt_pack, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem((const void*)k_rt_pack);
     if (e != cudaSuccess) return e;
     k_rt_pack<<<dim3((unsigned)((max_K + RT_S - 1) / RT_S), v.n_sub), 256, smem, st>>>(v);
     return cudaGetLastError();

@@ -653,7 +653,7 @@ extern const int kStepLaunches = 8;
 // waves left the tail to the largest bases).  The kernels after the window of a
 // batch of 32 (1101 subdomains): 6.47 -> 4.81 ms at 60 steps, 12.1 -> 10.9 at 190.
 static cudaError_t step_blocks(const void* f, size_t smem, int n_sub, int nsm, unsigned* nb) {
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(f);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     int per_sm = 0;
@@ -729,7 +729,8 @@ size_t energy_smem(const SubDev& s) {
 cudaError_t launch_energy(const SwrDeviceView& v, cudaStream_t st, const int* d_win, const double* d_snorm,
                           int cap, double* d_part, double* d_energy, double* d_norm2, double* d_dipole,
                           double* psi_out, const long long* psi_off, size_t smem) {
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_dynamic_smem((const void*)k_energy);
+    if (e != cudaSuccess) return e;
     k_energy<<<dim3(ENERGY_BLOCKS, v.n_sub), 256, smem, st>>>(v, d_win, d_snorm, cap, d_part, psi_out, psi_off);
     k_energy_reduce<<<div_up(v.n_inst, 4), 128, 0, st>>>(v, d_part, d_energy, d_norm2, d_dipole);
     return cudaGetLastError();

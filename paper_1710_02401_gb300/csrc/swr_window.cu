@@ -2291,7 +2291,7 @@ cudaError_t window_occupancy(int* blocks_per_sm, size_t smem, int variant, bool 
     for (int o = 0; o < 2; ++o) {
         if (o == 1 && variant != WIN_FUSED && variant != WIN_SPLIT && variant != WIN_RESIDENT) break;
         const void* f = window_kernel(variant, df32, o == 1);
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_dynamic_smem(f);
         if (e != cudaSuccess) return e;
         int b = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, WIN_THREADS, smem);
@@ -2314,7 +2314,6 @@ cudaError_t launch_split_df32(const SwrDeviceView& v, cudaStream_t st, int max_K
     k_split_df32<<<dim3(gx, v.n_sub), 256, 0, st>>>(v);
     if (!make_w) return cudaGetLastError();
     size_t sm = ((size_t)max_K + 32 * 32) * sizeof(double);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_make_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     k_make_w<<<dim3(max_K < 512 ? max_K : 512, v.n_sub), 256, sm, st>>>(v);
     return cudaGetLastError();
 }
