@@ -98,6 +98,7 @@ struct swr_ctx {
     RtPlan rt_shape = {1, 1, 0};
     int qel = 0;                         // real time: elements of the largest subdomain's Q' factors
     unsigned* d_sweeps = nullptr;
+    int* d_gexp = nullptr;               // real time: exponent of every subdomain's G0
     std::vector<unsigned> sweeps_h;
     int* d_rtiles = nullptr;        // Robin response: first product tile of every subdomain
     double* d_dipole = nullptr;
@@ -843,7 +844,7 @@ static void plan(swr_ctx* c) {
 struct AuxPlan {
     size_t inst, sub, err, jobs1, jobs2, norm_part, tasks, task0, part_s, part_d, cta0, tc, scal, alive, own,
         ctal, wfix, snorm, sums_s, sums_d,
-        n_active, win, win_prev, bar, queue, qlist, clslots, cnneed, sweeps, ocb, ocr, rtiles, res_part, res, cv_part, cvtot, epart, energy, norm2, dipole, boff,
+        n_active, win, win_prev, bar, queue, qlist, clslots, cnneed, sweeps, gexp, ocb, ocr, rtiles, res_part, res, cv_part, cvtot, epart, energy, norm2, dipole, boff,
         psi, psi_off, tg, total;
 };
 static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -889,6 +890,7 @@ static AuxPlan aux_plan(const swr_ctx* c) {
     a.boff = o; o = al256(o + (c->boff.size() + 1) * sizeof(long long));
     a.cnneed = o; o = al256(o + c->cn_need.size() + 1);
     a.sweeps = o; o = al256(o + ns * sizeof(unsigned));
+    a.gexp = o; o = al256(o + ns * sizeof(int));
     a.ocb = o; o = al256(o + ni * 17 * sizeof(int));
     a.ocr = o; o = al256(o + ns * sizeof(int));
     a.rtiles = o; o = al256(o + (ns + 1) * sizeof(int));
@@ -1078,6 +1080,7 @@ extern "C" swr_status swr_setup(const swr_problem* p, swr_ctx** out) {
     c->d_boff = (long long*)(b + a.boff);
     c->d_cn_need = (unsigned char*)(b + a.cnneed);
     c->d_sweeps = (unsigned*)(b + a.sweeps);
+    c->d_gexp = (int*)(b + a.gexp);
     c->d_oc_bounds = (int*)(b + a.ocb);
     c->d_oc_row0 = (int*)(b + a.ocr);
     c->d_rtiles = (int*)(b + a.rtiles);
@@ -1189,7 +1192,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     CU(launch_assemble(view(c), c->stream, c->max_q, c->max_kd, c->max_K, c->any_ee, c->tdse, !c->tdse,
                        c->d_jobs1, c->d_jobs2, c->d_norm_part, c->tg));
     if (c->df32 && !c->tdse) CU(launch_split_df32(view(c), c->stream, c->max_K, c->has_w));
-    if (c->rt) CU(launch_rt_pack(view(c), c->stream, c->max_K));
+    if (c->rt) CU(launch_rt_pack(view(c), c->stream, c->max_K, c->d_gexp));
     else if (c->tdse) CU(launch_split_c_df32(view(c), c->stream, c->max_K));
     if (c->robin_w) CU(launch_robin_ge(view(c), c->stream, c->max_K, c->max_J));
     if (c->oc || c->w1) CU(launch_oc_make_w(view(c), c->stream, c->max_K));
@@ -1203,7 +1206,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 3) : 0) +
                       (c->tg ? 5 : 3) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
                       (!c->tg && (c->tdse || c->inst.size() == 1) ? 1 : 0) +
-                      (c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (!c->df32 && !c->tdse ? (c->w1 ? 2 : 1) : 0);
+                      (c->rt ? 2 : c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (!c->df32 && !c->tdse ? (c->w1 ? 2 : 1) : 0);
     c->assembled = true;
     c->k = 0;
     c->parity = 0;
@@ -1282,7 +1285,7 @@ static cudaError_t record_iteration(swr_ctx* c, cudaStream_t st, long long* win_
         if (e == cudaSuccess && c->rt) {
             *win_launches = 2;
             // (the normalisation factors' array holds the field: real time has none)
-            e = launch_rt_window(view(c), st, c->rt_shape, c->d_boff, c->d_win_prev, c->d_snorm, c->cap, c->d_sweeps,
+            e = launch_rt_window(view(c), st, c->rt_shape, c->d_boff, c->d_win_prev, c->d_snorm, c->cap, c->d_sweeps, c->d_gexp,
                                  c->max_K, c->qel, c->spin_limit);
         } else if (e == cudaSuccess) {
             e = launch_tdse_window(view(c), st, c->d_boff, c->d_win_prev, nmax, c->cn_need.data(), c->d_cn_need,

@@ -398,10 +398,10 @@ struct RtPlan {
     int cs, nst, own;
 };
 bool rt_plan(int n_sub, int kmax, int qel, RtPlan* out);
-cudaError_t launch_rt_pack(const SwrDeviceView& v, cudaStream_t st, int max_K);
+cudaError_t launch_rt_pack(const SwrDeviceView& v, cudaStream_t st, int max_K, int* d_gexp);
 cudaError_t launch_rt_window(const SwrDeviceView& v, cudaStream_t st, const RtPlan& plan, const long long* d_boff,
-                             const int* d_win_prev, double* d_theta, int cap, unsigned* d_sweeps, int max_K, int qel,
-                             long long spin_limit);
+                             const int* d_win_prev, double* d_theta, int cap, unsigned* d_sweeps, const int* d_gexp,
+                             int max_K, int qel, long long spin_limit);
 void set_error(swr_ctx* c, const char* msg);
 void set_setup_error(const char* msg);
 // Blocks per subdomain of the energy kernel (partials [n_sub][ENERGY_BLOCKS][3]).

@@ -118,6 +118,7 @@ struct RtArgs {
     const int* win_prev;
     const double* theta;      // [n_inst][cap + 1] dt/2 e(t_n)
     unsigned* sweeps;         // [n_sub] matrix sweeps of the window
+    const int* gexp;          // [n_sub] exponent of G0 (k_rt_scale)
     long long spin_limit;
     int cap, cs, kmax, qel, nst, own_smem;  // qel: elements of the Q' factors (both coordinates)
 };
@@ -137,20 +138,45 @@ __global__ void k_rt_theta(SwrDeviceView v, double* theta, int cap) {
     theta[(long long)blockIdx.y * (cap + 1) + n] = 0.5 * in.dt * e;
 }
 
-// Limbs of the lower triangle of G0 (|entries| <= 1: exponent 0), strip by strip
+// Exponent of a subdomain's G0: 2^(e - 1022) is the smallest power of two of
+// which no row's 2-norm exceeds sqrt(2) times (1 for the ||G0|| <= 1 of an
+// absorbing boundary with kinetic > 0; larger where G0 is, smaller where the
+// whole matrix is small), FX_BAD when an entry is not finite.  A warp per row.
+__global__ void k_rt_scale(SwrDeviceView v, int* gexp) {
+    const SubDev& s = v.sub[blockIdx.y];
+    const int K = s.K, lane = threadIdx.x & 31, r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    if (r >= K) return;
+    const double2* g = reinterpret_cast<const double2*>(v.arena + s.Gm) + (size_t)r * K;
+    int e = 0;
+    for (int c = lane; c < K; c += 32) e = max(e, max(fx_exp(g[c].x), fx_exp(g[c].y)));
+    e = __reduce_max_sync(0xffffffffu, e);
+    const double sc = e > 0 && e < 2045 ? __hiloint2double((2045 - e) << 20, 0) : 0.0;  // 2^(1022 - e)
+    float q = 0.f;
+    for (int c = lane; c < K; c += 32) {
+        const float a = (float)(g[c].x * sc), b = (float)(g[c].y * sc);
+        q += a * a + b * b;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    int x = -1;
+    while (x < 6 && 1.99f * ldexpf(1.f, 2 * x) <= q) ++x;  // (q <= 2 K)
+    if (lane == 0) atomicMax(gexp + blockIdx.y, e >= FX_BAD ? FX_BAD : max(e + x, 0));
+}
+
+// Limbs of the lower triangle of G0 relative to its exponent, strip by strip
 // in place through shared memory: columns of the chunk of block column J have
 // the pitch min(64, columns up to the strip's last row).
-__global__ void k_rt_pack(SwrDeviceView v) {
+__global__ void k_rt_pack(SwrDeviceView v, const int* gexp) {
     extern __shared__ int4 rt_strip[];
     const SubDev& s = v.sub[blockIdx.y];
-    const int K = s.K, r0 = blockIdx.x * RT_S;
+    const int K = s.K, r0 = blockIdx.x * RT_S, eg = gexp[blockIdx.y];
     if (r0 >= K) return;
     const int nr = min(RT_S, K - r0), nc = min(K, r0 + RT_S);  // columns kept of every row of the strip
     double2* G = reinterpret_cast<double2*>(v.arena + s.Gm) + (size_t)r0 * K;
     for (int e = threadIdx.x; e < nr * nc; e += blockDim.x) {
         const int i = e / nc, c = e - i * nc, J = c / RT_T, pitch = min(RT_T, nc - J * RT_T);
         const double2 g = G[(size_t)i * K + c];
-        const int2 a = fx_limbs(g.x, 1022), b = fx_limbs(g.y, 1022);
+        const int2 a = fx_limbs(g.x, eg), b = fx_limbs(g.y, eg);
         rt_strip[J * nr * RT_T + i * pitch + c - J * RT_T] = make_int4(a.x, a.y, b.x, b.y);
     }
     __syncthreads();
@@ -368,6 +394,7 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rt_window(RtArgs A) {
     const double* bvec = v.arena + s.bvec;
     const double* theta = A.theta + (long long)s.inst * (A.cap + 1);
     const double hk = 0.5 * in.dt * in.kappa;
+    const int eg = A.gexp[sid] - 1022;  // G0 = limbs x 2^(eg - 56)
     double qlo = 0, qhi = 0;
     for (int e = 0; e < s.N; ++e) {
         qlo += s.lo[e];
@@ -545,8 +572,8 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rt_window(RtArgs A) {
             ++nsweeps;
             rt_sync(CS);
             // ---- own rows of x_m, d_m = x_m - x_g and the norms of the stop test
-            const double unit = fx_unit(eu, 0), bad = eu == FX_BAD ? nan("") : 0.0;
-            const int en = 2045 - eu;  // scales the norms to the order of 1
+            const double unit = fx_unit(eu, eg), bad = eu == FX_BAD || eg >= FX_BAD - 1022 ? nan("") : 0.0;
+            const int en = 2045 - eu - eg;  // scales the norms to units of 2^56 sums
             const double inv = en > 0 && en < 0x7ff ? __hiloint2double(en << 20, 0) : 0.0;
             float nd = 0.f, nx = 0.f;
             for (int r = ra + tid; r < rb; r += RT_THREADS) {
@@ -672,25 +699,28 @@ bool rt_plan(int n_sub, int kmax, int qel, RtPlan* out) {
     return best < 1e300;
 }
 
-cudaError_t launch_rt_pack(const SwrDeviceView& v, cudaStream_t st, int max_K) {
+cudaError_t launch_rt_pack(const SwrDeviceView& v, cudaStream_t st, int max_K, int* d_gexp) {
     const int T = (max_K + RT_T - 1) / RT_T;
     const size_t smem = (size_t)T * RT_S * RT_T * sizeof(int4);
     cudaError_t e = allow_dynamic_smem((const void*)k_rt_pack);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_gexp, 0, v.n_sub * sizeof(int), st);
     if (e != cudaSuccess) return e;
-    k_rt_pack<<<dim3((unsigned)((max_K + RT_S - 1) / RT_S), v.n_sub), 256, smem, st>>>(v);
+    k_rt_scale<<<dim3((unsigned)((max_K + 7) / 8), v.n_sub), 256, 0, st>>>(v, d_gexp);
+    k_rt_pack<<<dim3((unsigned)((max_K + RT_S - 1) / RT_S), v.n_sub), 256, smem, st>>>(v, d_gexp);
     return cudaGetLastError();
 }
 
 // Two launches: the field of every step, the window.
 cudaError_t launch_rt_window(const SwrDeviceView& v, cudaStream_t st, const RtPlan& plan, const long long* d_boff,
-                             const int* d_win_prev, double* d_theta, int cap, unsigned* d_sweeps, int max_K, int qel,
-                             long long spin_limit) {
+                             const int* d_win_prev, double* d_theta, int cap, unsigned* d_sweeps, const int* d_gexp,
+                             int max_K, int qel, long long spin_limit) {
     RtArgs a;
     a.v = v;
     a.boff = d_boff;
     a.win_prev = d_win_prev;
     a.theta = d_theta;
     a.sweeps = d_sweeps;
+    a.gexp = d_gexp;
     a.spin_limit = spin_limit;
     a.cap = cap;
     a.cs = plan.cs;

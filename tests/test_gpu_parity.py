@@ -296,6 +296,15 @@ def test_parity_real_time_tile_edges(swr_mod, n_elec, L, K_d, precision):
     _compare(swr_mod, inst, kmax=2, precision=precision)
 
 
+@pytest.mark.parametrize("precision", [0, 1])
+def test_parity_real_time_where_the_inverse_exceeds_one(swr_mod, precision):
+    # kinetic < 0 turns the absorbing boundary into a source: entries of G0 up to 17.8
+    # instead of ||G0|| <= 1
+    inst = P.tise_1d_two_subdomains().replace(mode=P.TDSE, kinetic=-0.5, mu=-73.5j, dt=0.01, n_steps=3, ngf_tol=0.0,
+                                              K_d=20, delta=2.0)
+    _compare(swr_mod, inst, kmax=2, precision=precision)
+
+
 @pytest.mark.parametrize("inst", [
     P.tise_1d_two_subdomains().replace(K_d=3, delta=0.05, max_steps=60),    # 6 rows in all, one CTA
     P.small_tise_2d(L=2, K_d=16, q_p=16, n_mid=2, max_steps=60),            # K = 256, the largest
