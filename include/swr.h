@@ -145,8 +145,10 @@ typedef enum swr_window_variant {
  * products per subdomain) and the rank-32 trailing updates of the blocked
  * Gauss-Jordan inversion of the step matrices (Sec. 5.4 step 2: the local
  * systems I + dt H' and I + i dt/2 H').  Either on the integer pipes in 56-bit
- * fixed point (FP64 on the FP64 pipe for a batch of imaginary-time instances), or
- * on the 5th-generation tensor cores with FP64 emulated by exact BF16 slices:
+ * fixed point (FP64 on the FP64 pipe for an imaginary-time instance whose 1 + dt H'
+ * is not bounded below by 1/4: kinetic and mu terms count as 0, the potential at its
+ * deepest; where dt passes 1 / |E| of a local level the iteration amplifies
+ * rounding, whatever the arithmetic), or on the 5th-generation tensor cores with FP64 emulated by exact BF16 slices:
  * every operand row / column scaled by a power of two and cut into integer
  * slices that BF16 holds exactly (9 slices of 7 bits for the inversion's
  * 32-long inner products, 11 of 6 bits for the e-e products' inner length up
@@ -156,7 +158,7 @@ typedef enum swr_window_variant {
 typedef enum swr_contraction {
     SWR_CONTRACT_AUTO = 0,     /* tensor cores when every subdomain has K >= 768,
                                   else the integer / FP64 path                    */
-    SWR_CONTRACT_FP64 = 1,     /* fixed point on the integer pipes (batches: FP64);
+    SWR_CONTRACT_FP64 = 1,     /* fixed point on the integer pipes, or FP64;
                                   assembly of 64 complex subdomains of K = 1024
                                   91 ms against 410 on the tensor cores, of 16 real
                                   ones 15 against 44                              */

@@ -20,7 +20,7 @@
 namespace swr {
 struct TgState;
 cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, int max_kd, int max_K,
-                            bool any_ee, bool any_tdse, bool any_tise, const GemmJob* d_jobs1,
+                            bool any_ee, bool any_tdse, bool any_fx, bool any_64, const GemmJob* d_jobs1,
                             const GemmJob* d_jobs2, double* d_norm_part, const TgState* tg);
 size_t tg_scratch_bytes(const int* Ks, const int* qs, const int* kds, const int* nel, int n_sub, bool cplx_data,
                         bool any_ee);
@@ -52,6 +52,7 @@ size_t energy_smem(const SubDev& s);
 cudaError_t launch_tdse_window(const SwrDeviceView& v, cudaStream_t st, const long long* d_boff, const int* d_win_prev,
                                int n_steps, const unsigned char* h_need, const unsigned char* d_need, int max_K,
                                int max_kd, bool onep, long long* launches);
+bool assemble_fx(const InstDev& in);
 cudaError_t launch_split_c_df32(const SwrDeviceView& v, cudaStream_t st, int max_K);
 }  // namespace swr
 
@@ -90,6 +91,7 @@ struct swr_ctx {
     std::vector<unsigned char> cn_need;  // real time: fixed-point iterations [step][subdomain]
     std::vector<double> cn_sweeps;       // real time: matvecs with G0 per subdomain over the whole window
     unsigned char* d_cn_need = nullptr;
+    bool any_fx = false, any_64 = false; // instances assembled in fixed point, in FP64 (assemble_fx)
     bool oc = false;                     // FP64, automatic plan: on-chip window, one cluster per instance
     bool w1 = false;                     // FP64, automatic plan: one-pass grid window (k_window_fx)
     OcPlan oc_shape;
@@ -660,6 +662,7 @@ static void plan(swr_ctx* c) {
     c->tdse = p.instances[0].mode == SWR_MODE_TDSE;
     c->rt = c->tdse && p.precision != SWR_PREC_FP32_REFINED;
     c->qel = 0;
+    c->any_fx = c->any_64 = false;
     const int cx = c->tdse ? 2 : 1;
     for (int i = 0; i < p.n_instances; ++i) {
         const swr_instance& in = c->inst_h[i];
@@ -713,6 +716,8 @@ static void plan(swr_ctx* c) {
         d.x0[1] = in.phi0_center[1];
         d.orth_tau = in.orth_tau > 0.0 ? in.orth_tau : ORTH_TAU_DEFAULT;
         if (d.N == 2 && d.ee_coef != 0.0) c->any_ee = true;
+        d.fx = assemble_fx(d) ? 1 : 0;
+        (d.fx ? c->any_fx : c->any_64) = true;
         c->inst.push_back(d);
         c->inst_task0.push_back((int)c->tasks.size());
         for (int sidl = 0; sidl < d.n_sub; ++sidl) {
@@ -1189,7 +1194,7 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     if (!c) return fail(nullptr, SWR_EINVAL, "ctx is NULL");
     CU(cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream));
     CU(cudaEventRecord(c->ev0, c->stream));
-    CU(launch_assemble(view(c), c->stream, c->max_q, c->max_kd, c->max_K, c->any_ee, c->tdse, !c->tdse,
+    CU(launch_assemble(view(c), c->stream, c->max_q, c->max_kd, c->max_K, c->any_ee, c->tdse, c->any_fx, c->any_64,
                        c->d_jobs1, c->d_jobs2, c->d_norm_part, c->tg));
     if (c->df32 && !c->tdse) CU(launch_split_df32(view(c), c->stream, c->max_K, c->has_w));
     if (c->rt) CU(launch_rt_pack(view(c), c->stream, c->max_K, c->d_gexp));
@@ -1203,9 +1208,10 @@ extern "C" swr_status swr_assemble(swr_ctx* c) {
     float ams = 0;
     CU(cudaEventElapsedTime(&ams, c->ev0, c->ev1));
     c->counters[6] += ams;
-    c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 3) : 0) +
-                      (c->tg ? 5 : 3) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
-                      (!c->tg && (c->tdse || c->inst.size() == 1) ? 1 : 0) +
+    const int paths = (c->any_fx ? 1 : 0) + (c->any_64 ? 1 : 0);
+    c->counters[2] += kAssembleLaunchesFixed + (c->any_ee ? (c->tg ? 7 : 1 + 2 * paths) : 0) +
+                      (c->tg ? 4 + paths : 1 + 2 * paths) * ((c->max_K + GJ_NB_HOST - 1) / GJ_NB_HOST) +
+                      (!c->tg && c->any_fx ? 1 : 0) +
                       (c->rt ? 2 : c->tdse ? 1 : c->df32 ? (c->has_w ? 2 : 1) : 0) + (c->robin_w && c->max_J > 0 ? 1 : 0) + (!c->df32 && !c->tdse ? (c->w1 ? 2 : 1) : 0);
     c->assembled = true;
     c->k = 0;

@@ -466,13 +466,49 @@ __global__ void k_ee_operands(SwrDeviceView v) {
     }
 }
 
-// Assembly in fixed point or FP64: batches of instances stay in FP64.  A batch steps
-// every molecule with one dt; where dt passes 1 / |E| of one of them, its window
-// amplifies the last bits of the step matrix into leading digits (seeded batches
-// of 32: one in six holds such a molecule), and the results of the other kernels
-// are kept as they are bit for bit.  One instance takes the fixed point (16
-// subdomains of K = 576: 4.3 ms of products and elimination, 12.3 in FP64).
-__host__ __device__ static inline bool fp64_batch(const SwrDeviceView& v) { return v.n_inst > 1; }
+// Arithmetic of an instance's e-e products and elimination: fixed point where its
+// step matrices are safely positive definite, else FP64.  Where dt passes 1 / |E|
+// of a local level, 1 + dt E changes sign and the window amplifies the last bits of
+// the step matrix into leading digits; an elimination without pivots then also
+// meets pivots near zero.  The bound needs the parameters only: kinetic and Robin
+// terms are not negative, so 1 + dt H' >= 1 + dt (deepest potential), and with 1/4 at
+// least the inverse stays below 4.  Of 320 seeded molecules of the uneven batches
+// (200 steps each, alone) the two arithmetics differ by at most 9e-14 in psi, except
+// in three, by 3e-8 to 1.9: bounds -0.56, -0.78, -1.29.  201 of the 320 take the
+// fixed point.  Real time always does (a positive definite Hermitian part).  16
+// subdomains of K = 576: 4.3 ms of products and elimination, 12.3 in FP64.
+static const double FX_DEFINITE = 0.25;
+
+// Lower bound of the electron-nucleus and harmonic potential on the box, one electron.
+static double potential_floor(const InstDev& in) {
+    double lo = 1e300, hi = -1e300;
+    for (int a = 0; a < in.n_nuc; ++a)
+        if (in.Z_nuc[a] > 0.0) {
+            lo = fmin(lo, in.x_nuc[a]);
+            hi = fmax(hi, in.x_nuc[a]);
+        }
+    double deepest = 0.0;  // the attraction is deepest between the outermost nuclei: cell by cell, each at its nearest
+    const int cells = 64;
+    for (int k = 0; k < cells && lo <= hi; ++k) {
+        const double c0 = lo + (hi - lo) * k / cells, c1 = lo + (hi - lo) * (k + 1) / cells;
+        double v = 0.0;
+        for (int a = 0; a < in.n_nuc; ++a)
+            if (in.Z_nuc[a] > 0.0) {
+                const double r = fmax(0.0, fmax(c0 - in.x_nuc[a], in.x_nuc[a] - c1));
+                v -= in.Z_nuc[a] / sqrt(r * r + in.eta_en * in.eta_en);
+            }
+        if (!(v >= deepest)) deepest = v;
+    }
+    const double x = fmax(fabs(in.a - in.eps), fabs(in.b + in.eps));
+    return deepest + fmin(0.0, 0.5 * in.harmonic * x * x);
+}
+
+bool assemble_fx(const InstDev& in) {
+    if (in.mode == SWR_MODE_TDSE) return true;
+    if (!(in.kappa >= 0.0) || !(in.kappa * in.mu_re >= 0.0)) return false;
+    const double ee = in.ee_coef < 0.0 ? in.ee_coef / fabs(in.eta_ee) : 0.0;
+    return 1.0 + in.dt * (in.N * potential_floor(in) + ee) >= FX_DEFINITE;  // (false when not a number)
+}
 
 // Batched GEMM  C = op(A) * B  of FP64 matrices with 64x64 tiles, in 56-bit fixed
 // point on the integer pipes (swr_fixed.cuh: 4.5 multiply-adds per clock and SM
@@ -487,6 +523,7 @@ __host__ __device__ static inline bool fp64_batch(const SwrDeviceView& v) { retu
 #define GT 64
 #define GK 16
 __global__ void __launch_bounds__(256) k_fxgemm(SwrDeviceView v, const GemmJob* jobs) {
+    if (!v.inst[v.sub[blockIdx.z].inst].fx) return;
     const GemmJob jb = jobs[blockIdx.z];
     const int tm = blockIdx.y * GT, tn = blockIdx.x * GT;
     if (jb.M <= 0 || tm >= jb.M || tn >= jb.N) return;
@@ -580,8 +617,9 @@ __global__ void __launch_bounds__(256) k_fxgemm(SwrDeviceView v, const GemmJob* 
         }
 }
 
-// The same in FP64 (batches).
+// The same in FP64.
 __global__ void __launch_bounds__(256) k_dgemm(SwrDeviceView v, const GemmJob* jobs) {
+    if (v.inst[v.sub[blockIdx.z].inst].fx) return;
     const GemmJob jb = jobs[blockIdx.z];
     const int tm = blockIdx.y * GT, tn = blockIdx.x * GT;
     if (jb.M <= 0 || tm >= jb.M || tn >= jb.N) return;
@@ -822,7 +860,7 @@ __device__ inline int gj_exp(cplx x) { return max(fx_exp(x.re), fx_exp(x.im)); }
 __device__ inline double gj_make(const double* x, double) { return x[0]; }
 __device__ inline cplx gj_make(const double* x, cplx) { return mkc(x[0], x[1]); }
 
-// An operand in shared memory: limbs, or (batches, real) the FP64 value.
+// An operand in shared memory: limbs, or the FP64 value.
 template <bool FX> struct GjOperand { using type = int2; };
 template <> struct GjOperand<false> { using type = double; };
 template <bool FX> __device__ inline typename GjOperand<FX>::type gj_operand(double x, int e) {
@@ -905,7 +943,7 @@ __global__ void __launch_bounds__(256) k_gj_rows(SwrDeviceView v, int kb, int sy
     constexpr int P = GjParts<T>::v;
     const SubDev& s = v.sub[blockIdx.y];
     const int K = s.K, k0 = kb * GJ_NB, tn = blockIdx.x * GJ_T;
-    if (k0 >= K || tn >= K) return;
+    if (k0 >= K || tn >= K || (v.inst[s.inst].fx != 0) != FX) return;
     const int nb = min(GJ_NB, K - k0), tid = threadIdx.x;
     const double* M = v.arena + s.Gm;
     double* Pinv = v.arena + s.work;
@@ -981,7 +1019,7 @@ __global__ void __launch_bounds__(256) k_gj_update(SwrDeviceView v, int kb, int 
     constexpr int TL = GjTile<T>::v, P = GjParts<T>::v, N = TL * GJ_NB / 256, Q = TL / 16;
     const SubDev& s = v.sub[blockIdx.z];
     const int K = s.K, k0 = kb * GJ_NB;
-    if (k0 >= K) return;
+    if (k0 >= K || (v.inst[s.inst].fx != 0) != FX) return;
     const int tm = blockIdx.y * TL, tn = blockIdx.x * TL;
     if (tm >= K || tn >= K || (sym && tn > tm)) return;
     const int nb = min(GJ_NB, K - k0), tid = threadIdx.x;
@@ -1043,7 +1081,7 @@ template <typename T>
 __global__ void k_gj_mirror(SwrDeviceView v) {
     const SubDev& s = v.sub[blockIdx.z];
     const int K = s.K, r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (r0 >= K || c0 > r0) return;
+    if (r0 >= K || c0 > r0 || !v.inst[s.inst].fx) return;
     double* M = v.arena + s.Gm;
     __shared__ T t[32][33];
     for (int i = w; i < 32; i += 8)
@@ -1059,6 +1097,7 @@ __global__ void k_gj_mirror(SwrDeviceView v) {
 // under the diagonal are updated: with p eliminated and u remaining indices, M[p, u]
 // = -M[u, p]^T, the other two blocks are symmetric.  K = 576, 16 subdomains: 131 -> 86
 // us per block column; the other half follows the last one (k_gj_mirror).
+// Row block and update of block column kb, of the instances in this arithmetic.
 template <typename T, bool FX>
 static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int max_K, bool update) {
     const int sym = FX && update;
@@ -1068,7 +1107,6 @@ static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int
     cudaError_t e = cudaFuncSetAttribute(k_gj_rows<T, FX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_gj_update<T, FX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)su);
     if (e != cudaSuccess) return e;
-    k_gj_panel<T><<<v.n_sub, 256, 0, st>>>(v, kb);
     k_gj_rows<T, FX><<<dim3((max_K + GJ_T - 1) / GJ_T, v.n_sub), 256, sr, st>>>(v, kb, sym);
     if (update) k_gj_update<T, FX><<<dim3((max_K + TL - 1) / TL, (max_K + TL - 1) / TL, v.n_sub), 256, su, st>>>(v, kb, sym);
     if (sym && (kb + 1) * GJ_NB >= max_K)
@@ -1082,7 +1120,8 @@ static cudaError_t gj_block(const SwrDeviceView& v, cudaStream_t st, int kb, int
 // (projection of Sec. 6.1 in the orthonormal basis: c' = X^T c~).
 // out[sid] = partial PoU norm^2 of c0 (later summed per instance).  The node values
 // are formed once per coordinate (in every coefficient's own sum: 430 us at kd =
-// 24, q = 132) and the norm is summed over the block (216 us by one thread).
+// 24, q = 132) and the norm is summed over the block (216 us by one thread, as it
+// is still for instances assembled in FP64: theirs may amplify its rounding).
 __global__ void k_project(SwrDeviceView v, double* norm_part) {
     const int sid = blockIdx.x;
     const SubDev& s = v.sub[sid];
@@ -1108,7 +1147,7 @@ __global__ void k_project(SwrDeviceView v, double* norm_part) {
             u[d][a] = acc;
         }
         __syncthreads();
-        if (!fp64_batch(v)) {  // rows of the quadratic form, then their sum, over lanes
+        if (in.fx) {  // rows of the quadratic form, then their sum, over lanes
             for (int a = warp; a < kd; a += nw) {
                 double acc = 0;
                 for (int c = lane; c < kd; c += 32) acc += T[lay.mat(M_PP) + a * kd + c] * u[d][c];
@@ -1228,7 +1267,7 @@ cudaError_t te_products(const TgState* g, const SwrDeviceView& v, cudaStream_t s
 
 // tg: the tensor-core Gauss-Jordan state (swr_tcgj.cu) or null for the FP64 updates.
 cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, int max_kd, int max_K,
-                            bool any_ee, bool any_tdse, bool any_tise, const GemmJob* d_jobs1,
+                            bool any_ee, bool any_tdse, bool any_fx, bool any_64, const GemmJob* d_jobs1,
                             const GemmJob* d_jobs2, double* d_norm_part, const TgState* tg) {
     dim3 g2(v.n_sub, 2);
     k_tabulate<<<g2, 256, 0, st>>>(v);
@@ -1246,10 +1285,12 @@ cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, 
         } else {
             int kd2 = max_kd * max_kd;
             // Mee = Wv (q x q) * P2 (q x kd^2)
-            const auto gemm = fp64_batch(v) ? k_dgemm : k_fxgemm;
-            gemm<<<dim3(div_up(kd2, GT), div_up(max_q, GT), v.n_sub), 256, 0, st>>>(v, d_jobs1);
+            const dim3 gm(div_up(kd2, GT), div_up(max_q, GT), v.n_sub), gh(div_up(kd2, GT), div_up(kd2, GT), v.n_sub);
+            if (any_fx) k_fxgemm<<<gm, 256, 0, st>>>(v, d_jobs1);
+            if (any_64) k_dgemm<<<gm, 256, 0, st>>>(v, d_jobs1);
             // V'ee[(a,c),(b,e)] = P1^T (kd^2 x q) * Mee (q x kd^2), scattered into H'
-            gemm<<<dim3(div_up(kd2, GT), div_up(kd2, GT), v.n_sub), 256, 0, st>>>(v, d_jobs2);
+            if (any_fx) k_fxgemm<<<gh, 256, 0, st>>>(v, d_jobs2);
+            if (any_64) k_dgemm<<<gh, 256, 0, st>>>(v, d_jobs2);
         }
     }
     dim3 ge(div_up((long long)max_K * max_K, 256 * 8), v.n_sub);
@@ -1258,9 +1299,12 @@ cudaError_t launch_assemble(const SwrDeviceView& v, cudaStream_t st, int max_q, 
     k_step_matrix<<<ge, 256, 0, st>>>(v);
     int nkb = (max_K + GJ_NB - 1) / GJ_NB;
     for (int kb = 0; kb < nkb; ++kb) {
-        cudaError_t e = any_tdse      ? gj_block<cplx, true>(v, st, kb, max_K, !tg)
-                        : fp64_batch(v) ? gj_block<double, false>(v, st, kb, max_K, !tg)
-                                        : gj_block<double, true>(v, st, kb, max_K, !tg);
+        if (any_tdse) k_gj_panel<cplx><<<v.n_sub, 256, 0, st>>>(v, kb);
+        else k_gj_panel<double><<<v.n_sub, 256, 0, st>>>(v, kb);
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess && any_tdse) e = gj_block<cplx, true>(v, st, kb, max_K, !tg);
+        if (e == cudaSuccess && any_fx && !any_tdse) e = gj_block<double, true>(v, st, kb, max_K, !tg);
+        if (e == cudaSuccess && any_64) e = gj_block<double, false>(v, st, kb, max_K, !tg);
         if (e == cudaSuccess && tg) e = tg_update(tg, v, st, kb, max_K);
         if (e != cudaSuccess) return e;
     }

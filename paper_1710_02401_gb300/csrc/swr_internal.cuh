@@ -41,6 +41,7 @@ struct InstDev {
     double orth_tau;              // Cholesky acceptance / canonical cut-off of the 1-D overlaps
     int tc;                       // transmission condition (swr_tc)
     int anti;                     // antisymmetric states: steps act on the antisymmetric part (swr_symmetry)
+    int fx;                       // e-e products and elimination in fixed point (else FP64), see swr_assemble.cu
 };
 
 // Per-subdomain descriptor.  Offsets are in doubles from the arena base.

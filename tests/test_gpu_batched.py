@@ -174,3 +174,32 @@ def test_window_edge_cases_in_one_launch(S, edge_refs, precision, variant):
     assert s.window_plan()["variant"] == (3 if precision == 1 else 1)
     s.assemble()
     _check(*_steps(s, 2), edge_refs)
+
+
+def _double_well(dt):
+    """One electron, two deep wells.  dt = 0.125 puts 1 + dt E past zero for the two
+    lowest levels (-8.23, -8.01): the odd one, which the initial data do not hold,
+    grows out of the rounding 16-fold a step."""
+    box = (-6.0, 6.0)
+    return P.tise_1d_two_subdomains().replace(L=1, box=box, nuclei=((-1.0, 3.0), (1.0, 3.0)), eta_en=0.3, K_d=40,
+                                              delta=P.spacing_rule_delta(box, 1, 1.0, 40), q_p=20, n_mid=9, dt=dt,
+                                              ngf_tol=0.0, n_steps=60)
+
+
+def test_an_instance_has_the_same_step_matrices_alone_and_in_a_batch(S):
+    # the arithmetic of the assembly is the instance's own: bits equal, with the same row tasks
+    insts = [_double_well(0.125), P.small_tise_2d(K_d=9).replace(ngf_tol=0.0, n_steps=60), _double_well(0.02)]
+    kw = dict(precision=S.PREC_FP64, window_variant=S.WINDOW_TWO_PHASE, rows_per_task=8)
+    both = S.SWR(insts, **kw)
+    both.assemble()
+    both.step()
+    psi, energy, o = both.get(S.FIELD_PSI_NODES), both.energy(), 0
+    for j, inst in enumerate(insts):
+        one = S.SWR(inst, **kw)
+        one.assemble()
+        one.step()
+        p = one.get(S.FIELD_PSI_NODES)
+        np.testing.assert_array_equal(p, psi[o:o + p.size], err_msg=str(j))
+        assert one.energy()[0] == energy[j]
+        o += p.size
+    assert o == psi.size
