@@ -458,6 +458,14 @@ swr_status swr_residual_noalloc(swr_ctx* ctx, double* res_host, size_t n);
  * otherwise); real-time problems have no window kernel (SWR_EINVAL).  The
  * window state it writes is re-initialised by the first swr_step.  `out`
  * (may be NULL) receives the choice.                                         */
+typedef enum swr_window_form {
+    SWR_FORM_VARIANT = 0,    /* the kernel named by swr_window_variant          */
+    SWR_FORM_ON_CHIP = 1,    /* FP64 two-phase recursion in the shared memory of one
+                                cluster per instance                            */
+    SWR_FORM_ONE_PASS = 2    /* FP64 two-phase recursion in one pass over G and
+                                W = (Pp (x) Pp) G per step                      */
+} swr_window_form;
+
 typedef struct swr_tune_report {
     int    variant;          /* swr_window_variant chosen                       */
     int    rows_per_task;    /* row-task target chosen                          */
@@ -470,12 +478,19 @@ typedef struct swr_tune_report {
     double seconds_default;  /* time per step of the plan before tuning         */
     int    tensor_contractions; /* 1: assembly runs the Gauss-Jordan updates and
                                    e-e products on the tensor cores             */
+    int    form;             /* swr_window_form.  Forms 1 and 2 are what the automatic
+                                FP64 plan makes of SWR_WINDOW_TWO_PHASE: ask for them
+                                with window_variant 0 and rows_per_task 0 (naming the
+                                variant or a row target selects the plain kernel).
+                                On chip, tasks are the CTAs' shares of rows and
+                                rows_per_task the largest of them               */
 } swr_tune_report;
 swr_status swr_autotune(swr_ctx* ctx, int steps, swr_tune_report* out);
 
 /* The window plan in use (variant, rows_per_task, tasks, ctas,
- * task_state_global, graph, tensor_contractions; the timing fields are zero).  variant is 0 for
- * real-time problems, whose steps are launched from the host.               */
+ * task_state_global, graph, tensor_contractions, form; the timing fields are zero).  variant is 0
+ * for real-time problems, which have one window kernel (SWR_PREC_FP32_REFINED: steps
+ * launched from the host).                                                  */
 swr_status swr_window_plan(const swr_ctx* ctx, swr_tune_report* out);
 
 /* ------------------------------------------------------------------------

@@ -1489,15 +1489,22 @@ static swr_status time_window_plan(swr_ctx* c, int steps, double* sec_per_step) 
     return SWR_OK;
 }
 
+// The plan in use, in the fields that describe one.
+static void report_plan(const swr_ctx* c, swr_tune_report* out) {
+    const int shares = (int)c->inst.size() * c->oc_shape.cs;
+    out->variant = c->tdse ? 0 : c->variant;
+    out->form = c->oc ? SWR_FORM_ON_CHIP : c->w1 ? SWR_FORM_ONE_PASS : SWR_FORM_VARIANT;
+    out->rows_per_task = c->oc ? c->oc_shape.rows_max : c->rows_target;
+    out->tasks = c->oc ? shares : (int)c->tasks.size();
+    out->ctas = c->oc ? shares : c->grid;
+    out->task_state_global = c->oc ? 0 : c->many;
+    out->graph = (c->prob.launch_mode == SWR_LAUNCH_GRAPH && !c->graph_failed) ? 1 : 0;
+}
+
 extern "C" swr_status swr_window_plan(const swr_ctx* c, swr_tune_report* out) {
     if (!c || !out) return fail(nullptr, SWR_EINVAL, "ctx or out is NULL");
     memset(out, 0, sizeof(*out));
-    out->variant = c->tdse ? 0 : c->variant;
-    out->rows_per_task = c->rows_target;
-    out->tasks = (int)c->tasks.size();
-    out->ctas = c->oc ? (int)c->inst.size() * c->oc_shape.cs : c->grid;
-    out->task_state_global = c->oc ? 0 : c->many;
-    out->graph = (c->prob.launch_mode == SWR_LAUNCH_GRAPH && !c->graph_failed) ? 1 : 0;
+    report_plan(c, out);
     out->tensor_contractions = c->use_tg ? 1 : 0;
     return SWR_OK;
 }
@@ -1552,13 +1559,8 @@ extern "C" swr_status swr_autotune(swr_ctx* c, int steps, swr_tune_report* out) 
     c->prob.window_variant = best.variant;
     c->prob.rows_per_task = best.rows;
     if (out) {
-        out->variant = c->variant;
-        out->rows_per_task = c->rows_target;
-        out->tasks = (int)c->tasks.size();
-        out->ctas = c->oc ? (int)c->inst.size() * c->oc_shape.cs : c->grid;
-        out->task_state_global = c->oc ? 0 : c->many;
+        report_plan(c, out);
         out->candidates = timed;
-        out->graph = (c->prob.launch_mode == SWR_LAUNCH_GRAPH && !c->graph_failed) ? 1 : 0;
         out->seconds_per_step = best_t;
         out->seconds_default = t_default;
     }

@@ -59,7 +59,7 @@ class swr_tune_report(C.Structure):
     _fields_ = [("variant", C.c_int), ("rows_per_task", C.c_int), ("tasks", C.c_int), ("ctas", C.c_int),
                 ("task_state_global", C.c_int), ("candidates", C.c_int), ("graph", C.c_int),
                 ("seconds_per_step", C.c_double),
-                ("seconds_default", C.c_double), ("tensor_contractions", C.c_int)]
+                ("seconds_default", C.c_double), ("tensor_contractions", C.c_int), ("form", C.c_int)]
 
 
 class swr_iter_report(C.Structure):

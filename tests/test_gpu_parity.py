@@ -319,6 +319,40 @@ def test_parity_fp64_window_on_chip_edges(swr_mod, inst):
     _compare(swr_mod, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE)
 
 
+ON_CHIP, ONE_PASS, PLAIN = 1, 2, 0
+
+
+def _one_large_subdomain(K_d):
+    base = P.small_tise_2d(L=2, q_p=K_d, n_mid=2, max_steps=40)
+    kds = [K_d, 4, 4, 4]
+    return base.replace(K_d=kds, delta=[P.spacing_rule_delta(base.box, 2, base.overlap, k) for k in kds])
+
+
+@pytest.mark.parametrize("inst,form", [
+    (_one_large_subdomain(16), ON_CHIP),                                       # K = 256, the sums' bound
+    (P.small_tise_2d(L=2, K_d=15, q_p=15, n_mid=2, max_steps=60), ON_CHIP),    # 221,608 of 229,376 bytes a CTA
+    (P.small_tise_2d(L=2, K_d=16, q_p=16, n_mid=2, max_steps=40), ONE_PASS),   # past the shared memory of 16 CTAs
+    (_one_large_subdomain(17), ONE_PASS),                                      # past K = 256
+    (P.tise_1d_two_subdomains().replace(K_d=3, delta=0.05, max_steps=60), ON_CHIP),
+    (P.small_tise_2d(L=3, K_d=32, q_p=32, n_mid=1, max_steps=6), PLAIN)],      # G and W past L2
+    ids=["k256", "k225-memory", "4x256", "k289", "tiny", "k1024"])
+def test_fp64_window_form_follows_the_size(swr_mod, inst, form):
+    S = swr_mod
+    s = S.SWR(inst)
+    plan = s.window_plan()
+    assert plan["variant"] == S.WINDOW_TWO_PHASE and plan["form"] == form
+    if form == ON_CHIP:
+        assert plan["tasks"] == plan["ctas"] <= 16 and plan["ctas"] * plan["rows_per_task"] >= sum(
+            int(K) for _q, _ng, K in s.node_counts())
+    for kw in (dict(window_variant=S.WINDOW_TWO_PHASE), dict(rows_per_task=8), dict(precision=S.PREC_MIXED)):
+        assert S.SWR(inst, **kw).window_plan()["form"] == PLAIN
+    if form != PLAIN:
+        s.assemble()
+        rep = s.autotune(steps=6)
+        assert rep["form"] == s.window_plan()["form"] and (form != ON_CHIP or rep["form"] == ON_CHIP)
+        _compare(S, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE)
+
+
 @pytest.mark.parametrize("mode", [P.TISE, P.TDSE])
 @pytest.mark.parametrize("K_d", [31, 32, 33, 63, 65])
 def test_parity_step_matrix_inverse_at_block_edges(swr_mod, K_d, mode):
