@@ -354,7 +354,9 @@ typedef enum swr_field {
                                        8 K^2 per matrix sweep, 1 + m sweeps per step,
                                        in real time),
                                    [4] algorithmic bytes of the window kernels
-                                       (step-matrix bytes read per local step solve),
+                                       (step-matrix bytes read per local step solve,
+                                       from HBM, L2 or on chip; kernels that also read
+                                       W = (Pp (x) Pp) G twice those of [10]),
                                    [5] local step solves,
                                    [6] ms of swr_assemble (events), [7] ms of swr_step,
                                    [8] host->device bytes copied, [9] device->host bytes,

@@ -1419,9 +1419,11 @@ extern "C" swr_status swr_step(swr_ctx* c, swr_iter_report* rep) {
         for (size_t i = 0; i < ni; ++i) nsolve[i] = c->win_h[i];
         // bytes per matrix element: complex G0 16 (four FP32 planes), 8 in fixed
         // point (only the lower triangle is read);
-        // real G 8 (FP64 or FP32 hi/lo); the fused variant also streams W (16);
-        // half of each with the FP32-rounded matrices (hi planes only)
-        const double bel = (c->rt ? 8.0 : c->tdse ? 16.0 : (c->variant == WIN_FUSED ? 16.0 : 8.0)) * (go ? 0.5 : 1.0);
+        // real G 8 (FP64 or FP32 hi/lo); the fused, the one-pass and the on-chip
+        // kernels also read W (16); half of each with the FP32-rounded matrices
+        // (hi planes only)
+        const bool reads_w = c->variant == WIN_FUSED || c->w1 || c->oc;
+        const double bel = (c->rt ? 8.0 : c->tdse ? 16.0 : reads_w ? 16.0 : 8.0) * (go ? 0.5 : 1.0);
         for (size_t sid = 0; sid < c->sub.size(); ++sid) {
             const SubDev& sd = c->sub[sid];
             if (c->inst[sd.inst].anti && sd.N == 2 && sd.idx[0] > sd.idx[1]) continue;  // mirror image, not solved

@@ -353,6 +353,22 @@ def test_fp64_window_form_follows_the_size(swr_mod, inst, form):
         _compare(S, inst, kmax=2, rel_robin=REL_ROBIN_PROJECTED_EDGE)
 
 
+@pytest.mark.parametrize("precision,kw,per_element", [
+    (0, {}, 16), (0, {"L": 2, "K_d": 16}, 16), (0, {"window_variant": 1}, 8),  # on chip, one pass, two-phase
+    (1, {"window_variant": 2}, 16), (1, {"window_variant": 3}, 8)])             # fused, split
+def test_step_matrix_bytes_of_the_window_count_what_it_reads(swr_mod, precision, kw, per_element):
+    shape = {k: kw[k] for k in kw if k != "window_variant"}
+    inst = P.small_tise_2d(**{"L": 3, "K_d": 8, **shape}).replace(ngf_tol=0.0, n_steps=7)
+    s = swr_mod.SWR(inst, precision=precision, window_variant=kw.get("window_variant", 0))
+    s.assemble()
+    before = s.counters()
+    s.step()
+    got = s.counters()
+    elements = 7 * sum(int(K) ** 2 for _q, _ng, K in s.node_counts())
+    assert got["window_bytes"] - before["window_bytes"] == per_element * elements
+    assert got["window_bytes_alg"] - before["window_bytes_alg"] == 8 * elements
+
+
 @pytest.mark.parametrize("mode", [P.TISE, P.TDSE])
 @pytest.mark.parametrize("K_d", [31, 32, 33, 63, 65])
 def test_parity_step_matrix_inverse_at_block_edges(swr_mod, K_d, mode):
