@@ -133,12 +133,14 @@ __device__ inline unsigned tc_begin(TcShared& sh) {
 // (mma(stage address, block)) and frees the stage on their completion.  Every
 // thread then waits for the last product.  All waits are bounded; a thread that
 // gives up records it, the others run into their own limit or the done
-// barrier, and copies in flight are waited for before the CTA returns.
+// barrier, and then the copies issued last into every stage are waited for,
+// whichever thread gave up: a CTA must not return while one still writes its
+// shared memory.
 template <int STAGES, class Load, class Mma>
 __device__ inline bool tc_pipeline(TcShared& sh, unsigned char* ring, int stage_bytes, int nblk, unsigned bytes, Load load,
                                    Mma mma) {
+    int issued = 0;
     if (threadIdx.x == 0) {
-        int issued = 0;
         bool ok = true;
         for (int b = 0; b < nblk && ok; ++b) {
             const int st = b % STAGES;
@@ -149,11 +151,7 @@ __device__ inline bool tc_pipeline(TcShared& sh, unsigned char* ring, int stage_
             load(tc_smem(ring + (size_t)st * stage_bytes), b, bar);
             issued = b + 1;
         }
-        if (!ok) {
-            sh.fail = 1;
-            for (int b = issued > STAGES ? issued - STAGES : 0; b < issued; ++b)
-                tc_wait(tc_smem(&sh.full[b % STAGES]), (b / STAGES) & 1);
-        }
+        if (!ok) sh.fail = 1;
     } else if (threadIdx.x == 32) {
         bool ok = true;
         for (int b = 0; b < nblk && ok; ++b) {
@@ -170,6 +168,9 @@ __device__ inline bool tc_pipeline(TcShared& sh, unsigned char* ring, int stage_
     __syncwarp();
     if (!tc_wait(tc_smem(&sh.done), 0)) sh.fail = 1;
     __syncthreads();
+    if (sh.fail && threadIdx.x == 0)
+        for (int b = issued > STAGES ? issued - STAGES : 0; b < issued; ++b)
+            tc_wait(tc_smem(&sh.full[b % STAGES]), (b / STAGES) & 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
     return sh.fail == 0;
 }
