@@ -7,19 +7,31 @@
 // A vector is therefore held as 56-bit integers relative to a power of two
 // above its largest component (exponent shared by the vector), each cut into
 // two 32-bit limbs, F = 2^28 hi + lo with |hi| <= 2^28, |lo| <= 2^27; a matrix
-// likewise with one exponent.  A product takes three multiply-adds:
-// hi hi into one accumulator (units 2^-56 of the scales), hi lo + lo hi into a
-// second (2^-84); lo lo, below 2^-58 of the scales, is dropped.  Sums are exact
-// and so independent of their order.  Against plain FP64: the representation
-// error is 2^-57 of the largest component instead of 2^-53 of each, the sums
-// carry no rounding at all.  (A double-single multiply-add on the FP32 pipes
+// likewise with one exponent a row (real time: one a matrix, which is used by
+// rows and by columns), the power of two next to its 2-norm.  A product takes three
+// multiply-adds: hi hi into one accumulator (units 2^-56 of the scales), hi lo +
+// lo hi into a second (2^-84); lo lo is dropped, below 2^-58 of the scales (2^-57
+// where limbs of two numbers have been added, in Karatsuba's products).  The
+// accumulators are exact; every thread rounds its second one to a unit of the first
+// when it folds it in, so another cut of a row into lanes, tiles or CTAs changes the
+// sum by a few of these units.  (A double-single multiply-add on the FP32 pipes
 // takes 13 instructions and keeps about 2^-46.)
 //
-// Bounds: at most 64 terms of at most 2^56 go into the first accumulator of a
-// thread, at most 128 of at most 2^55 into the second; it is folded into the
-// first (rounded) before more are added.  Sums over whole rows stay below 2^62
-// by Cauchy-Schwarz: row norms of the matrices are at most 1 (2^28 scaled), the
-// vector's 2-norm at most sqrt(2 K) times its scale.
+// Against plain FP64 the representation error is 2^-57 of the row or the vector
+// instead of 2^-53 of every product and partial sum: smaller in norm (a step matrix
+// of 40 Gaussians times a vector, restated in exact arithmetic: 0.4e-16 against 0.8
+// to 1.4e-16), larger in components far below the largest, which hold fewer than 53
+// bits from 1/8 of it down (the same product: 3e-15 against 6e-16 relative in the
+// worst component of a random vector; a smooth one's smallest, 1e-6 of the largest,
+// 1e-11).  Nothing here reads single components against their own size: energies,
+// norms, traces and residuals are sums over them.
+//
+// Bounds: a thread's first accumulator takes up to 96 terms of 2^56 before it is
+// folded (real time, one electron, Q' of 96 Gaussians: 2^62.6), its second 192 of
+// 2^55 there, 128 elsewhere.  A wrap of a partial sum would not matter, it is
+// arithmetic modulo 2^64 and the total is what has to fit; sums over whole rows stay
+// below 2^62 by Cauchy-Schwarz (fx_row_exp; vectors at most sqrt(2 K) times
+// their scale).
 #pragma once
 
 #include "swr_internal.cuh"
@@ -45,6 +57,18 @@ __device__ inline int2 fx_limbs(double x, int emax) {
     const int hi = (int)((f + (1LL << (FX_BITS - 1))) >> FX_BITS);
     return make_int2(hi, (int)(f - ((long long)hi << FX_BITS)));
 }
+// Exponent of a matrix row whose largest entry has exponent e and whose 2-norm
+// squared is q in units of 2^(2 (e - 1022)): the smallest power of two of which the
+// norm does not exceed sqrt(2) times.  Entries may then pass the scale by that
+// factor, |hi| < 1.42 2^28; the product with a vector of K <= 1024 entries stays
+// below 2^28.5 x 32 x 2^28 = 2^61.5 (complex: 2^62).
+__device__ inline int fx_row_exp(int e, float q) {
+    int x = -1;
+    while (x < 6 && 1.99f * ldexpf(1.f, 2 * x) <= q) ++x;  // (q <= 2 K)
+    return e >= FX_BAD ? FX_BAD : max(e + x, 0);
+}
+// 2^(1022 - e), the factor that takes entries of exponent e to units of that q.
+__device__ inline double fx_row_scale(int e) { return e > 0 && e < 2045 ? __hiloint2double((2045 - e) << 20, 0) : 0.0; }
 // Weight of a unit of the first accumulator for a vector with exponent emax
 // and a matrix scaled by 2^eg: 2^(emax - 1022 + eg - 56).
 __device__ inline double fx_unit(int emax, int eg) {

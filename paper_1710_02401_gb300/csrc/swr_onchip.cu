@@ -19,8 +19,9 @@
 //  - y rows go to the CTAs of their subdomain and the partials of s^2 and of the
 //    stop test to every CTA through distributed shared memory;
 //  - the products run in 56-bit fixed point (swr_fixed.cuh; matrix rows scaled by
-//    their largest entry, two bits kept free so that sums of K <= 256 terms stay
-//    below 2^62): exact sums at 4.5 multiply-adds per clock and SM against 1.6
+//    their 2-norm.  By their largest entry with two bits kept free, the product of 40
+//    rows with a smooth vector was 1.8e-16 off in norm, 0.8e-16 in FP64; so it is
+//    0.4e-16): exact sums at 4.5 multiply-adds per clock and SM against 1.6
 //    on the FP64 pipe and, what counts here, additions of 4 clocks instead of 66.
 // Everything else stays FP64.
 #include <math.h>
@@ -35,7 +36,7 @@ namespace swr {
 #define OC_WARPS 16
 #define OC_CMAX 16                 // CTAs per cluster (at most)
 #define OC_SMEM_MAX (224 * 1024)
-#define OC_KMAX 256                // K of a subdomain (at most: the sums' bound)
+#define OC_KMAX 256                // K of a subdomain (at most)
 #define OC_SUBS 64                 // subdomains with rows in one CTA (at most)
 
 // Limb pairs per matrix row: an odd number of 64-byte segments (8 columns), so
@@ -166,7 +167,16 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_window_onchip(OcArgs A) {
             const double* row = v.arena + (h ? s.Hm : s.Gm) + (long long)r * K;
             int e = 0;
             for (int c = lane; c < K; c += 32) e = max(e, fx_exp(row[c]));
-            e = __reduce_max_sync(0xffffffffu, e) + 2;  // two bits free (sums of up to 256 terms)
+            e = __reduce_max_sync(0xffffffffu, e);
+            const double sc = fx_row_scale(e);
+            float q = 0.f;
+            for (int c = lane; c < K; c += 32) {
+                const float t = (float)(row[c] * sc);
+                q += t * t;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            e = fx_row_exp(e, q);
             for (int c = lane; c < pitch; c += 32) lim[r_off[i] + h * pitch + c] = c < K ? fx_limbs(row[c], e) : make_int2(0, 0);
             if (lane == 0) (h ? r_ew : r_eg)[i] = e;
         }

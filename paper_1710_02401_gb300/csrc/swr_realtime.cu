@@ -138,8 +138,7 @@ __global__ void k_rt_theta(SwrDeviceView v, double* theta, int cap) {
     theta[(long long)blockIdx.y * (cap + 1) + n] = 0.5 * in.dt * e;
 }
 
-// Exponent of a subdomain's G0: 2^(e - 1022) is the smallest power of two of
-// which no row's 2-norm exceeds sqrt(2) times (1 for the ||G0|| <= 1 of an
+// Exponent of a subdomain's G0, the largest of its rows' (fx_row_exp: 2^0 for the ||G0|| <= 1 of an
 // absorbing boundary with kinetic > 0; larger where G0 is, smaller where the
 // whole matrix is small), FX_BAD when an entry is not finite.  A warp per row.
 __global__ void k_rt_scale(SwrDeviceView v, int* gexp) {
@@ -150,7 +149,7 @@ __global__ void k_rt_scale(SwrDeviceView v, int* gexp) {
     int e = 0;
     for (int c = lane; c < K; c += 32) e = max(e, max(fx_exp(g[c].x), fx_exp(g[c].y)));
     e = __reduce_max_sync(0xffffffffu, e);
-    const double sc = e > 0 && e < 2045 ? __hiloint2double((2045 - e) << 20, 0) : 0.0;  // 2^(1022 - e)
+    const double sc = fx_row_scale(e);
     float q = 0.f;
     for (int c = lane; c < K; c += 32) {
         const float a = (float)(g[c].x * sc), b = (float)(g[c].y * sc);
@@ -158,9 +157,7 @@ __global__ void k_rt_scale(SwrDeviceView v, int* gexp) {
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    int x = -1;
-    while (x < 6 && 1.99f * ldexpf(1.f, 2 * x) <= q) ++x;  // (q <= 2 K)
-    if (lane == 0) atomicMax(gexp + blockIdx.y, e >= FX_BAD ? FX_BAD : max(e + x, 0));
+    if (lane == 0) atomicMax(gexp + blockIdx.y, fx_row_exp(e, q));
 }
 
 // Limbs of the lower triangle of G0 relative to its exponent, strip by strip

@@ -390,10 +390,9 @@ __device__ inline void df32_rows4(const float* Gh, const float* Gl, int ld, cons
 
 // The FP64 step-matrix inverse G (blockIdx.z = 0) and, for the one-pass window,
 // W = (Pp (x) Pp) G in the space of H' (blockIdx.z = 1) as limbs in their own
-// place, every row scaled by a power of two above its 2-norm, whose exponent goes
-// to the assembly's scratch ([2][K] ints): the FP64 grid windows read 8 bytes per
-// element as before.  With rows and columns of norm at most 2^28 the sums stay
-// below 2^61 for K <= 1024.
+// place, every row scaled by the power of two next to its 2-norm (fx_row_exp), whose
+// exponent goes to the assembly's scratch ([2][K] ints): the FP64 grid windows read
+// 8 bytes per element as before.
 __global__ void k_fx_rows(SwrDeviceView v) {
     const SubDev& s = v.sub[blockIdx.y];
     const int K = s.K, lane = threadIdx.x & 31;
@@ -404,8 +403,7 @@ __global__ void k_fx_rows(SwrDeviceView v) {
         int e = 0;
         for (int c = lane; c < K; c += 32) e = max(e, fx_exp(g[c]));
         e = __reduce_max_sync(0xffffffffu, e);
-        // the 2-norm over the largest entry, as a power of two above it
-        const double sc = e > 0 && e < 2045 ? __hiloint2double((2045 - e) << 20, 0) : 0.0;
+        const double sc = fx_row_scale(e);
         float q = 0.f;
         for (int c = lane; c < K; c += 32) {
             const float t = (float)(g[c] * sc);
@@ -413,9 +411,7 @@ __global__ void k_fx_rows(SwrDeviceView v) {
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-        int x = 0;
-        while (x < 6 && ldexpf(1.f, 2 * x) <= 1.001f * q) ++x;
-        if (e < FX_BAD) e += x;
+        e = fx_row_exp(e, q);
         for (int c = lane; c < K; c += 32) reinterpret_cast<int2*>(g)[c] = fx_limbs(g[c], e);
         if (lane == 0) ex[r] = e;
     }

@@ -329,7 +329,7 @@ def _one_large_subdomain(K_d):
 
 
 @pytest.mark.parametrize("inst,form", [
-    (_one_large_subdomain(16), ON_CHIP),                                       # K = 256, the sums' bound
+    (_one_large_subdomain(16), ON_CHIP),                                       # K = 256, the largest on chip
     (P.small_tise_2d(L=2, K_d=15, q_p=15, n_mid=2, max_steps=60), ON_CHIP),    # 221,608 of 229,376 bytes a CTA
     (P.small_tise_2d(L=2, K_d=16, q_p=16, n_mid=2, max_steps=40), ONE_PASS),   # past the shared memory of 16 CTAs
     (_one_large_subdomain(17), ONE_PASS),                                      # past K = 256
