@@ -349,9 +349,13 @@ static swr_status validate(swr_ctx* c, const swr_problem* p) {
 static const int ROWS_MIN = 8;          // smallest row task
 static const int ROWS_MANY_MAX = 256;    // largest row task (task state in global memory)
 static const size_t WIN_SMEM_TASKS_MAX = 100 * 1024;  // dynamic shared memory for two CTAs per SM
-// FP64 one-pass window (k_window_fx): G and W must stay in L2 (129 MB).  us per step
-// one-pass / two-phase: 16 x 576^2 (85 MB) 18.8 / 32.2, 100 x 256^2 (105 MB) 30.4 /
-// 59.4, 25 x 576^2 (133 MB) 32.1 / 40.2, 9 x 1024^2 (151 MB) 47.2 / 38.8.
+// FP64 one-pass window (k_window_fx): bytes of G and W with which it was faster at
+// every size tried (L2 holds 129 MB).  us per step one-pass / two-phase: 16 x 576^2
+// (85 MB) 18.8 / 32.2, 36 x 400^2 (92 MB) 35.8 / 46.2, 100 x 256^2 (105 MB) 30.4 / 59.4,
+// 81 x 289^2 (108 MB) 35.6 / 60.0.  Past it bytes alone do not tell: most sizes
+// still gain (49 x 400^2, 125 MB, 42.4 / 58.2; 25 x 576^2, 133 MB, 32.2 / 37.0; 25 x 784^2,
+// 246 MB, 72.4 / 84.9), few large subdomains lose (9 x 961^2, 133 MB, 45.0 / 39.4;
+// 9 x 1024^2, 151 MB, 44.7 / 37.4), so the line stays below both.
 static const double W1_BYTES_MAX = 110e6;
 static const int SPLIT_STAGES = 2;       // split window: stages of staged step-matrix rows in flight per CTA
 static const int SPLIT_STAGE_ROWS = 4;   // split window: rows of the widest subdomain per stage (at most)

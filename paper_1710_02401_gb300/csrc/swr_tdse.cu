@@ -1,4 +1,6 @@
-// swr_tdse.cu -- real-time time window (Crank-Nicolson under the dipole field).
+// swr_tdse.cu -- real-time time window (Crank-Nicolson under the dipole field) by
+// sweeps launched from the host: SWR_PREC_FP32_REFINED.  The other precisions run
+// the same step in one persistent kernel (swr_realtime.cu).
 //
 // Sec. 5.4 step 2 (real time) with the Robin data of Sec. 5.1 and the
 // length-gauge field of Sec. 1.2, in the orthonormal local basis (A' = I):
@@ -11,9 +13,9 @@
 //   r = 2 c^n + i (theta_{n+1} - theta_n) Q' c^n + i dt/2 kappa (b'^{n+1} + b'^n),
 //   solve (M0 + i theta_{n+1} Q') x = r  by  x <- G0 (r - i theta_{n+1} Q' x),
 //   c^{n+1} = x - c^n.
-// The Hermitian part of M0 is I - (dt/2) kappa mu_im R' >= I for mu_im <= 0,
-// so ||G0|| <= 1 and the fixed point contracts with
-// rho <= (dt/2) max|e| max_{Omega_i}|x_1 + ... + x_N|; the host chooses the
+// The Hermitian part of M0 is I - (dt/2) kappa mu_im R' >= I for kappa > 0 and
+// mu_im <= 0, so ||G0|| <= 1 and the fixed point contracts with
+// rho <= (dt/2) max|e| max_{Omega_i}|x_1 + ... + x_N|; here the host chooses the
 // iteration count from rho so that rho^(m+1) <= 1e-15.
 //
 // Complex vectors are planar: [re block K][im block K].  G0 is interleaved
