@@ -1,7 +1,7 @@
 """Contexts of different sizes side by side: the kernels' attributes belong to
 the process, so no context may depend on the limits another one needs.
 
-A problem with large tables (K_d = 32, q = 64: more than 48 KB of dynamic
+A problem with large tables (K_d = 32, q = 96: more than 48 KB of dynamic
 shared memory in its window, trace and energy kernels) and one with small ones
 are set up, assembled and stepped alternately and from two threads.
 """
